@@ -28,6 +28,7 @@ using namespace hqs;
 #define HQS_BATCH_MAX 64
 #define HQS_BATCH_BD 256
 #define HQS_BATCH_MAXR 24
+static_assert(HQS_BATCH_BD == 16 * hqs::kLines, "the Toeplitz items' CTA");
 
 namespace {
 
@@ -229,6 +230,55 @@ HQS_DEV void blur_tile(const BatchSlice& S, int tile, const float* g, int r, flo
     __syncthreads();
 }
 
+// The Toeplitz and preconditioner items as functions of their own (one body per slice
+// size): the persistent kernels call them from several places, and inlined into the
+// kernels' loops their transforms spilled (2.4 to 4.8 KB of stack a thread) and each
+// copy was compiled anew.  They name the dynamic shared memory themselves, so that its
+// accesses stay shared-memory instructions; the 2n-point twiddles are staged there by
+// the caller (STAGE_TW2).
+constexpr size_t kBatchTwOff = (size_t)768 * kLines + 384;
+
+__device__ __noinline__ void item_rows_fwd(const BatchSlice& S, int it, const float2* src) {
+    extern __shared__ __align__(16) float2 s[];
+    const int n = S.A.n, ch = it / n, iy = it - ch * n;
+    HQS_BATCH_DISPATCH(n, (toep_rows_fwd_item<N2>(S.A, iy, ch, src, nullptr, 0.f, false, s, nullptr, s + kBatchTwOff)));
+}
+__device__ __noinline__ void item_cols(const BatchSlice& S, int it) {
+    extern __shared__ __align__(16) float2 s[];
+    const int n = S.A.n, N2v = 2 * n;
+    if (S.colcap > 0) {
+        const int f0 = it * S.colcap, nl = min(S.colcap, N2v * S.A.L - f0);
+        HQS_BATCH_DISPATCH(n, (toep_cols_flat_item<N2>(S.A, f0, nl, s, s + kBatchTwOff)));
+    } else {
+        const int ch = it / N2v, kx = it - ch * N2v;
+        HQS_BATCH_DISPATCH(n, (toep_cols_item<N2>(S.A, kx, ch, s, s + kBatchTwOff)));
+    }
+}
+__device__ __noinline__ double item_rows_adj(const BatchSlice& S, int it, float2* out, const float2* pvec, float a,
+                                             float b, int mode) {
+    extern __shared__ __align__(16) float2 s[];
+    const int n = S.A.n, ch = it / n, iy = it - ch * n;
+    double v = 0.0;
+    HQS_BATCH_DISPATCH(n, (v = toep_rows_adj_item<N2>(S.A, iy, ch, out, pvec, a, b, mode, s, s + kBatchTwOff)));
+    return v;
+}
+__device__ __noinline__ void item_zp(const BatchSlice& S, int it, float beta, bool first) {
+    extern __shared__ __align__(16) float2 s[];
+    HQS_BATCH_DISPATCH(S.A.n, (z_and_p_rows<N2, N>(S, it * batch_zq<N>(), beta, first, s, S.twN)));
+}
+__device__ __noinline__ double item_pc_rows(const BatchSlice& S, int it, float alpha, bool update) {
+    extern __shared__ __align__(16) float2 s[];
+    double v = 0.0;
+    HQS_BATCH_DISPATCH(S.A.n, (v = pc_rows<N>(S, it * batch_pq<N>(), alpha, update, s, S.twN)));
+    return v;
+}
+__device__ __noinline__ double item_pc_cols(const BatchSlice& S, int it, float a, float b) {
+    extern __shared__ __align__(16) float2 s[];
+    double v = 0.0;
+    HQS_BATCH_DISPATCH(S.A.n, (v = pc_cols<N>(S, it * batch_pq<N>(), a, b, s, S.twN)));
+    return v;
+}
+
 // smem: lines buffer [768][16] | row [384] | tw 2n [768]; the n-point twiddles
 // of the preconditioner FFTs are read from global memory (L1), which keeps two
 // CTAs resident per SM.
@@ -246,11 +296,10 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
     __shared__ double rzs[HQS_BATCH_MAX], alphas[HQS_BATCH_MAX], betas[HQS_BATCH_MAX];
     __shared__ int sl_cache, tw_cur;
     const int ns = B.ns, G = gridDim.x, bid = blockIdx.x;
-    const float2* twN = nullptr;   // n-point twiddles of the current slice (global)
     // the 2n-point twiddles of the Toeplitz items stay in the shared region after the
     // largest lines buffer and its image row (the blur and preconditioner items use
     // less than the lines buffer), restaged only when the slice size changes
-    float2* twT = s + (size_t)768 * kLines + 384;
+    float2* twT = s + kBatchTwOff;
     if (threadIdx.x == 0) tw_cur = 0;
 #define STAGE_TW2(AA)                                                                    \
     if (tw_cur != 2 * (AA).n) {                                                          \
@@ -281,7 +330,6 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
             __VA_ARGS__;                                                                   \
         }                                                                                  \
     }
-#define STAGE_TWN(S, si) twN = (S).twN;
 #define CLEAR_ACC()                                                      \
     for (int i_ = threadIdx.x; i_ < 2 * HQS_BATCH_MAX; i_ += blockDim.x) \
         (&acc[0][0])[i_] = 0.0;                                          \
@@ -307,28 +355,18 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
         BB_BARRIER();
         // q = H u
         FOR_ITEMS(BL_ROWS, {
-            const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
             STAGE_TW2(S.A);
-            HQS_BATCH_DISPATCH(n, (toep_rows_fwd_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.u, nullptr, 0.f, false, s,
-                                                                        nullptr, twT)));
+            item_rows_fwd(S, it_, S.u);
         });
         BB_BARRIER();
         FOR_ITEMS(BL_COLS, {
-            const int n = S.A.n, N2v = 2 * n, ch = it_ / N2v, kx = it_ - ch * N2v;
             STAGE_TW2(S.A);
-            if (S.colcap > 0) {
-                const int f0 = it_ * S.colcap, nl = min(S.colcap, N2v * S.A.L - f0);
-                HQS_BATCH_DISPATCH(n, (toep_cols_flat_item<N2, HQS_BATCH_BD>(S.A, f0, nl, s, twT)));
-            } else {
-                HQS_BATCH_DISPATCH(n, (toep_cols_item<N2, HQS_BATCH_BD>(S.A, kx, ch, s, twT)));
-            }
+            item_cols(S, it_);
         });
         BB_BARRIER();
         FOR_ITEMS(BL_ROWS, {
-            const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
             STAGE_TW2(S.A);
-            HQS_BATCH_DISPATCH(n, (toep_rows_adj_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.q, S.u, acoef, bcoef, mode0, s,
-                                                                        twT)));
+            item_rows_adj(S, it_, S.q, S.u, acoef, bcoef, mode0);
         });
         EPI_BARRIER();
         FOR_ITEMS(BL_EPI, {   // several coil chunks: fixed-order chunk sum + epilogue
@@ -380,15 +418,12 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
         slice_totals(B.part + (size_t)BS_BB * ns * G, ns, tot[1]);
         // preconditioner of the initial residual
         FOR_ITEMS(BL_PC, {
-            STAGE_TWN(S, si);
-            HQS_BATCH_DISPATCH(S.A.n, (pc_rows<N>(S, it_ * batch_pq<N>(), 0.f, false, s, twN)));
+            item_pc_rows(S, it_, 0.f, false);
         });
         BB_BARRIER();
         CLEAR_ACC();
         FOR_ITEMS(BL_PC, {
-            STAGE_TWN(S, si);
-            double v = 0.0;
-            HQS_BATCH_DISPATCH(S.A.n, (v = pc_cols<N>(S, it_ * batch_pq<N>(), acoef, bcoef, s, twN)));
+            double v = item_pc_cols(S, it_, acoef, bcoef);
             v = cta_sum(v, red);
             if (threadIdx.x == 0) acc[0][si] += v;
         });
@@ -405,35 +440,23 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
         for (int cg = 0; cg < B.cg_iters; ++cg) {
             // A0: z rows and p = z + beta p
             FOR_ITEMS(BL_ZP, {
-                STAGE_TWN(S, si);
-                HQS_BATCH_DISPATCH(S.A.n, (z_and_p_rows<N2, N>(S, it_ * batch_zq<N>(), (float)betas[si], cg == 0, s, twN)));
+                item_zp(S, it_, (float)betas[si], cg == 0);
             });
             BB_BARRIER();
             FOR_ITEMS(BL_ROWS, {
-                const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
-                STAGE_TW2(S.A);
-                HQS_BATCH_DISPATCH(n, (toep_rows_fwd_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.p, nullptr, 0.f, false, s,
-                                                                            nullptr, twT)));
-            });
+            STAGE_TW2(S.A);
+            item_rows_fwd(S, it_, S.p);
+        });
             BB_BARRIER();
             FOR_ITEMS(BL_COLS, {
-                const int n = S.A.n, N2v = 2 * n, ch = it_ / N2v, kx = it_ - ch * N2v;
-                STAGE_TW2(S.A);
-                if (S.colcap > 0) {
-                    const int f0 = it_ * S.colcap, nl = min(S.colcap, N2v * S.A.L - f0);
-                    HQS_BATCH_DISPATCH(n, (toep_cols_flat_item<N2, HQS_BATCH_BD>(S.A, f0, nl, s, twT)));
-                } else {
-                    HQS_BATCH_DISPATCH(n, (toep_cols_item<N2, HQS_BATCH_BD>(S.A, kx, ch, s, twT)));
-                }
-            });
+            STAGE_TW2(S.A);
+            item_cols(S, it_);
+        });
             BB_BARRIER();
             CLEAR_ACC();
             FOR_ITEMS(BL_ROWS, {
-                const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
-                double v = 0.0;
                 STAGE_TW2(S.A);
-                HQS_BATCH_DISPATCH(n, (v = toep_rows_adj_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.q, S.p, acoef, bcoef, 1, s,
-                                                                                 twT)));
+            double v = item_rows_adj(S, it_, S.q, S.p, acoef, bcoef, 1);
                 v = cta_sum(v, red);
                 if (threadIdx.x == 0) acc[0][si] += v;
             });
@@ -462,9 +485,7 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
             // D: u, r update, ||r||^2, row FFTs of r
             CLEAR_ACC();
             FOR_ITEMS(BL_PC, {
-                STAGE_TWN(S, si);
-                double v = 0.0;
-                HQS_BATCH_DISPATCH(S.A.n, (v = pc_rows<N>(S, it_ * batch_pq<N>(), (float)alphas[si], true, s, twN)));
+                double v = item_pc_rows(S, it_, (float)alphas[si], true);
                 v = cta_sum(v, red);
                 if (threadIdx.x == 0) acc[1][si] += v;
             });
@@ -475,9 +496,7 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
             // E: preconditioner columns, <r, z>
             CLEAR_ACC();
             FOR_ITEMS(BL_PC, {
-                STAGE_TWN(S, si);
-                double v = 0.0;
-                HQS_BATCH_DISPATCH(S.A.n, (v = pc_cols<N>(S, it_ * batch_pq<N>(), acoef, bcoef, s, twN)));
+                double v = item_pc_cols(S, it_, acoef, bcoef);
                 v = cta_sum(v, red);
                 if (threadIdx.x == 0) acc[0][si] += v;
             });
@@ -519,7 +538,6 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
 #undef BB_BARRIER
 #undef EPI_BARRIER
 #undef FOR_ITEMS
-#undef STAGE_TWN
 #undef STAGE_TW2
 #undef CLEAR_ACC
 }
@@ -562,7 +580,7 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
     const float a = B.a, bcoef = B.b;
     // the 2n-point twiddles of the Toeplitz items stay in a fixed shared region after
     // the largest transform buffer and its image row, restaged only when the size changes
-    float2* twT = s + (size_t)768 * kLines + 384;
+    float2* twT = s + kBatchTwOff;
     if (threadIdx.x == 0) tw_cur = 0;
 #define STAGE_TW2(AA)                                                                    \
     if (tw_cur != 2 * (AA).n) {                                                          \
@@ -572,7 +590,6 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
         if (threadIdx.x == 0) tw_cur = 2 * (AA).n;                                       \
         __syncthreads();                                                                 \
     }
-    const float2* twN = nullptr;
     // optional phase trace, kept by thread 0 of CTA 0 (count in shared memory: no registers)
     __shared__ int ntr;
     if (B.trace && bid == 0 && threadIdx.x == 0) {
@@ -613,7 +630,6 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
             __VA_ARGS__;                                                                   \
         }                                                                                  \
     }
-#define STAGE_TWN(S, si) twN = (S).twN;
 #define CLEAR_ACC()                                                      \
     for (int i_ = threadIdx.x; i_ < 2 * HQS_BATCH_MAX; i_ += blockDim.x) \
         (&acc[0][0])[i_] = 0.0;                                          \
@@ -669,15 +685,12 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
     __syncthreads();
     // preconditioner of the initial residual, <r, z>
     FOR_ITEMS(BL_PC, {
-        STAGE_TWN(S, si);
-        HQS_BATCH_DISPATCH(S.A.n, (pc_rows<N>(S, it_ * batch_pq<N>(), 0.f, false, s, twN)));
+        item_pc_rows(S, it_, 0.f, false);
     });
     BB_BARRIER();
     CLEAR_ACC();
     FOR_ITEMS(BL_PC, {
-        STAGE_TWN(S, si);
-        double v = 0.0;
-        HQS_BATCH_DISPATCH(S.A.n, (v = pc_cols<N>(S, it_ * batch_pq<N>(), a, bcoef, s, twN)));
+        double v = item_pc_cols(S, it_, a, bcoef);
         v = cta_sum(v, red);
         if (threadIdx.x == 0) acc[0][si] += v;
     });
@@ -698,35 +711,24 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
     for (int cg = 0; cg < B.max_iter && nact > 0; ++cg) {
         // p = z + beta p
         FOR_ITEMS(BL_ZP, {
-            STAGE_TWN(S, si);
-            HQS_BATCH_DISPATCH(S.A.n, (z_and_p_rows<N2, N>(S, it_ * batch_zq<N>(), (float)betas[si], cg == 0, s, twN)));
+            item_zp(S, it_, (float)betas[si], cg == 0);
         });
         BB_BARRIER();
         // q = a A^H A p + b p, <p, q>
         FOR_ITEMS(BL_ROWS, {
-            const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
             STAGE_TW2(S.A);
-            HQS_BATCH_DISPATCH(n, (toep_rows_fwd_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.p, nullptr, 0.f, false, s,
-                                                                        nullptr, twT)));
+            item_rows_fwd(S, it_, S.p);
         });
         BB_BARRIER();
         FOR_ITEMS(BL_COLS, {
-            const int n = S.A.n, N2v = 2 * n, ch = it_ / N2v, kx = it_ - ch * N2v;
             STAGE_TW2(S.A);
-            if (S.colcap > 0) {
-                const int f0 = it_ * S.colcap, nl = min(S.colcap, N2v * S.A.L - f0);
-                HQS_BATCH_DISPATCH(n, (toep_cols_flat_item<N2, HQS_BATCH_BD>(S.A, f0, nl, s, twT)));
-            } else {
-                HQS_BATCH_DISPATCH(n, (toep_cols_item<N2, HQS_BATCH_BD>(S.A, kx, ch, s, twT)));
-            }
+            item_cols(S, it_);
         });
         BB_BARRIER();
         CLEAR_ACC();
         FOR_ITEMS(BL_ROWS, {
-            const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
-            double v = 0.0;
             STAGE_TW2(S.A);
-            HQS_BATCH_DISPATCH(n, (v = toep_rows_adj_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.q, S.p, a, bcoef, 1, s, twT)));
+            double v = item_rows_adj(S, it_, S.q, S.p, a, bcoef, 1);
             v = cta_sum(v, red);
             if (threadIdx.x == 0) acc[0][si] += v;
         });
@@ -759,9 +761,7 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
         // x += alpha p, r -= alpha q, ||r||^2, row FFTs of r
         CLEAR_ACC();
         FOR_ITEMS(BL_PC, {
-            STAGE_TWN(S, si);
-            double v = 0.0;
-            HQS_BATCH_DISPATCH(S.A.n, (v = pc_rows<N>(S, it_ * batch_pq<N>(), (float)alphas[si], true, s, twN)));
+            double v = item_pc_rows(S, it_, (float)alphas[si], true);
             v = cta_sum(v, red);
             if (threadIdx.x == 0) acc[1][si] += v;
         });
@@ -790,9 +790,7 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
         // preconditioner columns, <r, z>, beta
         CLEAR_ACC();
         FOR_ITEMS(BL_PC, {
-            STAGE_TWN(S, si);
-            double v = 0.0;
-            HQS_BATCH_DISPATCH(S.A.n, (v = pc_cols<N>(S, it_ * batch_pq<N>(), a, bcoef, s, twN)));
+            double v = item_pc_cols(S, it_, a, bcoef);
             v = cta_sum(v, red);
             if (threadIdx.x == 0) acc[0][si] += v;
         });
@@ -826,7 +824,6 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_pcg_batch(DcBatchArgs B) {
 #undef BB_BARRIER
 #undef EPI_BARRIER
 #undef FOR_ITEMS
-#undef STAGE_TWN
 #undef CLEAR_ACC
 #undef STAGE_TW2
 #undef COUNT_ACTIVE
@@ -852,7 +849,7 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_aha_batch(AhaBatchArgs B) {
     extern __shared__ __align__(16) float2 s[];
     __shared__ int tw_cur;
     const int ns = B.ns, G = gridDim.x, bid = blockIdx.x;
-    float2* twT = s + (size_t)768 * kLines + 384;
+    float2* twT = s + kBatchTwOff;
     if (threadIdx.x == 0) tw_cur = 0;
     __syncthreads();
 #define STAGE_TW2(AA)                                                                    \
@@ -878,27 +875,18 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_aha_batch(AhaBatchArgs B) {
         }                                                                                  \
     }
     FOR_ITEMS(BL_ROWS, {
-        const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
-        STAGE_TW2(S.A);
-        HQS_BATCH_DISPATCH(n, (toep_rows_fwd_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.u, nullptr, 0.f, false, s, nullptr,
-                                                                    twT)));
-    });
+            STAGE_TW2(S.A);
+            item_rows_fwd(S, it_, S.u);
+        });
     AB_BARRIER();
     FOR_ITEMS(BL_COLS, {
-        const int n = S.A.n, N2v = 2 * n, ch = it_ / N2v, kx = it_ - ch * N2v;
-        STAGE_TW2(S.A);
-        if (S.colcap > 0) {
-            const int f0 = it_ * S.colcap, nl = min(S.colcap, N2v * S.A.L - f0);
-            HQS_BATCH_DISPATCH(n, (toep_cols_flat_item<N2, HQS_BATCH_BD>(S.A, f0, nl, s, twT)));
-        } else {
-            HQS_BATCH_DISPATCH(n, (toep_cols_item<N2, HQS_BATCH_BD>(S.A, kx, ch, s, twT)));
-        }
-    });
+            STAGE_TW2(S.A);
+            item_cols(S, it_);
+        });
     AB_BARRIER();
     FOR_ITEMS(BL_ROWS, {
-        const int n = S.A.n, ch = it_ / n, iy = it_ - ch * n;
         STAGE_TW2(S.A);
-        HQS_BATCH_DISPATCH(n, (toep_rows_adj_item<N2, HQS_BATCH_BD>(S.A, iy, ch, S.q, nullptr, 1.f, 0.f, 0, s, twT)));
+            item_rows_adj(S, it_, S.q, nullptr, 1.f, 0.f, 0);
     });
     if (B.off[BL_EPI * (ns + 1) + ns] > 0) {   // several coil chunks: fixed-order chunk sum
         AB_BARRIER();
@@ -1046,10 +1034,9 @@ extern "C" int hqs_batch_create(hqs_batch* out, hqs_plan* plans, int n, int max_
         hqs_plan_s* p = plans[i];
         BatchSlice& S = hs[i];
         S.A = toep_args(p);
-        // coil chunk: as many lines as fill the CTA at this FFT size (16 lines of
-        // 640 points, 8 of 512 or 768), chunks of equal size
-        const int tpl = dispatch_fft_size(p->n2, [&]<int NN>() { return FftSize<NN>::TPL; });
-        const int lcmax = std::max(1, std::min(kLines, HQS_BATCH_BD / tpl));
+        // coil chunk: a work item holds kLines lines at every size (16 threads each),
+        // chunks of equal size
+        const int lcmax = kLines;
         const int nch = ceil_div(p->L, lcmax);
         S.A.nchunk = nch;
         S.A.LC = ceil_div(p->L, nch);

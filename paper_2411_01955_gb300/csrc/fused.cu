@@ -171,13 +171,36 @@ template <int N2, int N> constexpr size_t fused_smem_floats2() {
     return (size_t)N2 * kLines + N + N2 + N + N;   // lines | row | tw N2 | tw N | z row
 }
 
+// The items as functions of their own: inlined into the kernel's loops their transforms
+// spilled (860 bytes of stack a thread at 640 points).  They name the dynamic shared
+// memory themselves, so that its accesses stay shared-memory instructions.
 template <int N2, int N>
-__global__ void __launch_bounds__(FftSize<N2>::TPL * kLines,
-                                  (512 / (FftSize<N2>::TPL * kLines)) > 1 ? 512 / (FftSize<N2>::TPL * kLines) : 1)
-    k_pcg_persistent(FusedArgs F) {
+__device__ __noinline__ void item_z_rows_fwd(const FusedArgs& F, int iy, float beta) {
+    extern __shared__ __align__(16) float2 s[];
+    float2* twN = s + (size_t)N2 * kLines + N + N2;
+    float2* zs = twN + N;
+    z_row<N>(F, iy, s, twN, zs);
+    toep_rows_fwd_item<N2>(F.A, iy, 0, nullptr, F.p, beta, true, s, zs);
+}
+template <int N2> __device__ __noinline__ void item_rows_fwd(const FusedArgs& F, int w, const float2* src) {
+    extern __shared__ __align__(16) float2 s[];
+    toep_rows_fwd_item<N2>(F.A, w % F.A.n, w / F.A.n, src, nullptr, 0.f, false, s);
+}
+template <int N2> __device__ __noinline__ void item_cols(const FusedArgs& F, int w) {
+    extern __shared__ __align__(16) float2 s[];
+    toep_cols_item<N2>(F.A, w % N2, w / N2, s);
+}
+template <int N2> __device__ __noinline__ double item_rows_adj(const FusedArgs& F, int w, const float2* pvec) {
+    extern __shared__ __align__(16) float2 s[];
+    return toep_rows_adj_item<N2>(F.A, w % F.A.n, w / F.A.n, F.q, pvec, F.a, F.b, 1, s);
+}
+
+template <int N2, int N>
+__global__ void __launch_bounds__(toep_threads<N2>(), 512 / toep_threads<N2>())
+    k_pcg_persistent(const __grid_constant__ FusedArgs F) {
     extern __shared__ __align__(16) float2 s[];
     __shared__ double red[33];
-    constexpr int BD = FftSize<N2>::TPL * kLines;   // == blockDim.x
+    constexpr int BD = toep_threads<N2>();   // == blockDim.x
     const ToepArgs& A = F.A;
     const int n = A.n, nch = A.nchunk;
     const int G = gridDim.x, bid = blockIdx.x;
@@ -202,11 +225,11 @@ __global__ void __launch_bounds__(FftSize<N2>::TPL * kLines,
 
     // ---- r = rhs - H x  (x = 0: r = rhs without an A^H A apply)
     if (!F.x0_zero) {
-        for (int it = bid; it < n * nch; it += G) toep_rows_fwd_item<N2>(A, it % n, it / n, F.x, nullptr, 0.f, false, s);
+        for (int it = bid; it < n * nch; it += G) item_rows_fwd<N2>(F, it, F.x);
         BARRIER();
-        for (int it = bid; it < N2 * nch; it += G) toep_cols_item<N2>(A, it % N2, it / N2, s);
+        for (int it = bid; it < N2 * nch; it += G) item_cols<N2>(F, it);
         BARRIER();
-        for (int it = bid; it < n * nch; it += G) toep_rows_adj_item<N2>(A, it % n, it / n, F.q, F.x, F.a, F.b, 1, s);
+        for (int it = bid; it < n * nch; it += G) item_rows_adj<N2>(F, it, F.x);
         if (nch > 1) {
             BARRIER();
             double dummy = 0.0;
@@ -269,10 +292,7 @@ __global__ void __launch_bounds__(FftSize<N2>::TPL * kLines,
         // A: p = z + beta p, S_l p, FFT rows
         const float fb = (float)beta;
         if (nch == 1) {
-            for (int iy = bid; iy < n; iy += G) {
-                z_row<N>(F, iy, s, twN, zs);
-                toep_rows_fwd_item<N2>(A, iy, 0, nullptr, F.p, fb, true, s, zs);
-            }
+            for (int iy = bid; iy < n; iy += G) item_z_rows_fwd<N2, N>(F, iy, fb);
         } else {
             for (int iy = bid; iy < n; iy += G) {
                 z_row<N>(F, iy, s, twN, zs);
@@ -289,15 +309,15 @@ __global__ void __launch_bounds__(FftSize<N2>::TPL * kLines,
                 __syncthreads();
             }
             BARRIER();
-            for (int w = bid; w < n * nch; w += G) toep_rows_fwd_item<N2>(A, w % n, w / n, F.p, nullptr, 0.f, false, s);
+            for (int w = bid; w < n * nch; w += G) item_rows_fwd<N2>(F, w, F.p);
         }
         BARRIER();
         // B: columns
-        for (int w = bid; w < N2 * nch; w += G) toep_cols_item<N2>(A, w % N2, w / N2, s);
+        for (int w = bid; w < N2 * nch; w += G) item_cols<N2>(F, w);
         BARRIER();
         // C: q = a A^H A p + b p, <p, q>
         double pq = 0.0;
-        for (int w = bid; w < n * nch; w += G) pq += toep_rows_adj_item<N2>(A, w % n, w / n, F.q, F.p, F.a, F.b, 1, s);
+        for (int w = bid; w < n * nch; w += G) pq += item_rows_adj<N2>(F, w, F.p);
         if (nch > 1) {
             BARRIER();
             pq = 0.0;
@@ -383,7 +403,8 @@ static int pcg_fused_impl(hqs_plan_s* p, float a, float b, const float2* rhs, fl
     F.pcb = p->pc_buf;
     F.lam = p->lam;
     F.twN = plan_twiddles(p, N);
-    F.Q = std::max(1, std::min(p->pc_lines, kLines));
+    // as many n-point lines as the CTA's threads hold at once (8 at 256 points)
+    F.Q = std::max(1, std::min({p->pc_lines, kLines, toep_threads<N2>() / FftSize<N>::TPL}));
     F.precond = precond == HQS_PRECOND_DC ? 1 : 0;
     F.x0_zero = x0_zero ? 1 : 0;
     F.max_iter = max_iter;
@@ -396,7 +417,7 @@ static int pcg_fused_impl(hqs_plan_s* p, float a, float b, const float2* rhs, fl
     F.trace = p->trace;
     F.trace_max = p->trace ? HQS_TRACE_MAX : 0;
     auto kern = k_pcg_persistent<N2, N>;
-    const int threads = FftSize<N2>::TPL * kLines;
+    const int threads = toep_threads<N2>();
     const size_t sm = fused_smem_floats2<N2, N>() * sizeof(float2);
     HQS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     int per_sm = 0, nsm = 0, dev = 0;

@@ -44,6 +44,12 @@ const float2* plan_twiddles(const hqs_plan_s* p, int N) {
     return nullptr;
 }
 
+// the second table of each size in the bank (see plan_build)
+const float2* plan_twiddles16(const hqs_plan_s* p, int N) {
+    const float2* t = plan_twiddles(p, N);
+    return t ? t + N : nullptr;
+}
+
 // ------------------------------------------------------------- kernels
 
 // (L, n, n) -> (n, n, L)
@@ -339,7 +345,9 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
     HQS_CUDA_TRY(cudaMemsetAsync(p->dev_err, 0, 4 * sizeof(unsigned), s));
     HQS_CUDA_TRY(cudaMemsetAsync(p->barrier, 0, 64 * sizeof(unsigned), s));
 
-    // twiddle bank for the distinct FFT sizes (forward roots, fp64 -> fp32)
+    // twiddle bank for the distinct FFT sizes (forward roots, fp64 -> fp32): the N roots in
+    // order, then the same roots in the order of the two-stage transforms (fft16.cuh),
+    // w_N^(i kk) at i * 16 + kk
     {
         int sizes[3] = {G, n2, n};
         int ns = 0, total = 0;
@@ -349,7 +357,7 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
             if (!seen) {
                 p->tw_sizes[ns] = sizes[i];
                 p->tw_offs[ns] = total;
-                total += sizes[i];
+                total += 2 * sizes[i];
                 ++ns;
             }
         }
@@ -359,6 +367,9 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
                 const double a = -2.0 * M_PI * (double)m / (double)p->tw_sizes[k];
                 h[p->tw_offs[k] + m] = make_float2((float)cos(a), (float)sin(a));
             }
+        for (int k = 0; k < ns; ++k)
+            for (int m = 0; m < p->tw_sizes[k]; ++m)
+                h[p->tw_offs[k] + p->tw_sizes[k] + m] = h[p->tw_offs[k] + (m / 16) * (m % 16)];
         HQS_TRY(dev_alloc(p, &p->tw, (size_t)total));
         HQS_CUDA_TRY(cudaMemcpyAsync(p->tw, h.data(), total * sizeof(float2), cudaMemcpyHostToDevice, s));
         HQS_CUDA_TRY(cudaStreamSynchronize(s));

@@ -110,6 +110,8 @@ struct hqs_plan_s {
 };
 
 const float2* plan_twiddles(const hqs_plan_s* p, int N);
+// [N / 16][16]: w_N^(i kk) at i * 16 + kk (N a multiple of 16 in the plan's twiddle bank)
+const float2* plan_twiddles16(const hqs_plan_s* p, int N);
 // hqs_plan_create; with nufft_only the plan serves hqs_forward / hqs_adjoint only:
 // its Toeplitz kernel and density symbol are left zero (for internal helpers such as
 // the S-map estimation, which grids one coil at a time)

@@ -21,33 +21,33 @@ using namespace hqs;
 #include "toep_items.cuh"
 
 // --------------------------------------------------------- plain kernels
-template <int N2>
-__global__ void k_toep_rows_fwd(ToepArgs A, const float2* __restrict__ src, float2* __restrict__ pvec,
+template <int N2, int LINES>
+__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>()) k_toep_rows_fwd(ToepArgs A, const float2* __restrict__ src, float2* __restrict__ pvec,
                                 int fuse, const CgScalars* __restrict__ cg) {
     HQS_PDL_ENTRY();
     if (cg && cg->done) return;
     extern __shared__ __align__(16) float2 s[];
     const float beta = (fuse && cg) ? (float)cg->beta : 0.f;
-    toep_rows_fwd_item<N2>(A, blockIdx.x, blockIdx.y, src, pvec, beta, fuse != 0, s);
+    toep_rows_fwd_item<N2, LINES>(A, blockIdx.x, blockIdx.y, src, pvec, beta, fuse != 0, s);
 }
 
-template <int N2>
-__global__ void k_toep_cols(ToepArgs A, const CgScalars* __restrict__ cg) {
+template <int N2, int LINES>
+__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>()) k_toep_cols(ToepArgs A, const CgScalars* __restrict__ cg) {
     HQS_PDL_ENTRY();
     if (cg && cg->done) return;
     extern __shared__ __align__(16) float2 s[];
-    toep_cols_item<N2>(A, blockIdx.x, blockIdx.y, s);
+    toep_cols_item<N2, LINES>(A, blockIdx.x, blockIdx.y, s);
 }
 
-template <int N2>
-__global__ void k_toep_rows_adj(ToepArgs A, float2* __restrict__ out, const float2* __restrict__ pvec,
+template <int N2, int LINES>
+__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>()) k_toep_rows_adj(ToepArgs A, float2* __restrict__ out, const float2* __restrict__ pvec,
                                 float a, float b, int mode, double* __restrict__ part,
                                 const CgScalars* __restrict__ cg) {
     HQS_PDL_ENTRY();
     if (cg && cg->done) return;
     extern __shared__ __align__(16) float2 s[];
     __shared__ double red[32];
-    const double v = toep_rows_adj_item<N2>(A, blockIdx.x, blockIdx.y, out, pvec, a, b, mode, s);
+    const double v = toep_rows_adj_item<N2, LINES>(A, blockIdx.x, blockIdx.y, out, pvec, a, b, mode, s);
     if (part && A.nchunk == 1) {
         const double t = block_sum(v, red);
         if (threadIdx.x == 0) part[blockIdx.x] = t;
@@ -248,7 +248,7 @@ ToepArgs toep_args(hqs_plan_s* p) {
     A.nchunk = p->nchunk;
     A.smaps = p->smaps;
     A.khat = p->khat;
-    A.tw = plan_twiddles(p, p->n2);
+    A.tw = p->n2 >= 128 ? plan_twiddles16(p, p->n2) : plan_twiddles(p, p->n2);
     A.T = p->work;
     A.chunk = p->chunk_buf;
     return A;
@@ -259,25 +259,25 @@ int toep_partial_count(const hqs_plan_s* p) {
     return p->nchunk == 1 ? p->n : std::min(ceil_div(p->n * p->n, 256), 1024);
 }
 
-template <int N2>
+template <int N2, int LINES>
 static int toep_impl(hqs_plan_s* p, const float2* src, float2* pvec, int fuse, float2* out,
                      const float2* pmul, float a, float b, int mode, double* part,
                      const CgScalars* cg, cudaStream_t st) {
     ToepArgs A = toep_args(p);
-    const int th = fft_threads<N2>(p->LC);
-    const size_t sm = toep_smem_floats2<N2>(p->n) * sizeof(float2);
-    HQS_CUDA_TRY(cudaFuncSetAttribute(k_toep_rows_fwd<N2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    HQS_CUDA_TRY(cudaFuncSetAttribute(k_toep_cols<N2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    HQS_CUDA_TRY(cudaFuncSetAttribute(k_toep_rows_adj<N2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    const int th = fft16_ok<N2>() ? toep_threads<N2, LINES>() : fft_threads<N2>(p->LC);
+    const size_t sm = toep_smem_floats2<N2, LINES>(p->n) * sizeof(float2);
+    HQS_CUDA_TRY(cudaFuncSetAttribute((k_toep_rows_fwd<N2, LINES>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HQS_CUDA_TRY(cudaFuncSetAttribute((k_toep_cols<N2, LINES>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    HQS_CUDA_TRY(cudaFuncSetAttribute((k_toep_rows_adj<N2, LINES>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const dim3 grows(p->n, p->nchunk), gcols(N2, p->nchunk);
     if (fuse && p->nchunk > 1) {
         k_cg_pupdate<<<std::min(ceil_div(p->n * p->n, 256), 1024), 256, 0, st>>>(src, pvec, p->n * p->n, cg);
         src = pvec;
         fuse = 0;
     }
-    HQS_CUDA_TRY(launch_pdl(k_toep_rows_fwd<N2>, grows, th, sm, st, A, src, pvec, fuse, cg));
-    HQS_CUDA_TRY(launch_pdl(k_toep_cols<N2>, gcols, th, sm, st, A, cg));
-    HQS_CUDA_TRY(launch_pdl(k_toep_rows_adj<N2>, grows, th, sm, st, A, out, pmul, a, b, mode, part, cg));
+    HQS_CUDA_TRY(launch_pdl((k_toep_rows_fwd<N2, LINES>), grows, th, sm, st, A, src, pvec, fuse, cg));
+    HQS_CUDA_TRY(launch_pdl((k_toep_cols<N2, LINES>), gcols, th, sm, st, A, cg));
+    HQS_CUDA_TRY(launch_pdl((k_toep_rows_adj<N2, LINES>), grows, th, sm, st, A, out, pmul, a, b, mode, part, cg));
     if (p->nchunk > 1)
         HQS_CUDA_TRY(launch_pdl(k_toep_chunk_epilogue, dim3(toep_partial_count(p)), dim3(256), 0, st, A, out, pmul, a,
                                 b, mode, part, cg));
@@ -288,8 +288,15 @@ static int toep_impl(hqs_plan_s* p, const float2* src, float2* pvec, int fuse, f
 int launch_toeplitz_ex(hqs_plan_s* p, const float2* src, float2* pvec, int fuse, float2* out,
                        const float2* pmul, float a, float b, int mode, double* part,
                        const CgScalars* cg, cudaStream_t st) {
-    return dispatch_fft_size(p->n2, [&]<int NN>() {
-        return toep_impl<NN>(p, src, pvec, fuse, out, pmul, a, b, mode, part, cg, st);
+    return dispatch_fft_size(p->n2, [&]<int NN>() -> int {
+        if constexpr (fft16_ok<NN>()) {
+            // lines per CTA: the smallest of 4, 8, 16 that holds the plan's coil chunk
+            if (p->LC <= 4) return toep_impl<NN, 4>(p, src, pvec, fuse, out, pmul, a, b, mode, part, cg, st);
+            if (p->LC <= 8) return toep_impl<NN, 8>(p, src, pvec, fuse, out, pmul, a, b, mode, part, cg, st);
+        }
+        if constexpr (fft16_ok<NN>() || NN == 32 || NN == 64)
+            return toep_impl<NN, kLines>(p, src, pvec, fuse, out, pmul, a, b, mode, part, cg, st);
+        return HQS_ERR_INVALID_ARG;
     });
 }
 
