@@ -9,8 +9,39 @@
 #define HQS_DEV __device__ __forceinline__
 
 // ---------------------------------------------------------------- complex
-HQS_DEV float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-HQS_DEV float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Complex add and subtract as one packed FP32x2 instruction each (sm_100 and later; every
+// component rounded to nearest as by the scalar instruction).  The transform passes are
+// bound by instruction issue: A^H A at 320^2 x 16 coils 51.1 -> 49.8 us, the one-slice
+// solve step 788 -> 750 us, the volume solve 1883 -> 1762 us.
+HQS_DEV float2 cadd(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 p, q, s;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\t"
+        "add.rn.f32x2 s, p, q;\n\tmov.b64 {%0, %1}, s;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+HQS_DEV float2 csub(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 p, q, s;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\t"
+        "sub.rn.f32x2 s, p, q;\n\tmov.b64 {%0, %1}, s;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+// acc + a s and a s for a real factor, packed the same way
+HQS_DEV float2 cfma_r(float2 a, float s, float2 acc) {
+    float2 r;
+    asm("{\n\t.reg .b64 p, q, t, u;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %4};\n\tmov.b64 t, {%5, %6};\n\t"
+        "fma.rn.f32x2 u, p, q, t;\n\tmov.b64 {%0, %1}, u;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(s), "f"(acc.x), "f"(acc.y));
+    return r;
+}
+HQS_DEV float2 cmul_r(float2 a, float s) {
+    float2 r;
+    asm("{\n\t.reg .b64 p, q, u;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %4};\n\t"
+        "mul.rn.f32x2 u, p, q;\n\tmov.b64 {%0, %1}, u;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(s));
+    return r;
+}
 HQS_DEV float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 HQS_DEV float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);

@@ -44,8 +44,8 @@ template <bool INV> struct Dft<3, INV> {
         const float h = 0.86602540378443864676f;
         float2 t = cadd(v[1], v[2]);
         float2 d = csub(v[1], v[2]);
-        float2 m = make_float2(v[0].x - 0.5f * t.x, v[0].y - 0.5f * t.y);
-        float2 j = mul_mi<INV>(cscale(d, h));      // -+ i * sqrt(3)/2 * d
+        float2 m = cfma_r(t, -0.5f, v[0]);
+        float2 j = mul_mi<INV>(cmul_r(d, h));      // -+ i * sqrt(3)/2 * d
         v[0] = cadd(v[0], t);
         v[1] = cadd(m, j);
         v[2] = csub(m, j);
@@ -72,12 +72,12 @@ template <bool INV> struct Dft<5, INV> {
         float2 a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
         float2 a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
         float2 x0 = v[0];
-        float2 m1 = make_float2(x0.x + c1 * a1.x + c2 * a2.x, x0.y + c1 * a1.y + c2 * a2.y);
-        float2 m2 = make_float2(x0.x + c2 * a1.x + c1 * a2.x, x0.y + c2 * a1.y + c1 * a2.y);
+        float2 m1 = cfma_r(a2, c2, cfma_r(a1, c1, x0));
+        float2 m2 = cfma_r(a2, c1, cfma_r(a1, c2, x0));
         // forward: out1 = m1 - i(s1 b1 + s2 b2); out2 = m2 - i(s2 b1 - s1 b2)
-        float2 n1 = mul_mi<INV>(make_float2(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y));
-        float2 n2 = mul_mi<INV>(make_float2(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y));
-        v[0] = make_float2(x0.x + a1.x + a2.x, x0.y + a1.y + a2.y);
+        float2 n1 = mul_mi<INV>(cfma_r(b2, s2, cmul_r(b1, s1)));
+        float2 n2 = mul_mi<INV>(cfma_r(b2, -s1, cmul_r(b1, s2)));
+        v[0] = cadd(cadd(x0, a1), a2);
         v[1] = cadd(m1, n1);
         v[4] = csub(m1, n1);
         v[2] = cadd(m2, n2);
