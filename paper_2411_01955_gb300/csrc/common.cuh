@@ -42,6 +42,14 @@ HQS_DEV float2 cmul_r(float2 a, float s) {
         : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(s));
     return r;
 }
+// acc + a b component by component (a real factor kept as a pair)
+HQS_DEV float2 cfma2(float2 a, float2 b, float2 acc) {
+    float2 r;
+    asm("{\n\t.reg .b64 p, q, t, u;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tmov.b64 t, {%6, %7};\n\t"
+        "fma.rn.f32x2 u, p, q, t;\n\tmov.b64 {%0, %1}, u;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(acc.x), "f"(acc.y));
+    return r;
+}
 HQS_DEV float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 HQS_DEV float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -61,6 +69,13 @@ HQS_DEV void cp_async16(void* smem_dst, const void* gmem_src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
 }
+// 8-byte form (through L1; both addresses 8-byte aligned)
+HQS_DEV void cp_async8(void* smem_dst, const void* gmem_src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gmem_src) : "memory");
+}
+HQS_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> HQS_DEV void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 HQS_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Programmatic dependent launch (kernels launched with launch_pdl): the

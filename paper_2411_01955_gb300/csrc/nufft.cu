@@ -833,6 +833,14 @@ inline size_t spread_smem(int W, int lcs, int tile) {
            (size_t)HQS_SPREAD_CAND * (sizeof(int2) + sizeof(int)) + (size_t)HQS_SPREAD_CAND * tile * sizeof(float);
 }
 
+int launch_y_to_sorted(const float2* y, const int* inv, int64_t M, int L, float2* ysort, cudaStream_t st) {
+    if (M == 0) return HQS_OK;
+    const size_t smy = (size_t)kSortPts * (L + 1) * sizeof(float2);
+    HQS_CUDA_TRY(launch_pdl(k_y_to_sorted, dim3((unsigned)ceil_div64(M, kSortPts)), dim3(256), smy, st, y, inv, (int)M, L,
+                            ysort));
+    return HQS_OK;
+}
+
 template <int W, int TT>
 static int spread_tiles_impl(hqs_plan_s* p, const float2* y, cudaStream_t st) {
     const int lcs = spread_lcs(TT, p->L);
@@ -840,11 +848,7 @@ static int spread_tiles_impl(hqs_plan_s* p, const float2* y, cudaStream_t st) {
     const size_t sm = spread_smem(W, lcs, full16 ? TT : 0);
     auto kern = full16 ? k_spread_tiles<W, TT, true> : k_spread_tiles<W, TT, false>;
     HQS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    if (p->M > 0) {
-        const size_t smy = (size_t)kSortPts * (p->L + 1) * sizeof(float2);
-        HQS_CUDA_TRY(launch_pdl(k_y_to_sorted, dim3((unsigned)ceil_div64(p->M, kSortPts)), dim3(256), smy, st, y,
-                                p->invperm, (int)p->M, p->L, p->spread.ysort));
-    }
+    if (const int rc = launch_y_to_sorted(y, p->invperm, p->M, p->L, p->spread.ysort, st); rc != HQS_OK) return rc;
     HQS_CUDA_TRY(launch_pdl(kern, dim3(p->spread.nitems), dim3(256), sm, st, p->spread.ysort, p->pts, p->spread.kbw,
                             p->spread.tile_nb, p->spread.items, p->spread.tile_info, p->spread.tickets,
                             p->spread.partial, p->G, p->L, lcs, p->nbx, p->grid));

@@ -4,10 +4,10 @@
 //
 //   forward : apodise + coil-multiply fused into the x-axis FFT of the
 //             centred, sigma-oversampled grid, then the y and z FFTs, then
-//             W^3-tap Kaiser-Bessel interpolation (gather, one half-warp per
-//             point, lanes over coils);
-//   adjoint : shared-memory tiled spreading (TB^3 bins), z / y / x inverse
-//             FFTs with crop, conj(S_l) per coil, coil sum + deapodisation;
+//             W^3-tap Kaiser-Bessel interpolation (gather, units of up to 4
+//             points of one footprint, lanes over coils);
+//   adjoint : tile-owned spreading (8^3 tiles), z / y / x inverse FFTs with
+//             crop, conj(S_l) per coil, coil sum + deapodisation;
 //   A^H A   : the 2N^3 circulant embedding (Sec. 3.4 form of the normal
 //             operator): pad(S_l x) -> FFT_x, FFT_y, FFT_z * Khat * IFFT_z,
 //             IFFT_y, IFFT_x -> crop, conj(S_l) sum.  Zero-padded inputs use
@@ -35,6 +35,7 @@ using namespace hqs;
 #define HQS3_TILE 8           // spreading bin edge on the grid
 #define HQS3_MAXPTS 256       // points per spreading sub-problem
 #define HQS3_KERNEL_W 8       // KB width used to grid the Toeplitz kernel
+#define HQS3_UNIT 4           // points of one footprint interpolated together
 
 struct Cg3 {
     double rr, rz, pq, alpha, beta, bnorm2, tol2;
@@ -54,8 +55,18 @@ struct hqs_plan3d_s {
     float2* smaps = nullptr;  // [nz][ny][nx][L]
     float* apod[3] = {nullptr, nullptr, nullptr};
     int4* pti = nullptr;      // sorted points: (i0x, i0y, i0z, caller index)
-    float4* ptd = nullptr;    // (dx, dy, dz, 0)
-    int4* subs = nullptr;     // (bin, start, count, 0)
+    int* inv = nullptr;       // caller index -> sorted position
+    float* kbw = nullptr;     // [M][32] Kaiser-Bessel weights of the sorted points (k_weights3)
+    int2* units = nullptr;    // runs of <= HQS3_UNIT sorted points of one footprint: (first, count)
+    int nunits = 0;
+    int2* list = nullptr;     // the units touching each tile, tile by tile: (first point, offsets of the first
+                              // tap from the tile's origin + 16 in one byte per axis, count in the top byte)
+    int4* items = nullptr;    // spreading items: (tile, first entry, end entry, partial slot or -1)
+    int nitems = 0;
+    int2* tinfo = nullptr;    // [tiles] (items, first partial slot) of tiles with several items
+    unsigned* tickets = nullptr;   // [tiles][coil chunks] arrivals (reset by the last)
+    float2* partial = nullptr;     // [slots][coil chunks][512][4 CPL] partial tiles
+    float2* ysort = nullptr;       // [M][L] k-space data in sorted order, coil-innermost
     float* khat = nullptr;    // [2nz][2ny][2nx], includes 1 / (8 Nvox)
     float2* tw = nullptr;     // twiddle bank
     int tw_sizes[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -147,90 +158,447 @@ __global__ void k_smaps3_coil_inner(const float2* __restrict__ in, float2* __res
     }
 }
 
+// ------------------------------------------------------ point order
+// Points lie in the order (bin, cell of the bin): points of one footprint (the same
+// W^3 cells) are consecutive.  One CTA orders one bin: a histogram of its 512 cells,
+// its exclusive sum, and the scatter.
+constexpr int kCells3 = HQS3_TILE * HQS3_TILE * HQS3_TILE;
+HQS_DEV int local_cell3(int4 p, int W, int Gx, int Gy, int Gz) {
+    const int cx = wrap(p.x + W / 2, Gx), cy = wrap(p.y + W / 2, Gy), cz = wrap(p.z + W / 2, Gz);
+    return ((cz % HQS3_TILE) * HQS3_TILE + cy % HQS3_TILE) * HQS3_TILE + cx % HQS3_TILE;
+}
+// exclusive sums of c[0 .. kCells3) in place (blockDim.x == 256); returns the total
+HQS_DEV int exclusive_sums3(int* c, int* wsum) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int a = c[2 * threadIdx.x], b = c[2 * threadIdx.x + 1];
+    int v = a + b;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    if (lane == 31) wsum[warp] = v;
+    __syncthreads();
+    int base = 0, tot = 0;
+    for (int w = 0; w < 8; ++w) {
+        base += w < warp ? wsum[w] : 0;
+        tot += wsum[w];
+    }
+    c[2 * threadIdx.x] = base + v - a - b;
+    c[2 * threadIdx.x + 1] = base + v - b;
+    __syncthreads();
+    return tot;
+}
+__global__ void __launch_bounds__(256) k_bin_sort3(const int4* __restrict__ pin, const float4* __restrict__ din,
+                                                   const int* __restrict__ binoff, int W, int Gx, int Gy, int Gz,
+                                                   int4* __restrict__ pti, float4* __restrict__ ptd,
+                                                   int* __restrict__ inv, int* __restrict__ unit_counts) {
+    __shared__ int cur[kCells3], wsum[8];
+    __shared__ int nu;
+    const int b0 = binoff[blockIdx.x], b1 = binoff[blockIdx.x + 1];
+    for (int c = threadIdx.x; c < kCells3; c += blockDim.x) cur[c] = 0;
+    if (threadIdx.x == 0) nu = 0;
+    __syncthreads();
+    for (int j = b0 + threadIdx.x; j < b1; j += blockDim.x) atomicAdd(&cur[local_cell3(pin[j], W, Gx, Gy, Gz)], 1);
+    __syncthreads();
+    int u = 0;
+    for (int c = threadIdx.x; c < kCells3; c += blockDim.x) u += (cur[c] + HQS3_UNIT - 1) / HQS3_UNIT;
+    if (u > 0) atomicAdd(&nu, u);
+    __syncthreads();
+    if (threadIdx.x == 0) unit_counts[blockIdx.x] = nu;
+    exclusive_sums3(cur, wsum);
+    for (int j = b0 + threadIdx.x; j < b1; j += blockDim.x) {
+        const int4 p = pin[j];
+        const int pos = b0 + atomicAdd(&cur[local_cell3(p, W, Gx, Gy, Gz)], 1);
+        pti[pos] = p;
+        ptd[pos] = din[j];
+        inv[p.w] = pos;
+    }
+}
+__global__ void __launch_bounds__(256) k_units3(const int4* __restrict__ pti, const int* __restrict__ binoff,
+                                                const int* __restrict__ unit_off, int W, int Gx, int Gy, int Gz,
+                                                int2* __restrict__ units) {
+    __shared__ int cnt[kCells3], first[kCells3], uo[kCells3], wsum[8];
+    const int b0 = binoff[blockIdx.x], b1 = binoff[blockIdx.x + 1];
+    if (b0 == b1) return;
+    for (int c = threadIdx.x; c < kCells3; c += blockDim.x) cnt[c] = 0;
+    __syncthreads();
+    for (int j = b0 + threadIdx.x; j < b1; j += blockDim.x) atomicAdd(&cnt[local_cell3(pti[j], W, Gx, Gy, Gz)], 1);
+    __syncthreads();
+    for (int c = threadIdx.x; c < kCells3; c += blockDim.x) {
+        first[c] = cnt[c];
+        uo[c] = (cnt[c] + HQS3_UNIT - 1) / HQS3_UNIT;
+    }
+    __syncthreads();
+    exclusive_sums3(first, wsum);
+    exclusive_sums3(uo, wsum);
+    for (int c = threadIdx.x; c < kCells3; c += blockDim.x)
+        for (int k = 0; k * HQS3_UNIT < cnt[c]; ++k)
+            units[unit_off[blockIdx.x] + uo[c] + k] =
+                make_int2(b0 + first[c] + k * HQS3_UNIT, min(HQS3_UNIT, cnt[c] - k * HQS3_UNIT));
+}
+// Kaiser-Bessel weights of the sorted points, 32 floats (128 bytes) each: x taps [8],
+// z taps [8], y taps as pairs [8][2] (the operand of packed multiply-adds); zero beyond W.
+__global__ void k_weights3(const float4* __restrict__ ptd, int64_t M, int W, float beta, float* __restrict__ kbw) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= M * 24) return;
+    const int64_t j = e / 24;
+    const int h = (int)(e - j * 24), b = h & 7;
+    const float4 d = ptd[j];
+    const float t = (h < 8 ? d.x : (h < 16 ? d.z : d.y)) - (float)b;
+    const float w = b < W ? kb_phi3(t, (float)W, beta) : 0.f;
+    float* o = kbw + j * 32;
+    if (h < 16) o[h] = w;
+    else o[16 + 2 * b] = o[17 + 2 * b] = w;
+}
+
+// The tiles (up to two per axis) that a footprint touches: f(tile, offsets).
+template <class F> HQS_DEV void touched_tiles3(int4 p, int W, int Gx, int Gy, int Gz, F&& f) {
+    constexpr int T = HQS3_TILE;
+    const int i0[3] = {p.x, p.y, p.z}, G[3] = {Gx, Gy, Gz};
+    int t[3][2], o[3][2], n[3];
+    for (int a = 0; a < 3; ++a) {
+        t[a][0] = i0[a] / T;
+        o[a][0] = i0[a] - t[a][0] * T;
+        t[a][1] = wrap(i0[a] + W - 1, G[a]) / T;
+        const int d = i0[a] - t[a][1] * T;
+        o[a][1] = d > 0 ? d - G[a] : d;   // taps that wrap start before cell 0
+        n[a] = t[a][1] != t[a][0] ? 2 : 1;
+    }
+    for (int c = 0; c < n[2]; ++c)
+        for (int b = 0; b < n[1]; ++b)
+            for (int a = 0; a < n[0]; ++a)
+                f((t[2][c] * (Gy / T) + t[1][b]) * (Gx / T) + t[0][a],
+                  (o[0][a] + 16) | ((o[1][b] + 16) << 8) | ((o[2][c] + 16) << 16));
+}
+__global__ void k_tile_count3(const int4* __restrict__ pti, const int2* __restrict__ units, int nunits, int W, int Gx,
+                              int Gy, int Gz, int* __restrict__ counts) {
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < nunits) touched_tiles3(pti[units[u].x], W, Gx, Gy, Gz, [&](int t, int) { atomicAdd(&counts[t], 1); });
+}
+__global__ void k_tile_fill3(const int4* __restrict__ pti, const int2* __restrict__ units, int nunits, int W, int Gx,
+                             int Gy, int Gz, int* __restrict__ cursor, int2* __restrict__ list) {
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u >= nunits) return;
+    const int2 un = units[u];
+    touched_tiles3(pti[un.x], W, Gx, Gy, Gz,
+                   [&](int t, int off) { list[atomicAdd(&cursor[t], 1)] = make_int2(un.x, off | (un.y << 24)); });
+}
+
 // ------------------------------------------------------ interpolation
-// Type-2 interpolation: a half-warp per point, lane = coil (looping beyond
-// 16 coils).  The 3W separable weights are computed once per point by the
-// lanes (index q on lane q and q - 16) and broadcast with shuffles.
-template <int W>
-__global__ void __launch_bounds__(256) k_interp3(const float2* __restrict__ Gh, const int4* __restrict__ pti,
-                                                 const float4* __restrict__ ptd, int M, int Gx, int Gy,
-                                                 int Gz, int L, float beta, float2* __restrict__ y) {
-    const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;
-    const int h = threadIdx.x & 15;
-    const int base = threadIdx.x & 16;
-    const bool valid = j < M;
-    const int4 pi = valid ? pti[j] : make_int4(0, 0, 0, 0);
-    const float4 pd = valid ? ptd[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-    float w0 = 0.f, w1 = 0.f;
-    if (valid) {
-        const float dd[3] = {pd.x, pd.y, pd.z};
-        if (h < 3 * W) w0 = kb_phi3(dd[h / W] - (float)(h % W), (float)W, beta);
-        const int q = h + 16;
-        if (q < 3 * W) w1 = kb_phi3(dd[q / W] - (float)(q % W), (float)W, beta);
+// Type-2 interpolation, a group of LPP lanes per unit (up to 4 points of one
+// footprint), lane q owning VEC coils: every grid value is read once for the unit's
+// points, so the loads fall with the footprints' occupancy (a stack of 64 spirals of
+// 8 x 1024 on the 128^3 grid has 6 points per distinct footprint) and the FMAs of the 4
+// points hide their latency.  CTAs take consecutive units, which share an L1-sized
+// neighbourhood.  Bound: L1 wavefronts (one per 128 bytes read) and the FMA pipe.
+// 64^3 x 16 coils, 524,288 points, W 6: 1556 -> 365 us against a half-warp per point (a
+// whole forward 1723 -> 521 us).
+template <int VEC> struct Vec3;
+template <> struct Vec3<2> {
+    float2 a, b;
+    HQS_DEV static Vec3 load(const float2* p) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+        return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
     }
-    float wx[W], wy[W], wz[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        const int qx = w, qy = W + w, qz = 2 * W + w;
-        wx[w] = qx < 16 ? __shfl_sync(0xffffffffu, w0, base + qx) : __shfl_sync(0xffffffffu, w1, base + qx - 16);
-        wy[w] = qy < 16 ? __shfl_sync(0xffffffffu, w0, base + qy) : __shfl_sync(0xffffffffu, w1, base + qy - 16);
-        wz[w] = qz < 16 ? __shfl_sync(0xffffffffu, w0, base + qz) : __shfl_sync(0xffffffffu, w1, base + qz - 16);
+    HQS_DEV void zero() { a = b = make_float2(0.f, 0.f); }
+    HQS_DEV void fma(const Vec3& v, float2 w) {
+        a = cfma2(v.a, w, a);
+        b = cfma2(v.b, w, b);
     }
-    if (!valid) return;
-    int gx[W];
-#pragma unroll
-    for (int b = 0; b < W; ++b) gx[b] = wrap(pi.x + b, Gx);
-    for (int l = h; l < L; l += 16) {
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 1
-        for (int c = 0; c < W; ++c) {
-            const int gz = wrap(pi.z + c, Gz);
-            float2 az = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                const int gy = wrap(pi.y + a, Gy);
-                const float2* row = Gh + ((int64_t)gz * Gy + gy) * Gx * L + l;
-                float2 ra = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const float2 g = __ldg(row + (int64_t)gx[b] * L);
-                    ra.x = fmaf(wx[b], g.x, ra.x);
-                    ra.y = fmaf(wx[b], g.y, ra.y);
-                }
-                az.x = fmaf(wy[a], ra.x, az.x);
-                az.y = fmaf(wy[a], ra.y, az.y);
-            }
-            acc.x = fmaf(wz[c], az.x, acc.x);
-            acc.y = fmaf(wz[c], az.y, acc.y);
+    HQS_DEV void put(float2* y, int64_t M, int lim) const {
+        y[0] = a;
+        if (lim > 1) y[M] = b;
+    }
+};
+template <> struct Vec3<1> {
+    float2 a;
+    HQS_DEV static Vec3 load(const float2* p) { return {__ldg(p)}; }
+    HQS_DEV void zero() { a = make_float2(0.f, 0.f); }
+    HQS_DEV void fma(const Vec3& v, float2 w) { a = cfma2(v.a, w, a); }
+    HQS_DEV void put(float2* y, int64_t, int) const { y[0] = a; }
+};
+constexpr int kInterpRounds = 4;   // most units of a lane group, one after the other
+template <int W, int VEC, int LPP>
+__global__ void __launch_bounds__(256, 2) k_interp3(const float2* __restrict__ Gh, const int4* __restrict__ pti,
+                                                    const float* __restrict__ kbw, const int2* __restrict__ units,
+                                                    int nunits, int rounds, int64_t M, int Gx, int Gy,
+                                                    int Gz, int L, float2* __restrict__ y) {
+    constexpr int NG = 256 / LPP, U = HQS3_UNIT;
+    static_assert(U == 4, "one float4 of weights per tap");
+    __shared__ __align__(16) float swt[NG][17][U];   // y taps 0..7, z taps 8..15 by point (17: distinct banks)
+    const int g = threadIdx.x / LPP, q = threadIdx.x % LPP;
+    for (int r = 0; r < rounds; ++r) {
+        const int64_t u = ((int64_t)blockIdx.x * rounds + r) * NG + g;
+        const bool valid = u < nunits;   // the lanes of a warp stay together: idle groups repeat the last unit
+        const int2 un = units[valid ? u : nunits - 1];
+        const int4 p0 = pti[un.x];
+        // weights of the unit's points; points beyond its count repeat the last one
+        __syncwarp();
+        for (int e = q; e < 16 * U; e += LPP) {
+            const int k = e & 3, h = e >> 2;
+            const float* kw = kbw + (int64_t)(un.x + min(k, un.y - 1)) * 32;
+            swt[g][h][k] = __ldg(kw + (h < 8 ? 16 + 2 * h : h));
         }
-        y[(int64_t)l * M + pi.w] = acc;
+        float wx[U][W];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const float* kw = kbw + (int64_t)(un.x + min(k, un.y - 1)) * 32;
+#pragma unroll
+            for (int b = 0; b < W; b += 4) {
+                const float4 v = __ldg(reinterpret_cast<const float4*>(kw + b));
+                const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    if (b + h < W) wx[k][b + h] = vv[h];
+            }
+        }
+        __syncwarp();
+        int gx[W];
+#pragma unroll
+        for (int b = 0; b < W; ++b) gx[b] = wrap(p0.x + b, Gx) * L;
+        for (int l = q * VEC; l < L; l += LPP * VEC) {
+            Vec3<VEC> acc[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) acc[k].zero();
+#pragma unroll 1
+            for (int c = 0; c < W; ++c) {
+                const float4 wz = *reinterpret_cast<const float4*>(swt[g][8 + c]);
+                const float2* plane = Gh + (int64_t)wrap(p0.z + c, Gz) * Gy * Gx * L + l;
+#pragma unroll
+                for (int a = 0; a < W; ++a) {
+                    const float2* row = plane + (int64_t)wrap(p0.y + a, Gy) * Gx * L;
+                    Vec3<VEC> t[W], ra[U];
+#pragma unroll
+                    for (int b = 0; b < W; ++b) t[b] = Vec3<VEC>::load(row + gx[b]);
+                    const float4 wy = *reinterpret_cast<const float4*>(swt[g][a]);
+                    const float wyz[U] = {wy.x * wz.x, wy.y * wz.y, wy.z * wz.z, wy.w * wz.w};
+#pragma unroll
+                    for (int k = 0; k < U; ++k) {
+                        ra[k].zero();
+#pragma unroll
+                        for (int b = 0; b < W; ++b) ra[k].fma(t[b], make_float2(wx[k][b], wx[k][b]));
+                        acc[k].fma(ra[k], make_float2(wyz[k], wyz[k]));
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                if (valid && k < un.y) acc[k].put(y + (int64_t)l * M + pti[un.x + k].w, M, L - l);
+        }
     }
 }
 
 // ------------------------------------------------------------ spreading
-// One sub-problem (<= HQS3_MAXPTS points of one TB^3 bin) is spread into a
-// (TB+W-1)^3 patch of LC coils (a power of two) in shared memory, then added
-// to the global grid with one float2 atomic per nonzero patch cell.  The
-// patch has no shared atomics: warp w owns the patch planes z = w (mod 8), so
-// for each point the (at most one) footprint plane of a warp is updated by
-// that warp alone, lanes over (cell, coil) entries of the plane, with a warp
-// barrier between points.  `unit` spreads the value 1 for every point (the
-// Toeplitz-kernel gridding).
+// Tile-owned type-1 spreading: each 8^3 tile of the grid is written once, with plain
+// stores, by the CTAs of its items (no atomics, no memset, a fixed order of the sums).
+// The plan lists the units (up to 4 points of one footprint) that touch each tile, with
+// the offset of their first tap; an item takes up to HQS3_ITEM of them, 32 at a time:
+// the weights and k-space values of a batch's points go to shared memory with cp.async
+// while the batch before is added.  A batch takes every (count / 32)-th entry, so that
+// it holds units of all planes and the warps meet its barriers together.
+// Warp w owns the tile's plane z = w; lane (x, coil group) keeps the 8 rows of its cell
+// column for CPL coils in registers, so a point updates a plane with exact y taps: its
+// value times the x and z weights once, then one packed multiply-add per row and coil,
+// the rows selected by a switch on the unit's y offset (registers need static names).
+// A tile with several items sums their partial tiles in slot order when the last
+// arrives.  Bound: instruction issue, the FMA pipe (about 19 packed operations per point
+// and plane) and the batches' barriers.  64^3 x 16 coils, 524,288 points, W 6: 824 us
+// against 2630 and a 41 us memset with patches of 4 coils added by atomics (a whole
+// adjoint 2824 -> 1013 us; units of one point and 256-point batches: 1297 us).
+#define HQS3_ITEM 256
+constexpr int kBatch3 = 32;    // units staged at once (one per lane of the plane test)
+// bytes of one point's slot: 32 weights, CL values
+template <int CPL> constexpr int spread3_slot() { return 128 + 4 * CPL * (int)sizeof(float2); }
+template <int CPL> constexpr size_t spread3_smem() { return (size_t)2 * kBatch3 * HQS3_UNIT * spread3_slot<CPL>(); }
+// n points (slots from sp on): wxl the byte offset of the lane's x weight, or -32; wzl
+// that of the plane's z weight; vl that of the lane's values
+template <int W, int CPL, int OY>
+HQS_DEV void spread_rows3(float2 (&acc)[HQS3_TILE][CPL], const char* sp, int n, int wxl, int wzl, int vl) {
+    constexpr int T = HQS3_TILE;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k, sp += spread3_slot<CPL>()) {
+        const float wx = *reinterpret_cast<const float*>(sp + (wxl & 31));
+        const float t = (wxl < 0 ? 0.f : wx) * *reinterpret_cast<const float*>(sp + wzl);
+        float2 u[CPL];
+        if constexpr (CPL == 4) {
+            const float4 v0 = *reinterpret_cast<const float4*>(sp + vl), v1 = *reinterpret_cast<const float4*>(sp + vl + 16);
+            u[0] = cmul_r(make_float2(v0.x, v0.y), t);
+            u[1] = cmul_r(make_float2(v0.z, v0.w), t);
+            u[2] = cmul_r(make_float2(v1.x, v1.y), t);
+            u[3] = cmul_r(make_float2(v1.z, v1.w), t);
+        } else {
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) u[c] = cmul_r(reinterpret_cast<const float2*>(sp + vl)[c], t);
+        }
+        const float4* wy = reinterpret_cast<const float4*>(sp + 64);
+#pragma unroll
+        for (int b = 0; b < W; ++b) {
+            if (OY + b < 0 || OY + b >= T) continue;
+            const float4 w4 = wy[b >> 1];
+            const float2 w = (b & 1) ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) acc[(OY + b) & (T - 1)][c] = cfma2(u[c], w, acc[(OY + b) & (T - 1)][c]);
+        }
+    }
+}
+template <int W, int CPL>
+__global__ void __launch_bounds__(256, 2)
+    k_spread3_tiles(const float2* __restrict__ ys, const float* __restrict__ kbw, const int2* __restrict__ list,
+                    const int4* __restrict__ items, const int2* __restrict__ tinfo, unsigned* __restrict__ tickets,
+                    float2* __restrict__ partial, int nbx, int nby, int Gx, int Gy, int L, float2* __restrict__ grid) {
+    constexpr int T = HQS3_TILE, CL = 4 * CPL, U = HQS3_UNIT, SLOT = spread3_slot<CPL>();
+    static_assert(T == 8 && W <= 8 && U == 4, "one plane per warp; two points per 32 lanes of copies");
+    extern __shared__ float4 smem4[];
+    char* sbuf = reinterpret_cast<char*>(smem4);   // [2][kBatch3 U] point slots
+    __shared__ int last;
+    const int4 it = items[blockIdx.x];
+    const int tile = it.x, l0 = blockIdx.y * CL, lc = min(CL, L - l0);
+    const int tx = tile % nbx, ty = (tile / nbx) % nby, tz = tile / (nbx * nby);
+    const int x0 = tx * T, y0 = ty * T, z0 = tz * T;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int xl = lane & 7, cq = lane >> 3;
+    float2 acc[T][CPL];
+#pragma unroll
+    for (int y = 0; y < T; ++y)
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) acc[y][c] = make_float2(0.f, 0.f);
+    // batch r: entries r, r + nbat, r + 2 nbat, ... of the item, lane i holding the i-th
+    // (0 beyond the item: no points, an offset that touches no plane)
+    const int cnt = it.z - it.y, nbat = (cnt + kBatch3 - 1) / kBatch3;
+    auto entry = [&](int r) {
+        const int e = r + lane * nbat;
+        return r < nbat && e < cnt ? __ldg(list + it.y + e) : make_int2(0, 0);
+    };
+    // this warp's share of a batch's copies: 4 entries, half a warp per point, lane q of
+    // the half-warp 16 bytes of weights (q < 8) or of values (pairs of coils, or single
+    // ones where an odd coil count leaves rows on 8-byte boundaries)
+    auto copy = [&](int2 ent, int buf) {
+        const int q = lane & 15;
+        const bool pairs = L % 2 == 0;
+#pragma unroll
+        for (int i = 0; i < kBatch3 / 8; ++i) {
+            const int e = warp * (kBatch3 / 8) + i;
+            const int first = __shfl_sync(0xffffffffu, ent.x, e), n = __shfl_sync(0xffffffffu, ent.y, e) >> 24;
+#pragma unroll
+            for (int h = 0; h < U / 2; ++h) {
+                const int k = 2 * h + (lane >> 4);
+                if (k >= n) continue;
+                char* d = sbuf + (size_t)((buf * kBatch3 + e) * U + k) * SLOT;
+                if (q < 8) {
+                    cp_async16(d + 16 * q, kbw + (int64_t)(first + k) * 32 + 4 * q);
+                } else {
+                    const float2* src = ys + (int64_t)(first + k) * L + l0;
+                    const int c = 2 * (q - 8);
+                    if (pairs && c < lc) {
+                        cp_async16(d + 128 + 8 * c, src + c);
+                    } else if (!pairs) {
+                        if (c < lc) cp_async8(d + 128 + 8 * c, src + c);
+                        if (c + 1 < lc) cp_async8(d + 136 + 8 * c, src + c + 1);
+                    }
+                }
+            }
+        }
+        cp_async_commit();
+    };
+    int2 cur = entry(0), nxt = entry(1);
+    copy(cur, 0);
+    for (int r = 0; r < nbat; ++r) {
+        const int2 nn = entry(r + 2);
+        copy(nxt, (r + 1) & 1);   // empty after the last batch
+        cp_async_wait_group<1>();
+        __syncthreads();
+        // the batch's units of this warp's plane
+        unsigned mask = __ballot_sync(0xffffffffu, (unsigned)(warp - (((cur.y >> 16) & 255) - 16)) < (unsigned)W);
+        while (mask) {
+            const int b = __ffs(mask) - 1;
+            mask &= mask - 1;
+            const int off = __shfl_sync(0xffffffffu, cur.y, b);
+            const char* sp = sbuf + (size_t)(((r & 1) * kBatch3 + b) * U) * SLOT;
+            const int bx = xl - ((off & 255) - 16);
+            const int wxl = (unsigned)bx < (unsigned)W ? 4 * bx : -32;   // -32: reads tap 0, counts as 0
+            const int wzl = 32 + 4 * (warp - (((off >> 16) & 255) - 16));
+            const int vl = 128 + cq * CPL * (int)sizeof(float2);
+            const int n = off >> 24;
+            switch (((off >> 8) & 255) - 16) {
+#define HQS3_ROWS(OY)                                                                  \
+    case OY:                                                                           \
+        if constexpr (OY > -W) spread_rows3<W, CPL, OY>(acc, sp, n, wxl, wzl, vl);     \
+        break;
+                HQS3_ROWS(-7) HQS3_ROWS(-6) HQS3_ROWS(-5) HQS3_ROWS(-4) HQS3_ROWS(-3)
+                HQS3_ROWS(-2) HQS3_ROWS(-1) HQS3_ROWS(0) HQS3_ROWS(1) HQS3_ROWS(2)
+                HQS3_ROWS(3) HQS3_ROWS(4) HQS3_ROWS(5) HQS3_ROWS(6) HQS3_ROWS(7)
+#undef HQS3_ROWS
+            }
+        }
+        __syncthreads();
+        cur = nxt;
+        nxt = nn;
+    }
+    cp_async_wait_all();
+    // the lane's column x of plane `warp`: CPL coils from coil cq CPL on
+    auto put = [&](float2* d, const float2* v, int n, bool pairs) {
+        if (CPL >= 2 && pairs && n == CPL) {
+#pragma unroll
+            for (int c = 0; c + 1 < CPL; c += 2)
+                reinterpret_cast<float4*>(d)[c / 2] = make_float4(v[c].x, v[c].y, v[c + 1].x, v[c + 1].y);
+        } else {
+#pragma unroll
+            for (int c = 0; c < CPL; ++c)
+                if (c < n) d[c] = v[c];
+        }
+    };
+    const int ncoil = lc - cq * CPL;   // coils of this lane that exist (may be <= 0)
+    float2* gcell = grid + (((int64_t)(z0 + warp) * Gy + y0) * Gx + x0 + xl) * L + l0 + cq * CPL;
+    const int64_t grow = (int64_t)Gx * L;
+    if (it.w < 0) {
+#pragma unroll
+        for (int y = 0; y < T; ++y) put(gcell + y * grow, acc[y], min(ncoil, CPL), L % 2 == 0);
+        return;
+    }
+    const int64_t slot = (int64_t)gridDim.y * kCells3 * CL;
+    float2* pcell = partial + ((int64_t)blockIdx.y * kCells3 + warp * T * T + xl) * CL + cq * CPL;
+#pragma unroll
+    for (int y = 0; y < T; ++y) put(pcell + it.w * slot + y * T * CL, acc[y], CPL, true);
+    __threadfence();
+    __syncthreads();
+    const int2 ti = tinfo[tile];
+    unsigned* ticket = tickets + (int64_t)tile * gridDim.y + blockIdx.y;
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == (unsigned)(ti.x - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int y = 0; y < T; ++y) {
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) acc[y][c] = make_float2(0.f, 0.f);
+    }
+    for (int k = 0; k < ti.x; ++k) {
+        const float2* pc = pcell + (ti.y + k) * slot;
+#pragma unroll
+        for (int y = 0; y < T; ++y)
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) acc[y][c] = cadd(acc[y][c], __ldcg(pc + y * T * CL + c));
+    }
+#pragma unroll
+    for (int y = 0; y < T; ++y) put(gcell + y * grow, acc[y], min(ncoil, CPL), L % 2 == 0);
+    if (threadIdx.x == 0) *ticket = 0u;
+}
+
+// Unit data (the Toeplitz kernel's gridding at plan time): one sub-problem (<=
+// HQS3_MAXPTS points of one 8^3 bin) is spread into a (8 + W - 1)^3 patch in shared
+// memory, then added to the zeroed grid with one atomic per nonzero cell.  Warp w owns
+// the patch planes z = w (mod 8), so a point's footprint plane is updated by one warp.
 #define HQS3_SPREAD_WARPS 8
 template <int W>
 __global__ void __launch_bounds__(HQS3_SPREAD_WARPS * 32)
-    k_spread3(const float2* __restrict__ y, const int4* __restrict__ pti, const float4* __restrict__ ptd,
-              const int4* __restrict__ subs, int64_t M, int Gx, int Gy, int Gz, int L, int lcs, int nchunk,
-              int TB, int nbx, int nby, float beta, int unit, float2* __restrict__ grid) {
+    k_spread3_unit(const int4* __restrict__ pti, const float4* __restrict__ ptd, const int4* __restrict__ subs, int Gx,
+                   int Gy, int Gz, int nbx, int nby, float beta, float2* __restrict__ grid) {
     static_assert(W <= HQS3_SPREAD_WARPS, "one footprint plane per warp and point");
+    constexpr int TB = HQS3_TILE, P = TB + W - 1, P3 = P * P * P;
     extern __shared__ float4 smem4[];
-    const int LC = 1 << lcs;
-    const int P = TB + W - 1;
-    const int P3 = P * P * P;
     int4* loc = reinterpret_cast<int4*>(smem4);
     float* wts = reinterpret_cast<float*>(loc + HQS3_MAXPTS);
-    float2* vals = reinterpret_cast<float2*>(wts + HQS3_MAXPTS * 3 * W);
-    float2* patch = vals + HQS3_MAXPTS * LC;
+    float* patch = wts + HQS3_MAXPTS * 3 * W;
     const int4 sb = subs[blockIdx.x];
     const int bin = sb.x, start = sb.y, cnt = sb.z;
     const int bx = bin % nbx, by = (bin / nbx) % nby, bz = bin / (nbx * nby);
@@ -246,59 +614,29 @@ __global__ void __launch_bounds__(HQS3_SPREAD_WARPS * 32)
         const int cx = wrap(pi.x + W / 2, Gx), cy = wrap(pi.y + W / 2, Gy), cz = wrap(pi.z + W / 2, Gz);
         loc[i] = make_int4(cx - bx * TB, cy - by * TB, cz - bz * TB, pi.w);
     }
-    __syncthreads();   // loc and wts are read by other threads below
+    for (int e = threadIdx.x; e < P3; e += blockDim.x) patch[e] = 0.f;
+    __syncthreads();   // loc, wts and the patch are read by other threads below
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ox = bx * TB - W / 2, oy = by * TB - W / 2, oz = bz * TB - W / 2;
-    // lane -> (x tap b, coil l) of a footprint row; W * LC <= 32 (LC = 4 needs W <= 6,
-    // the launcher uses LC <= 2 above that)
-    const bool has_tap = lane < (W << lcs);
-    const int lb = lane >> lcs, ll = lane & ((1 << lcs) - 1);
-    for (int ch = blockIdx.y; ch < nchunk; ch += gridDim.y) {
-        const int l0 = ch * LC;
-        const int lines = min(LC, L - l0);
-        for (int e = threadIdx.x; e < P3 * LC; e += blockDim.x) patch[e] = make_float2(0.f, 0.f);
-        for (int e = threadIdx.x; e < cnt * LC; e += blockDim.x) {
-            const int i = e >> lcs, l = e & (LC - 1);
-            float2 v = make_float2(0.f, 0.f);
-            if (l < lines) v = unit ? make_float2(1.f, 0.f) : y[(int64_t)(l0 + l) * M + loc[i].w];
-            vals[e] = v;
-        }
-        __syncthreads();
-        for (int i = 0; i < cnt; ++i) {
-            const int4 c0 = loc[i];
-            const int c = ((warp - c0.z) % HQS3_SPREAD_WARPS + HQS3_SPREAD_WARPS) % HQS3_SPREAD_WARPS;
-            if (c < W && has_tap) {
-                // this lane's (b, l): the value times the z and x weights once, then down
-                // the W rows of the plane
-                const float* wv = wts + i * 3 * W;
-                const float wzx = wv[2 * W + c] * wv[lb];
-                const float2 v = vals[(i << lcs) + ll];
-                const float2 t = make_float2(v.x * wzx, v.y * wzx);
-                float2* col = patch + ((((c0.z + c) * P + c0.y) * P + c0.x + lb) << lcs) + ll;
+    for (int i = 0; i < cnt; ++i) {
+        const int4 c0 = loc[i];
+        const int c = ((warp - c0.z) % HQS3_SPREAD_WARPS + HQS3_SPREAD_WARPS) % HQS3_SPREAD_WARPS;
+        if (c < W && lane < W) {
+            const float* wv = wts + i * 3 * W;
+            const float t = wv[2 * W + c] * wv[lane];
+            float* col = patch + ((c0.z + c) * P + c0.y) * P + c0.x + lane;
 #pragma unroll
-                for (int a = 0; a < W; ++a) {
-                    const float wy = wv[W + a];
-                    float2* dst = col + ((a * P) << lcs);
-                    float2 acc = *dst;
-                    acc.x = fmaf(wy, t.x, acc.x);
-                    acc.y = fmaf(wy, t.y, acc.y);
-                    *dst = acc;
-                }
-            }
-            __syncwarp();
+            for (int a = 0; a < W; ++a) col[a * P] = fmaf(wv[W + a], t, col[a * P]);
         }
-        __syncthreads();
-        for (int e = threadIdx.x; e < P3 * LC; e += blockDim.x) {
-            const int l = e & (LC - 1);
-            if (l >= lines) continue;
-            const float2 v = patch[e];
-            if (v.x == 0.f && v.y == 0.f) continue;
-            const int cell = e >> lcs;
-            const int cx = cell % P, cy = (cell / P) % P, cz = cell / (P * P);
-            const int gx = wrap(ox + cx, Gx), gy = wrap(oy + cy, Gy), gz = wrap(oz + cz, Gz);
-            atomicAdd(&grid[(((int64_t)gz * Gy + gy) * Gx + gx) * L + l0 + l], v);
-        }
-        __syncthreads();
+        __syncwarp();
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < P3; e += blockDim.x) {
+        const float v = patch[e];
+        if (v == 0.f) continue;
+        const int cx = e % P, cy = (e / P) % P, cz = e / (P * P);
+        const int gx = wrap(ox + cx, Gx), gy = wrap(oy + cy, Gy), gz = wrap(oz + cz, Gz);
+        atomicAdd(&grid[((int64_t)gz * Gy + gy) * Gx + gx].x, v);
     }
 }
 
@@ -895,10 +1233,11 @@ struct Points3 {
     int4* subs = nullptr;
     int nsub = 0;
     int nb[3] = {0, 0, 0};
+    std::vector<int> off;   // [bins + 1] first point of each bin
 };
 
 int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], int W, Points3* out,
-                 bool owned, cudaStream_t s) {
+                 cudaStream_t s) {
     for (int a = 0; a < 3; ++a) out->nb[a] = G[a] / HQS3_TILE;
     const int nbins = out->nb[0] * out->nb[1] * out->nb[2];
     int4* rawi = nullptr;
@@ -919,10 +1258,7 @@ int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], 
     }
     int rc = HQS_OK;
     do {
-        if (owned) {
-            if ((rc = alloc3(p, &out->pti, (size_t)Mp)) != HQS_OK) break;
-            if ((rc = alloc3(p, &out->ptd, (size_t)Mp)) != HQS_OK) break;
-        } else if (cudaMalloc(&out->pti, Mp * sizeof(int4)) || cudaMalloc(&out->ptd, Mp * sizeof(float4))) {
+        if (cudaMalloc(&out->pti, Mp * sizeof(int4)) || cudaMalloc(&out->ptd, Mp * sizeof(float4))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -933,7 +1269,8 @@ int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], 
         std::vector<int> hc(nbins);
         if (cudaMemcpyAsync(hc.data(), counts, nbins * sizeof(int), cudaMemcpyDeviceToHost, s) ||
             cudaStreamSynchronize(s)) { rc = HQS_ERR_CUDA; break; }
-        std::vector<int> offs(nbins);
+        std::vector<int>& offs = out->off;
+        offs.resize(nbins + 1);
         std::vector<int4> subs;
         int acc = 0;
         for (int b = 0; b < nbins; ++b) {
@@ -942,10 +1279,9 @@ int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], 
                 subs.push_back(make_int4(b, acc + st, std::min(HQS3_MAXPTS, hc[b] - st), 0));
             acc += hc[b];
         }
+        offs[nbins] = acc;
         out->nsub = (int)subs.size();
-        if (owned) {
-            if ((rc = alloc3(p, &out->subs, subs.size())) != HQS_OK) break;
-        } else if (cudaMalloc(&out->subs, std::max<size_t>(subs.size(), 1) * sizeof(int4))) {
+        if (cudaMalloc(&out->subs, std::max<size_t>(subs.size(), 1) * sizeof(int4))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -978,28 +1314,161 @@ template <class F> int dispatch_w3(int W, F&& f) {
     }
 }
 
-// Spread y (or unit data) onto `grid` (zeroed here) of size G with L coils.
-int spread3(const Points3& pts, const float2* y, int64_t M, const int G[3], int L, int W, double beta,
-            bool unit, float2* grid, cudaStream_t s) {
-    const size_t cells = (size_t)G[0] * G[1] * G[2] * L;
-    HQS_CUDA_TRY(cudaMemsetAsync(grid, 0, cells * sizeof(float2), s));
+// Spread unit data onto `grid` (zeroed here) of size G, the kernel's width.
+int spread3_unit(const Points3& pts, const int G[3], double beta, float2* grid, cudaStream_t s) {
+    constexpr int W = HQS3_KERNEL_W, P = HQS3_TILE + W - 1;
+    HQS_CUDA_TRY(cudaMemsetAsync(grid, 0, (size_t)G[0] * G[1] * G[2] * sizeof(float2), s));
     if (pts.nsub == 0) return HQS_OK;
-    return dispatch_w3(W, [&]<int WW>() {
-        const int P = HQS3_TILE + WW - 1;
-        const size_t cell_bytes = (size_t)P * P * P * sizeof(float2);
-        // coils per chunk: 4, or 2 where a 4-coil patch would exceed 72 KB or the
-        // W x 4 (tap, coil) lanes a warp (W > 6), or 1 for one coil
-        int lcs = (cell_bytes * 4 <= 72 * 1024 && WW <= 6) ? 2 : 1;
-        while (lcs > 0 && (1 << (lcs - 1)) >= L) --lcs;
-        const int nch = ceil_div(L, 1 << lcs);
-        const size_t sm = HQS3_MAXPTS * sizeof(int4) + HQS3_MAXPTS * 3 * WW * sizeof(float) +
-                          (size_t)HQS3_MAXPTS * (1 << lcs) * sizeof(float2) + cell_bytes * (1 << lcs);
-        HQS_CUDA_TRY(cudaFuncSetAttribute(k_spread3<WW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k_spread3<WW><<<dim3(pts.nsub, nch), HQS3_SPREAD_WARPS * 32, sm, s>>>(
-            y, pts.pti, pts.ptd, pts.subs, M, G[0], G[1], G[2], L, lcs, nch, HQS3_TILE, pts.nb[0], pts.nb[1],
-            (float)beta, unit ? 1 : 0, grid);
-        HQS_CUDA_TRY(cudaGetLastError());
-        return HQS_OK;
+    const size_t sm = HQS3_MAXPTS * (sizeof(int4) + 3 * W * sizeof(float)) + (size_t)P * P * P * sizeof(float);
+    HQS_CUDA_TRY(cudaFuncSetAttribute(k_spread3_unit<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    k_spread3_unit<W><<<pts.nsub, HQS3_SPREAD_WARPS * 32, sm, s>>>(pts.pti, pts.ptd, pts.subs, G[0], G[1], G[2],
+                                                                  pts.nb[0], pts.nb[1], (float)beta, grid);
+    HQS_CUDA_TRY(cudaGetLastError());
+    return HQS_OK;
+}
+
+// coils per lane of the tile-owned spreading (4 lanes share a cell)
+int spread3_cpl(int L) { return L <= 4 ? 1 : (L <= 8 ? 2 : 4); }
+
+// The plan's points in footprint order, their weights, the interpolation's units and the
+// spreading's items, from the points in bin order (host offsets pts.off).
+int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
+    const int nbins = pts.nb[0] * pts.nb[1] * pts.nb[2];
+    const int Gx = p->G[0], Gy = p->G[1], Gz = p->G[2], W = p->W;
+    const size_t Mp = (size_t)std::max<int64_t>(p->M, 1);
+    TRY3(alloc3(p, &p->pti, Mp));
+    TRY3(alloc3(p, &p->inv, Mp));
+    TRY3(alloc3(p, &p->kbw, Mp * 32));
+    TRY3(alloc3(p, &p->ysort, Mp * p->L));
+    float4* ptd = nullptr;
+    int *binoff = nullptr, *ucnt = nullptr, *tcnt = nullptr;
+    auto cleanup = [&]() {
+        cudaFree(ptd);
+        cudaFree(binoff);
+        cudaFree(ucnt);
+        cudaFree(tcnt);
+    };
+    int rc = HQS_OK;
+    do {
+        if (cudaMalloc(&ptd, Mp * sizeof(float4)) || cudaMalloc(&ucnt, nbins * sizeof(int)) ||
+            cudaMalloc(&tcnt, nbins * sizeof(int)) || cudaMalloc(&binoff, (nbins + 1) * sizeof(int))) {
+            rc = HQS_ERR_OOM;
+            break;
+        }
+        if (cudaMemcpyAsync(binoff, pts.off.data(), (nbins + 1) * sizeof(int), cudaMemcpyHostToDevice, s) ||
+            cudaMemsetAsync(tcnt, 0, nbins * sizeof(int), s)) {
+            rc = HQS_ERR_CUDA;
+            break;
+        }
+        k_bin_sort3<<<nbins, 256, 0, s>>>(pts.pti, pts.ptd, binoff, W, Gx, Gy, Gz, p->pti, ptd, p->inv, ucnt);
+        if (p->M > 0)
+            k_weights3<<<(unsigned)ceil_div64(p->M * 24, 256), 256, 0, s>>>(ptd, p->M, W, (float)p->beta, p->kbw);
+        std::vector<int> uc(nbins), tc(nbins);
+        if (cudaMemcpyAsync(uc.data(), ucnt, nbins * sizeof(int), cudaMemcpyDeviceToHost, s) ||
+            cudaStreamSynchronize(s)) {
+            rc = HQS_ERR_CUDA;
+            break;
+        }
+        int nu = 0;
+        for (int b = 0; b < nbins; ++b) {
+            const int c = uc[b];
+            uc[b] = nu;
+            nu += c;
+        }
+        p->nunits = nu;
+        if ((rc = alloc3(p, &p->units, (size_t)std::max(nu, 1))) != HQS_OK) break;
+        if (cudaMemcpyAsync(ucnt, uc.data(), nbins * sizeof(int), cudaMemcpyHostToDevice, s)) {
+            rc = HQS_ERR_CUDA;
+            break;
+        }
+        k_units3<<<nbins, 256, 0, s>>>(p->pti, binoff, ucnt, W, Gx, Gy, Gz, p->units);
+        const unsigned ublk = (unsigned)ceil_div(nu, 256);
+        if (nu > 0) k_tile_count3<<<ublk, 256, 0, s>>>(p->pti, p->units, nu, W, Gx, Gy, Gz, tcnt);
+        if (cudaMemcpyAsync(tc.data(), tcnt, nbins * sizeof(int), cudaMemcpyDeviceToHost, s) ||
+            cudaStreamSynchronize(s)) {
+            rc = HQS_ERR_CUDA;
+            break;
+        }
+        // spreading items, heaviest first: every tile's entries in pieces of HQS3_ITEM
+        std::vector<int4> items;
+        std::vector<int2> tinfo(nbins);
+        int slots = 0;
+        int64_t entries = 0;
+        for (int t = 0; t < nbins; ++t) {
+            const int64_t n = tc[t];
+            const int k = (int)std::max<int64_t>(1, ceil_div64(n, HQS3_ITEM));
+            tc[t] = (int)entries;
+            tinfo[t] = make_int2(k, k > 1 ? slots : -1);
+            for (int i = 0; i < k; ++i)
+                items.push_back(make_int4(t, (int)(entries + n * i / k), (int)(entries + n * (i + 1) / k),
+                                          k > 1 ? slots + i : -1));
+            if (k > 1) slots += k;
+            entries += n;
+        }
+        if (entries > 0x7fffffffLL) {
+            rc = HQS_ERR_INVALID_ARG;
+            break;
+        }
+        if ((rc = alloc3(p, &p->list, (size_t)entries)) != HQS_OK) break;
+        if (cudaMemcpyAsync(tcnt, tc.data(), nbins * sizeof(int), cudaMemcpyHostToDevice, s)) {
+            rc = HQS_ERR_CUDA;
+            break;
+        }
+        if (nu > 0) k_tile_fill3<<<ublk, 256, 0, s>>>(p->pti, p->units, nu, W, Gx, Gy, Gz, tcnt, p->list);
+        std::stable_sort(items.begin(), items.end(),
+                         [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
+        p->nitems = (int)items.size();
+        const int cl = 4 * spread3_cpl(p->L), nch = ceil_div(p->L, cl);
+        if ((rc = alloc3(p, &p->items, items.size())) != HQS_OK) break;
+        if ((rc = alloc3(p, &p->tinfo, tinfo.size())) != HQS_OK) break;
+        if ((rc = alloc3(p, &p->tickets, (size_t)nbins * nch)) != HQS_OK) break;
+        if ((rc = alloc3(p, &p->partial, (size_t)slots * nch * kCells3 * cl)) != HQS_OK) break;
+        if (cudaMemcpyAsync(p->items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, s) ||
+            cudaMemcpyAsync(p->tinfo, tinfo.data(), tinfo.size() * sizeof(int2), cudaMemcpyHostToDevice, s) ||
+            cudaMemsetAsync(p->tickets, 0, (size_t)nbins * nch * sizeof(unsigned), s) ||
+            cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
+            rc = HQS_ERR_CUDA;
+    } while (0);
+    cleanup();
+    return rc;
+}
+
+// Spread the k-space data y onto the plan's grid (every cell written).
+int spread3(hqs_plan3d_s* p, const float2* y, float2* grid, cudaStream_t s) {
+    TRY3(launch_y_to_sorted(y, p->inv, p->M, p->L, p->ysort, s));
+    const int cpl = spread3_cpl(p->L), nch = ceil_div(p->L, 4 * cpl);
+    return dispatch_w3(p->W, [&]<int WW>() {
+        auto go = [&]<int CPL>() {
+            const size_t sm = spread3_smem<CPL>();
+            auto kern = k_spread3_tiles<WW, CPL>;
+            HQS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            kern<<<dim3(p->nitems, nch), 256, sm, s>>>(p->ysort, p->kbw, p->list, p->items, p->tinfo, p->tickets,
+                                                      p->partial, p->nb[0], p->nb[1], p->G[0], p->G[1], p->L, grid);
+            HQS_CUDA_TRY(cudaGetLastError());
+            return HQS_OK;
+        };
+        return cpl == 1 ? go.template operator()<1>() : (cpl == 2 ? go.template operator()<2>() : go.template operator()<4>());
+    });
+}
+
+// Interpolate the plan's grid at the points: lanes per unit and coils per lane by the
+// coil count (pairs of coils as 16-byte loads need an even count).
+int interp3(hqs_plan3d_s* p, const float2* grid, float2* y, cudaStream_t s) {
+    if (p->M == 0) return HQS_OK;
+    return dispatch_w3(p->W, [&]<int WW>() {
+        auto go = [&]<int VEC, int LPP>() {
+            // several units one after the other only where the CTAs fill the GPU all the same
+            // (a whole forward at 16 x 64 x 64 x 2 coils, 5,568 points: 97 us with 4 rounds on 11
+            // CTAs, 44 us with one)
+            constexpr int NG = 256 / LPP;
+            const int rounds = std::max(1, std::min(kInterpRounds, p->nunits / (NG * 2 * 152)));
+            k_interp3<WW, VEC, LPP><<<ceil_div(p->nunits, NG * rounds), 256, 0, s>>>(
+                grid, p->pti, p->kbw, p->units, p->nunits, rounds, p->M, p->G[0], p->G[1], p->G[2], p->L, y);
+            HQS_CUDA_TRY(cudaGetLastError());
+            return HQS_OK;
+        };
+        if (p->L % 2 == 0) return p->L > 4 ? go.template operator()<2, 8>() : go.template operator()<2, 2>();
+        return p->L > 4 ? go.template operator()<1, 16>() : go.template operator()<1, 4>();
     });
 }
 
@@ -1022,26 +1491,13 @@ int fwd3(hqs_plan3d_s* p, const float2* x, float2* y, cudaStream_t s) {
     const int64_t plane = (int64_t)Gy * row;
     TRY3((run_pass<false, false, false>(p, Gz, LdCentred{p->bufB, {0, plane}, nz, Gz},
                                         StLine{p->bufA, {0, plane}, Gz, 0, Gz}, plane, plane, s)));
-    if (p->M == 0) return HQS_OK;
-    return dispatch_w3(p->W, [&]<int WW>() {
-        const int64_t threads = p->M * 16;
-        k_interp3<WW><<<(unsigned)ceil_div64(threads, 256), 256, 0, s>>>(p->bufA, p->pti, p->ptd, (int)p->M, Gx,
-                                                                        Gy, Gz, L, (float)p->beta, y);
-        HQS_CUDA_TRY(cudaGetLastError());
-        return HQS_OK;
-    });
+    return interp3(p, p->bufA, y, s);
 }
 
 int adj3(hqs_plan3d_s* p, const float2* y, float2* x, cudaStream_t s) {
     const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
     const int Gx = p->G[0], Gy = p->G[1], Gz = p->G[2], L = p->L;
-    Points3 pts;
-    pts.pti = p->pti;
-    pts.ptd = p->ptd;
-    pts.subs = p->subs;
-    pts.nsub = p->nsub;
-    for (int a = 0; a < 3; ++a) pts.nb[a] = p->nb[a];
-    TRY3(spread3(pts, y, p->M, p->G, L, p->W, p->beta, false, p->bufA, s));
+    TRY3(spread3(p, y, p->bufA, s));
     const int64_t row = (int64_t)Gx * L, plane = (int64_t)Gy * row;
     // z: [nz][Gy][Gx][L] in bufB
     TRY3((run_pass<true, false, false>(p, Gz, LdLine{p->bufA, {0, plane}, Gz},
@@ -1185,8 +1641,8 @@ int build_khat(hqs_plan3d_s* p, const float* traj, cudaStream_t s) {
             }
         }
         if (rc != HQS_OK) break;
-        if ((rc = build_points(p, traj, p->M, G4, Wk, &pts, false, s)) != HQS_OK) break;
-        if ((rc = spread3(pts, nullptr, p->M, G4, 1, Wk, bk, true, grid, s)) != HQS_OK) break;
+        if ((rc = build_points(p, traj, p->M, G4, Wk, &pts, s)) != HQS_OK) break;
+        if ((rc = spread3_unit(pts, G4, bk, grid, s)) != HQS_OK) break;
         // z: [2nz][4ny][4nx] in mid (circulant crop)
         const int64_t row4 = G4[0], plane4 = (int64_t)G4[1] * G4[0];
         if ((rc = run_pass<true, false, false>(p, G4[2], LdLine{grid, {0, plane4}, G4[2]},
@@ -1285,13 +1741,17 @@ int plan3d_build(hqs_plan3d_s* p, const float* traj, const float2* smaps_user, c
     k_smaps3_coil_inner<<<(unsigned)std::min<int64_t>(ceil_div64(nvox * L, 256), 8192), 256, 0, s>>>(
         smaps_user, p->smaps, nvox, L);
     HQS_CUDA_TRY(cudaGetLastError());
-    Points3 pts;
-    TRY3(build_points(p, traj, p->M, p->G, p->W, &pts, true, s));
-    p->pti = pts.pti;
-    p->ptd = pts.ptd;
-    p->subs = pts.subs;
-    p->nsub = pts.nsub;
-    for (int a = 0; a < 3; ++a) p->nb[a] = pts.nb[a];
+    {
+        Points3 pts;   // bin order, freed once the footprint order is made
+        int rc = build_points(p, traj, p->M, p->G, p->W, &pts, s);
+        for (int a = 0; a < 3; ++a) p->nb[a] = pts.nb[a];
+        p->nsub = pts.nsub;
+        if (rc == HQS_OK) rc = order_points(p, pts, s);
+        cudaFree(pts.pti);
+        cudaFree(pts.ptd);
+        cudaFree(pts.subs);
+        if (rc != HQS_OK) return rc;
+    }
     if (p->M > 0) {
         TRY3(build_khat(p, traj, s));
     } else {

@@ -132,6 +132,8 @@ int launch_half_group(int G, int n, int maxchunk, int count, const void* d_tab, 
                       cudaStream_t s);
 int launch_spread(hqs_plan_s* p, const float2* y, cudaStream_t s);
 int launch_interp(hqs_plan_s* p, float2* y, cudaStream_t s);
+// ysort[inv[m]][l] = y[l][m] (csrc/nufft.cu)
+int launch_y_to_sorted(const float2* y, const int* inv, int64_t M, int L, float2* ysort, cudaStream_t s);
 int launch_adj_chunks(hqs_plan_s* p, float2* x, float zc, const float2* z, cudaStream_t s);
 int launch_toeplitz(hqs_plan_s* p, const float2* x, float2* out, cudaStream_t s);
 int launch_fft2d(const hqs_plan_s* p, float2* data, int N, bool inverse, cudaStream_t s);
