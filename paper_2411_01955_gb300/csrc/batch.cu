@@ -946,7 +946,7 @@ struct hqs_batch_s {
     // batched forward / adjoint: the lower-half passes' argument tables of the slices
     // that take them, grouped by grid size (rebuilt when the pointers change)
     struct HalfGroup {
-        int G, n, maxchunk, first, count;
+        int G, n, lines, maxchunk, first, count;
     };
     void* d_half[2] = {nullptr, nullptr};   // [0] forward, [1] adjoint
     std::vector<HalfGroup> half_groups[2];
@@ -1318,8 +1318,8 @@ extern "C" int hqs_batch_toeplitz_normal(hqs_batch b, const hqs_c64* const* x, h
 }
 
 // Argument tables of the batched lower-half passes (dir 0: forward x -> grid,
-// dir 1: adjoint grid -> x with the axpy term z), grouped by grid size in slice
-// order; uploaded when the image pointers differ from the last call.
+// dir 1: adjoint grid -> x with the axpy term z), grouped by grid size and lines per
+// CTA in slice order; uploaded when the image pointers differ from the last call.
 static int half_tables(hqs_batch_s* b, int dir, const float2* const* xin, float2* const* xout,
                        const float2* const* z, cudaStream_t st) {
     std::vector<const void*> key;
@@ -1340,10 +1340,10 @@ static int half_tables(hqs_batch_s* b, int dir, const float2* const* xin, float2
     for (int i = 0; i < b->ns; ++i) {
         const hqs_plan_s* p = b->plans[i];
         if (done[i] || !plan_half_passes(p)) continue;
-        hqs_batch_s::HalfGroup g{p->G, p->n, 0, slot, 0};
+        hqs_batch_s::HalfGroup g{p->G, p->n, plan_half_lines(p), 0, slot, 0};
         for (int j = i; j < b->ns; ++j) {
             const hqs_plan_s* q = b->plans[j];
-            if (done[j] || !plan_half_passes(q) || q->G != p->G) continue;
+            if (done[j] || !plan_half_passes(q) || q->G != p->G || plan_half_lines(q) != g.lines) continue;
             fill_half_args(q, xin ? xin[j] : nullptr, xout ? xout[j] : nullptr, z ? z[j] : nullptr,
                            host.data() + sz * slot);
             g.maxchunk = std::max(g.maxchunk, q->nchunk);
@@ -1379,7 +1379,7 @@ extern "C" int hqs_batch_adjoint_axpy(hqs_batch b, const hqs_c64* const* y, floa
     }
     const size_t sz = half_args_bytes();
     for (const auto& g : b->half_groups[1])
-        HQS_TRY_RC(launch_half_group(g.G, g.n, g.maxchunk, g.count,
+        HQS_TRY_RC(launch_half_group(g.G, g.n, g.lines, g.maxchunk, g.count,
                                      static_cast<unsigned char*>(b->d_half[1]) + sz * g.first, 1, zc, st));
     for (int i = 0; i < b->ns; ++i)
         if (plan_half_passes(b->plans[i])) HQS_TRY_RC(launch_adj_chunks(b->plans[i], X[i], zc, Z ? Z[i] : nullptr, st));
@@ -1396,7 +1396,7 @@ extern "C" int hqs_batch_forward(hqs_batch b, const hqs_c64* const* x, hqs_c64* 
     HQS_TRY_RC(half_tables(b, 0, Xin, nullptr, nullptr, st));
     const size_t sz = half_args_bytes();
     for (const auto& g : b->half_groups[0])
-        HQS_TRY_RC(launch_half_group(g.G, g.n, g.maxchunk, g.count,
+        HQS_TRY_RC(launch_half_group(g.G, g.n, g.lines, g.maxchunk, g.count,
                                      static_cast<unsigned char*>(b->d_half[0]) + sz * g.first, 0, 0.f, st));
     for (int i = 0; i < b->ns; ++i) {
         hqs_plan_s* p = b->plans[i];

@@ -106,8 +106,9 @@ template <int LINES> HQS_DEV float2 swap_pair(float2 v) {
 
 // Forward head: ld(pos) reads the line's element pos < N/2 (the upper half is zero).
 // Every thread of the CTA calls it (the loads of threads without a line read the
-// caller's clamped line); no barrier inside.
-template <int N, int LINES, class LD> HQS_DEV void fft16_head(float2* s, const Lane16& T, LD&& ld) {
+// caller's clamped line); no barrier inside.  ROT: output k times i^k (the image's
+// centring, i^(kk + 16 m) = i^kk, folded into the lane factors).
+template <int N, int LINES, bool ROT = false, class LD> HQS_DEV void fft16_head(float2* s, const Lane16& T, LD&& ld) {
     constexpr int R = Fft16<N>::R, SUB = Fft16<N>::SUB;
     const bool odd = T.par != 0;
     float2 o[SUB][4];
@@ -123,6 +124,10 @@ template <int N, int LINES, class LD> HQS_DEV void fft16_head(float2* s, const L
         const float2 b = sel(odd, make_float2(-w16(3 * q).x, -w16(3 * q).y), w16(2 * q));
         ca[q] = make_float2(a.x, -a.y);
         cb[q] = make_float2(b.x, -b.y);
+        if (ROT) {   // kk = 4 m + par for the sums, 4 m + 2 + par for the differences
+            ca[q] = sel(odd, make_float2(-ca[q].y, ca[q].x), ca[q]);
+            cb[q] = sel(odd, make_float2(cb[q].y, -cb[q].x), make_float2(-cb[q].x, -cb[q].y));
+        }
     }
 #pragma unroll
     for (int b = 0; b < SUB; ++b) {
@@ -134,7 +139,7 @@ template <int N, int LINES, class LD> HQS_DEV void fft16_head(float2* s, const L
             const float2 w = sel(odd, make_float2(o[b][q].y, -o[b][q].x), o[b][q]);
             e[q] = cadd(w, p);
             f[q] = csub(w, p);
-            if (q > 0) {
+            if (q > 0 || ROT) {
                 e[q] = cmul(e[q], ca[q]);
                 f[q] = cmul(f[q], cb[q]);
             } else {
@@ -153,8 +158,9 @@ template <int N, int LINES, class LD> HQS_DEV void fft16_head(float2* s, const L
 }
 
 // Inverse tail: the lane's 4 outputs of each of its SUB columns go to put(b, q, pos, v),
-// pos = tp + 8 b + R (4 par + q) < N/2.
-template <int N, int LINES, class PUT> HQS_DEV void fft16_tail(const float2* s, const Lane16& T, PUT&& put) {
+// pos = tp + 8 b + R (4 par + q) < N/2.  ROT: the transformed line was (-i)^k times the
+// one given.
+template <int N, int LINES, bool ROT = false, class PUT> HQS_DEV void fft16_tail(const float2* s, const Lane16& T, PUT&& put) {
     constexpr int R = Fft16<N>::R, SUB = Fft16<N>::SUB;
     const bool odd = T.par != 0;
     float2 ca[4], cb[4];
@@ -162,6 +168,10 @@ template <int N, int LINES, class PUT> HQS_DEV void fft16_tail(const float2* s, 
     for (int q = 0; q < 4; ++q) {
         ca[q] = sel(odd, w16(q), make_float2(1.f, 0.f));
         cb[q] = sel(odd, w16(3 * q), w16(2 * q));
+        if (ROT) {
+            ca[q] = sel(odd, make_float2(ca[q].y, -ca[q].x), ca[q]);
+            cb[q] = sel(odd, make_float2(-cb[q].y, cb[q].x), make_float2(-cb[q].x, -cb[q].y));
+        }
     }
 #pragma unroll
     for (int b = 0; b < SUB; ++b) {
@@ -176,7 +186,7 @@ template <int N, int LINES, class PUT> HQS_DEV void fft16_tail(const float2* s, 
         Dft<4, true>::run(f);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            if (q > 0) {
+            if (q > 0 || ROT) {
                 e[q] = cmul(e[q], ca[q]);
                 f[q] = cmul(f[q], cb[q]);
             }
@@ -216,6 +226,58 @@ template <int N> HQS_DEV void fft16_mid_inv(const Lane16& T, const float2* tw, f
         asm volatile("ld.volatile.shared.v2.f32 {%0, %1}, [%2];" : "=f"(w.x), "=f"(w.y) : "r"(base + i * 128));
         v[i] = cmulc(w, v[i]);
     }
+}
+
+// Sums over the LINES lanes of a line group (low lane bits) of CNT values per lane at
+// once, halving the values a lane carries at each exchange while there are several:
+// 15 exchanges for 16 values over 16 lanes against 64 for one butterfly per value; the
+// order of the sum is fixed.  Afterwards lane j holds in w[0 .. PER) the totals of the
+// values j PER + k (PER = CNT / LINES >= 1), or in w[0] that of value j >> SH, shared by
+// 2^SH lanes (CNT < LINES).
+template <int CNT, int LINES> HQS_DEV void lanes_sum(float2* w, int lane) {
+    int c = CNT;
+#pragma unroll
+    for (int bit = LINES / 2; bit > 0; bit >>= 1) {
+        if (c > 1) {
+            c >>= 1;
+            const bool up = (lane & bit) != 0;
+#pragma unroll
+            for (int k = 0; k < CNT / 2; ++k) {
+                if (k >= c) continue;
+                const float2 give = sel(up, w[k], w[k + c]), keep = sel(up, w[k + c], w[k]);
+                w[k] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, give.x, bit),
+                                   keep.y + __shfl_xor_sync(0xffffffffu, give.y, bit));
+            }
+        } else {
+            w[0] = make_float2(w[0].x + __shfl_xor_sync(0xffffffffu, w[0].x, bit),
+                               w[0].y + __shfl_xor_sync(0xffffffffu, w[0].y, bit));
+        }
+    }
+}
+template <int CNT, int LINES, class F> HQS_DEV void lanes_sum_each(float2* w, int lane, F&& f) {
+    lanes_sum<CNT, LINES>(w, lane);
+    if constexpr (CNT >= LINES) {
+        constexpr int PER = CNT / LINES;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) f(lane * PER + k, w[k]);
+    } else {
+        constexpr int REP = LINES / CNT;
+        if ((lane & (REP - 1)) == 0) f(lane / REP, w[0]);
+    }
+}
+
+// Inverse tail of a row of coils (line = coil) with the weighted coil sum fused:
+// put(ix, sum_l conj(S_l[ix]) v_l[ix]) once for each pixel ix < n of the row.  sv: the
+// lane's maps at its 4 SUB outputs (index 4 b + q), zero for lanes without a coil.
+template <int N, int LINES, bool ROT = false, class PUT>
+HQS_DEV void fft16_tail_coilsum(const float2* s, const Lane16& T, const float2* sv, PUT&& put) {
+    constexpr int R = Fft16<N>::R, CNT = 4 * Fft16<N>::SUB;
+    constexpr int C1 = CNT >= 16 ? 16 : CNT, C2 = CNT - C1;   // 16 + 4 at 640, 16 + 8 at 768
+    float2 w[CNT];
+    fft16_tail<N, LINES, ROT>(s, T, [&](int b, int q, int, float2 v) { w[4 * b + q] = cmulc(sv[4 * b + q], v); });
+    auto out = [&](int j, float2 v) { put(T.tp + 8 * (j >> 2) + R * (4 * T.par + (j & 3)), v); };
+    lanes_sum_each<C1, LINES>(w, T.line, out);
+    if constexpr (C2 > 0) lanes_sum_each<C2, LINES>(w + C1, T.line, [&](int j, float2 v) { out(C1 + j, v); });
 }
 
 }  // namespace hqs

@@ -9,7 +9,7 @@
 #include <algorithm>
 #include <cstring>
 
-#include "fft.cuh"
+#include "fft16.cuh"
 #include "plan.cuh"
 
 using namespace hqs;
@@ -103,14 +103,17 @@ __global__ void k_fwd_cols(const float2* __restrict__ U, int n, int L, int LC, i
     }
 }
 
-// ---- passes with the image in the lower half of each line (G = 2n, 16-coil chunks)
+// ---- passes with the image in the lower half of each line (G = 2n)
 // With G = 2n the centred placement p = (i - n/2) mod G of pixel i is the circular
 // shift by n/2 of position q = i, so FFT_G of the centred line is i^k times the FFT of
 // the line holding the image in its lower half [0, n), and the centred output pixels
-// of an inverse transform are the lower half of the inverse of (-i)^k X[k].  The first
-// forward stage then skips the zero half and reads straight from global memory, the
-// last inverse stage skips the discarded half, and stores go straight to global
-// memory (the I/O hooks of block_fft_io, which need every thread to own a line).
+// of an inverse transform are the lower half of the inverse of (-i)^k X[k].  Half of
+// every line is then zero or not wanted, and the two-stage transforms of fft16.cuh
+// apply (the rotations folded into their lane factors), at any coil count: 320^2 x 16
+// coils forward 55.5 -> 51.1 us, adjoint 98.8 -> 85.5; 384^2 x 13 coils, whose passes
+// were the general ones below, adjoint 178 -> 145; 320^2 x 2 coils forward 82 -> 24.  Grids of
+// 32 and 64 points keep the radix-8 stages with the rotations on load and store, for
+// full 16-coil chunks.
 // v * i^k and v * (-i)^k, k >= 0, with selects (k differs from lane to lane: no branches)
 HQS_DEV float2 mul_ipow(float2 v, int k) {
     const bool odd = k & 1, neg = k & 2;
@@ -123,8 +126,8 @@ HQS_DEV float2 mul_mipow(float2 v, int k) {
     return neg ? make_float2(-re, -im) : make_float2(re, im);
 }
 
-// Arguments of the lower-half FFT passes of one plan (G = 2n, chunks of 16 coils),
-// for the single-slice launches and, in a table over slices, the batched ones.
+// Arguments of the lower-half FFT passes of one plan (G = 2n), for the single-slice
+// launches and, in a table over slices, the batched ones.
 struct HalfArgs {
     const float2* x;       // forward: image
     float2* xo;            // adjoint: image (out)
@@ -132,90 +135,111 @@ struct HalfArgs {
     float zc;
     const float2* smaps;   // [n][n][L]
     const float* apod;     // [n]
-    const float2* tw;      // G-point twiddles
+    const float2* tw;      // G-point twiddles, in the order the size's transforms read
     float2* work;          // [n][G][L]
     float2* grid;          // [G][G][L]
     float2* part;          // [nchunk][n][n] coil-chunk sums (nchunk > 1)
-    int n, L, nchunk;
+    int n, L, LC, nchunk;
     float scale;
 };
+template <int G, int LINES> constexpr int half_threads() {
+    return fft16_ok<G>() ? 16 * LINES : FftSize<G>::TPL * kLines;
+}
+template <int G, int LINES> constexpr size_t half_smem() { return ((size_t)G * LINES + G) * sizeof(float2); }
+// the twiddle table, copied with cp.async (the pass waits for it before its first barrier)
+template <int G> HQS_DEV void half_twiddles(float2* dst, const float2* __restrict__ tw) {
+    for (int c = threadIdx.x; c < G / 2; c += blockDim.x) cp_async16(dst + 2 * c, tw + 2 * c);
+}
 
-template <int G> HQS_DEV void fwd_rows_h_item(const HalfArgs& A, int iy, int ch, float2* s) {
-    const float2* tw = stage_twiddles<G>(s + G * kLines, A.tw);
-    const int n = A.n, L = A.L, l0 = ch * kLines;
+// FFT of `lines` lines from ld(line, q) (q < n) to st(line, k)
+template <int G, int LINES, class LD, class ST>
+HQS_DEV void half_forward(float2* s, const float2* twg, int lines, LD&& ld, ST&& st) {
+    float2* tw = s + (size_t)G * LINES;
+    half_twiddles<G>(tw, twg);
+    if constexpr (fft16_ok<G>()) {
+        const Lane16 T(LINES);
+        const bool act = T.line < lines;
+        const int ln = act ? T.line : 0;
+        fft16_head<G, LINES, true>(s, T, [&](int q) { return ld(ln, q); });
+        cp_async_wait_all();
+        __syncthreads();
+        float2 v[Fft16<G>::R];
+        fft16_mid_read<G, LINES>(s, T, v);
+        fft16_mid_fwd<G>(T, tw, v);
+        if (act) {
+#pragma unroll
+            for (int m = 0; m < Fft16<G>::R; ++m) st(ln, T.t + 16 * m, v[m]);
+        }
+    } else {
+        cp_async_wait_all();
+        __syncthreads();
+        block_fft_io<G, false, true, false>(
+            s, lines, tw, [&](int line, int q, bool) { return ld(line, q); }, NoIO{},
+            [&](int line, int k, float2 v) { st(line, k, mul_ipow(v, k)); });
+    }
+}
+
+template <int G, int LINES> HQS_DEV void fwd_rows_h_item(const HalfArgs& A, int iy, int ch, float2* s) {
+    const int n = A.n, L = A.L, l0 = ch * A.LC;
     const float ay = A.apod[iy] * A.scale;
     const float2* xr = A.x + (int64_t)iy * n;
     const float2* sm = A.smaps + (int64_t)iy * n * L + l0;
     const float* apod = A.apod;
     float2* dst = A.work + (int64_t)iy * G * L + l0;
-    __syncthreads();
-    block_fft_io<G, false, true, false>(
-        s, kLines, tw,
-        [&](int line, int q, bool) { return cscale(cmul(__ldg(sm + (int64_t)q * L + line), __ldg(xr + q)), ay * __ldg(apod + q)); },
-        NoIO{}, [&](int line, int k, float2 v) { dst[(int64_t)k * L + line] = mul_ipow(v, k); });
+    half_forward<G, LINES>(
+        s, A.tw, min(A.LC, L - l0),
+        [&](int line, int q) { return cscale(cmul(__ldg(sm + (int64_t)q * L + line), __ldg(xr + q)), ay * __ldg(apod + q)); },
+        [&](int line, int k, float2 v) { dst[(int64_t)k * L + line] = v; });
 }
 
-template <int G> HQS_DEV void fwd_cols_h_item(const HalfArgs& A, int gx, int ch, float2* s) {
-    const float2* tw = stage_twiddles<G>(s + G * kLines, A.tw);
-    const int L = A.L, l0 = ch * kLines;
+template <int G, int LINES> HQS_DEV void fwd_cols_h_item(const HalfArgs& A, int gx, int ch, float2* s) {
+    const int L = A.L, l0 = ch * A.LC;
     const int64_t rs = (int64_t)G * L;
     const float2* col = A.work + (int64_t)gx * L + l0;
     float2* dst = A.grid + (int64_t)gx * L + l0;
-    __syncthreads();
-    block_fft_io<G, false, true, false>(
-        s, kLines, tw, [&](int line, int q, bool) { return __ldg(col + q * rs + line); }, NoIO{},
-        [&](int line, int k, float2 v) { dst[k * rs + line] = mul_ipow(v, k); });
+    half_forward<G, LINES>(
+        s, A.tw, min(A.LC, L - l0), [&](int line, int q) { return __ldg(col + q * rs + line); },
+        [&](int line, int k, float2 v) { dst[k * rs + line] = v; });
 }
 
-template <int G> HQS_DEV void adj_cols_h_item(const HalfArgs& A, int gx, int ch, float2* s) {
-    const float2* tw = stage_twiddles<G>(s + G * kLines, A.tw);
-    const int L = A.L, l0 = ch * kLines;
+template <int G, int LINES> HQS_DEV void adj_cols_h_item(const HalfArgs& A, int gx, int ch, float2* s) {
+    const int L = A.L, l0 = ch * A.LC, lines = min(A.LC, L - l0);
     const int64_t rs = (int64_t)G * L;
     const float2* col = A.grid + (int64_t)gx * L + l0;
     float2* dst = A.work + (int64_t)gx * L + l0;
-    __syncthreads();
-    block_fft_io<G, true, false, true>(
-        s, kLines, tw, [&](int line, int p, bool) { return mul_mipow(__ldg(col + p * rs + line), p); }, NoIO{},
-        [&](int line, int q, float2 v) { dst[q * rs + line] = v; });
+    float2* tw = s + (size_t)G * LINES;
+    half_twiddles<G>(tw, A.tw);
+    if constexpr (fft16_ok<G>()) {
+        const Lane16 T(LINES);
+        const bool act = T.line < lines;
+        const int ln = act ? T.line : 0;
+        float2 v[Fft16<G>::R];
+#pragma unroll
+        for (int m = 0; m < Fft16<G>::R; ++m) v[m] = __ldg(col + (T.t + 16 * m) * rs + ln);
+        cp_async_wait_all();
+        __syncthreads();
+        fft16_mid_inv<G>(T, tw, v);
+        fft16_mid_write<G, LINES>(s, T, v);
+        __syncthreads();
+        fft16_tail<G, LINES, true>(s, T, [&](int, int, int q, float2 w) {
+            if (act) dst[q * rs + ln] = w;
+        });
+    } else {
+        cp_async_wait_all();
+        __syncthreads();
+        block_fft_io<G, true, false, true>(
+            s, lines, tw, [&](int line, int p, bool) { return mul_mipow(__ldg(col + p * rs + line), p); }, NoIO{},
+            [&](int line, int q, float2 v) { dst[q * rs + line] = v; });
+    }
 }
 
-// The row's coil maps go with cp.async to the upper half of the lines buffer once
-// the last stage has read it (that stage keeps the lower half only), so their
-// latency overlaps the stage instead of following the transform.
-template <int G> HQS_DEV void adj_rows_h_item(const HalfArgs& A, int iy, int ch, float2* s) {
-    const float2* tw = stage_twiddles<G>(s + G * kLines, A.tw);
-    const int n = A.n, L = A.L, l0 = ch * kLines;
+template <int G, int LINES> HQS_DEV void adj_rows_h_item(const HalfArgs& A, int iy, int ch, float2* s) {
+    const int n = A.n, L = A.L, l0 = ch * A.LC, lines = min(A.LC, L - l0);
     const float2* src = A.work + (int64_t)iy * G * L + l0;
     const float2* sm = A.smaps + (int64_t)iy * n * L + l0;
-    float2* msm = s + (int64_t)n * kLines;   // upper half: [n][kLines]
-    bool issued = false;
-    __syncthreads();
-    block_fft_io<G, true, false, true>(
-        s, kLines, tw, [&](int line, int p, bool) { return mul_mipow(__ldg(src + (int64_t)p * L + line), p); },
-        [&](int, int, float2 v) {
-            if (!issued) {   // every thread owns a line position (16 lines, blockDim = 16 TPL)
-                issued = true;
-                for (int e = threadIdx.x; e < n * (kLines / 2); e += blockDim.x) {
-                    const int ix = e / (kLines / 2), h = e - ix * (kLines / 2);
-                    cp_async16(msm + ix * kLines + 2 * h, sm + (int64_t)ix * L + 2 * h);
-                }
-            }
-            return v;
-        },
-        NoIO{});
-    cp_async_wait_all();
-    __syncthreads();
     const float ay = A.apod[iy] * A.scale;
-    for (int ix = threadIdx.x; ix < n; ix += blockDim.x) {
-        const float4* s4 = reinterpret_cast<const float4*>(msm + ix * kLines);
-        float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int h = 0; h < kLines / 2; ++h) {
-            const float4 sv = s4[h];
-            const float2 g0 = s[ix * kLines + 2 * h], g1 = s[ix * kLines + 2 * h + 1];
-            a.x += sv.x * g0.x + sv.y * g0.y + sv.z * g1.x + sv.w * g1.y;
-            a.y += sv.x * g0.y - sv.y * g0.x + sv.z * g1.y - sv.w * g1.x;
-        }
+    float2* tw = s + (size_t)G * LINES;
+    auto store = [&](int ix, float2 a) {
         if (A.nchunk == 1) {
             const int64_t e = (int64_t)iy * n + ix;
             float2 v = cscale(a, ay * A.apod[ix]);
@@ -228,24 +252,62 @@ template <int G> HQS_DEV void adj_rows_h_item(const HalfArgs& A, int iy, int ch,
         } else {
             A.part[((int64_t)ch * n + iy) * n + ix] = a;
         }
+    };
+    half_twiddles<G>(tw, A.tw);
+    if constexpr (fft16_ok<G>()) {
+        constexpr int R = Fft16<G>::R, SUB = Fft16<G>::SUB;
+        const Lane16 T(LINES);
+        const bool act = T.line < lines;
+        const int ln = act ? T.line : 0;
+        float2 v[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[m] = __ldg(src + (int64_t)(T.t + 16 * m) * L + ln);
+        cp_async_wait_all();
+        __syncthreads();
+        fft16_mid_inv<G>(T, tw, v);
+        fft16_mid_write<G, LINES>(s, T, v);
+        // the maps of the lane's outputs load while the CTA meets at the barrier
+        float2 sv[4 * SUB];
+#pragma unroll
+        for (int k = 0; k < 4 * SUB; ++k) {
+            const int ix = T.tp + 8 * (k >> 2) + R * (4 * T.par + (k & 3));
+            sv[k] = __ldg(sm + (int64_t)ix * L + ln);
+            if (!act) sv[k] = make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+        fft16_tail_coilsum<G, LINES, true>(s, T, sv, store);
+    } else {
+        cp_async_wait_all();
+        __syncthreads();
+        block_fft_io<G, true, false, true>(
+            s, lines, tw, [&](int line, int p, bool) { return mul_mipow(__ldg(src + (int64_t)p * L + line), p); }, NoIO{},
+            NoIO{});
+        for (int ix = threadIdx.x; ix < n; ix += blockDim.x) {
+            float2 a = make_float2(0.f, 0.f);
+            for (int l = 0; l < lines; ++l) a = cadd(a, cmulc(__ldg(sm + (int64_t)ix * L + l), s[ix * kLines + l]));
+            store(ix, a);
+        }
     }
 }
 
 // single slice: grid (rows or columns, chunks); batched: grid (rows or columns,
 // largest chunk count, slices), the slice's arguments from a device table
-#define HQS_HALF_KERNELS(NAME)                                                            \
-    template <int G> __global__ void k_##NAME(HalfArgs A) {                               \
-        HQS_PDL_ENTRY();                                                                  \
-        extern __shared__ __align__(16) float2 s[];                                       \
-        NAME##_item<G>(A, blockIdx.x, blockIdx.y, s);                                     \
-    }                                                                                     \
-    template <int G> __global__ void k_##NAME##_b(const HalfArgs* __restrict__ tab, float zc) { \
-        HQS_PDL_ENTRY();                                                                  \
-        extern __shared__ __align__(16) float2 s[];                                       \
-        HalfArgs A = tab[blockIdx.z];                                                     \
-        A.zc = zc;                                                                        \
-        if ((int)blockIdx.y >= A.nchunk) return;                                          \
-        NAME##_item<G>(A, blockIdx.x, blockIdx.y, s);                                     \
+#define HQS_HALF_KERNELS(NAME)                                                                                \
+    template <int G, int LINES>                                                                               \
+    __global__ void __launch_bounds__(half_threads<G, LINES>(), 512 / half_threads<G, LINES>()) k_##NAME(HalfArgs A) { \
+        HQS_PDL_ENTRY();                                                                                      \
+        extern __shared__ __align__(16) float2 s[];                                                           \
+        NAME##_item<G, LINES>(A, blockIdx.x, blockIdx.y, s);                                                  \
+    }                                                                                                         \
+    template <int G, int LINES>                                                                               \
+    __global__ void __launch_bounds__(half_threads<G, LINES>(), 512 / half_threads<G, LINES>())               \
+        k_##NAME##_b(const HalfArgs* __restrict__ tab, float zc) {                                            \
+        HQS_PDL_ENTRY();                                                                                      \
+        extern __shared__ __align__(16) float2 s[];                                                           \
+        HalfArgs A = tab[blockIdx.z];                                                                         \
+        A.zc = zc;                                                                                            \
+        if ((int)blockIdx.y >= A.nchunk) return;                                                              \
+        NAME##_item<G, LINES>(A, blockIdx.x, blockIdx.y, s);                                                  \
     }
 HQS_HALF_KERNELS(fwd_rows_h)
 HQS_HALF_KERNELS(fwd_cols_h)
@@ -705,8 +767,21 @@ __global__ void k_adj_chunk_sum(const float2* __restrict__ part, const float* __
 }
 
 // ---------------------------------------------------------------- launchers
-// the lower-half passes apply when G = 2n and every coil chunk has 16 coils
-inline bool half_passes(const hqs_plan_s* p) { return p->G == 2 * p->n && p->LC == kLines && p->L % kLines == 0; }
+// the lower-half passes apply when G = 2n: at any coil count for the sizes of the
+// two-stage transforms, for full 16-coil chunks below (a thread without a line would
+// leave the radix-8 stages' hooks reading line 0)
+inline bool half_passes(const hqs_plan_s* p) {
+    return p->G == 2 * p->n && (p->G >= 128 || (p->LC == kLines && p->L % kLines == 0));
+}
+// lines per CTA of these passes: the smallest of 4, 8, 16 that holds the coil chunk
+inline int half_lines(const hqs_plan_s* p) { return p->G >= 128 && p->LC <= 8 ? (p->LC <= 4 ? 4 : 8) : kLines; }
+template <int G, class F> static int dispatch_half(int lines, F&& f) {
+    if constexpr (fft16_ok<G>()) {
+        if (lines == 4) return f.template operator()<4>();
+        if (lines == 8) return f.template operator()<8>();
+    }
+    return f.template operator()<kLines>();
+}
 
 static HalfArgs half_args(const hqs_plan_s* p, const float2* x, float2* xo, float zc, const float2* z) {
     HalfArgs A;
@@ -716,12 +791,13 @@ static HalfArgs half_args(const hqs_plan_s* p, const float2* x, float2* xo, floa
     A.zc = zc;
     A.smaps = p->smaps;
     A.apod = p->apod;
-    A.tw = plan_twiddles(p, p->G);
+    A.tw = p->G >= 128 ? plan_twiddles16(p, p->G) : plan_twiddles(p, p->G);
     A.work = p->work;
     A.grid = p->grid;
     A.part = p->chunk_buf;
     A.n = p->n;
     A.L = p->L;
+    A.LC = p->LC;
     A.nchunk = p->nchunk;
     A.scale = p->scale;
     return A;
@@ -732,14 +808,19 @@ static int fwd_fft_impl(hqs_plan_s* p, const float2* x, cudaStream_t st) {
     const float2* tw = plan_twiddles(p, G);
     const int th = fft_threads<G>(p->LC);
     const size_t sm = nufft_smem_floats2<G>() * sizeof(float2);
-    if (half_passes(p)) {
-        HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        const HalfArgs A = half_args(p, x, nullptr, 0.f, nullptr);
-        HQS_CUDA_TRY(launch_pdl(k_fwd_rows_h<G>, dim3(p->n, p->nchunk), th, sm, st, A));
-        HQS_CUDA_TRY(launch_pdl(k_fwd_cols_h<G>, dim3(G, p->nchunk), th, sm, st, A));
-        HQS_CUDA_TRY(cudaGetLastError());
-        return HQS_OK;
+    if constexpr (G % 2 == 0 && G != 16 && G != 320 && G != 384) {   // twice a supported image
+        if (half_passes(p))
+            return dispatch_half<G>(half_lines(p), [&]<int LN>() -> int {
+                constexpr int ht = half_threads<G, LN>();
+                constexpr size_t hs = half_smem<G, LN>();
+                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h<G, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
+                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h<G, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
+                const HalfArgs A = half_args(p, x, nullptr, 0.f, nullptr);
+                HQS_CUDA_TRY(launch_pdl(k_fwd_rows_h<G, LN>, dim3(p->n, p->nchunk), ht, hs, st, A));
+                HQS_CUDA_TRY(launch_pdl(k_fwd_cols_h<G, LN>, dim3(G, p->nchunk), ht, hs, st, A));
+                HQS_CUDA_TRY(cudaGetLastError());
+                return HQS_OK;
+            });
     }
     HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
@@ -756,17 +837,21 @@ static int adj_fft_impl(hqs_plan_s* p, float2* x, float zc, const float2* z, cud
     const float2* tw = plan_twiddles(p, G);
     const int th = fft_threads<G>(p->LC);
     const size_t sm = nufft_smem_floats2<G>() * sizeof(float2);
-    if (half_passes(p)) {
-        HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_cols_h<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows_h<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        const HalfArgs A = half_args(p, nullptr, x, zc, z);
-        HQS_CUDA_TRY(launch_pdl(k_adj_cols_h<G>, dim3(G, p->nchunk), th, sm, st, A));
-        HQS_CUDA_TRY(launch_pdl(k_adj_rows_h<G>, dim3(p->n, p->nchunk), th, sm, st, A));
-        if (p->nchunk > 1)
-            HQS_CUDA_TRY(launch_pdl(k_adj_chunk_sum, dim3(std::min(ceil_div(p->n * p->n, 256), 1024)), dim3(256), 0, st,
-                                    p->chunk_buf, p->apod, p->n, p->nchunk, p->scale, x, zc, z));
-        HQS_CUDA_TRY(cudaGetLastError());
-        return HQS_OK;
+    if constexpr (G % 2 == 0 && G != 16 && G != 320 && G != 384) {
+        if (half_passes(p)) {
+            const int rc = dispatch_half<G>(half_lines(p), [&]<int LN>() -> int {
+                constexpr int ht = half_threads<G, LN>();
+                constexpr size_t hs = half_smem<G, LN>();
+                HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_cols_h<G, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
+                HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows_h<G, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
+                const HalfArgs A = half_args(p, nullptr, x, zc, z);
+                HQS_CUDA_TRY(launch_pdl(k_adj_cols_h<G, LN>, dim3(G, p->nchunk), ht, hs, st, A));
+                HQS_CUDA_TRY(launch_pdl(k_adj_rows_h<G, LN>, dim3(p->n, p->nchunk), ht, hs, st, A));
+                return HQS_OK;
+            });
+            if (rc != HQS_OK) return rc;
+            return launch_adj_chunks(p, x, zc, z, st);
+        }
     }
     HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_cols<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
@@ -894,37 +979,35 @@ int launch_adj_axpy(hqs_plan_s* p, const float2* y, float zc, const float2* z, f
 
 // ---- the passes of several plans in one launch per pass (batched operators)
 bool plan_half_passes(const hqs_plan_s* p) { return half_passes(p); }
+int plan_half_lines(const hqs_plan_s* p) { return half_lines(p); }
 size_t half_args_bytes() { return sizeof(HalfArgs); }
 void fill_half_args(const hqs_plan_s* p, const float2* x, float2* xo, const float2* z, void* dst) {
     const HalfArgs A = half_args(p, x, xo, 0.f, z);
     std::memcpy(dst, &A, sizeof(HalfArgs));
 }
 
-// `count` plans with grid G = 2n and 16-coil chunks whose arguments are the
+// `count` plans with grid G = 2n and `lines` lines per CTA whose arguments are the
 // consecutive HalfArgs at d_tab: the forward's row and column passes (adjoint 0)
 // or the adjoint's column and row passes (adjoint 1), grid (lines, chunks, plans)
-int launch_half_group(int G, int n, int maxchunk, int count, const void* d_tab, int adjoint, float zc,
+int launch_half_group(int G, int n, int lines, int maxchunk, int count, const void* d_tab, int adjoint, float zc,
                       cudaStream_t st) {
     return dispatch_fft_size(G, [&]<int GG>() -> int {
-        if constexpr (GG % 2 != 0 || GG < 32) {
+        if constexpr (GG == 16 || GG == 320 || GG == 384) {
             return HQS_ERR_UNSUPPORTED;
         } else {
-            const int th = fft_threads<GG>(kLines);
-            const size_t sm = nufft_smem_floats2<GG>() * sizeof(float2);
-            const HalfArgs* tab = static_cast<const HalfArgs*>(d_tab);
-            if (adjoint) {
-                HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_cols_h_b<GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows_h_b<GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                HQS_CUDA_TRY(launch_pdl(k_adj_cols_h_b<GG>, dim3(GG, maxchunk, count), th, sm, st, tab, zc));
-                HQS_CUDA_TRY(launch_pdl(k_adj_rows_h_b<GG>, dim3(n, maxchunk, count), th, sm, st, tab, zc));
-            } else {
-                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h_b<GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h_b<GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                HQS_CUDA_TRY(launch_pdl(k_fwd_rows_h_b<GG>, dim3(n, maxchunk, count), th, sm, st, tab, zc));
-                HQS_CUDA_TRY(launch_pdl(k_fwd_cols_h_b<GG>, dim3(GG, maxchunk, count), th, sm, st, tab, zc));
-            }
-            HQS_CUDA_TRY(cudaGetLastError());
-            return HQS_OK;
+            return dispatch_half<GG>(lines, [&]<int LN>() -> int {
+                constexpr int th = half_threads<GG, LN>();
+                constexpr size_t sm = half_smem<GG, LN>();
+                const HalfArgs* tab = static_cast<const HalfArgs*>(d_tab);
+                auto first = adjoint ? k_adj_cols_h_b<GG, LN> : k_fwd_rows_h_b<GG, LN>;
+                auto second = adjoint ? k_adj_rows_h_b<GG, LN> : k_fwd_cols_h_b<GG, LN>;
+                HQS_CUDA_TRY(cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                HQS_CUDA_TRY(cudaFuncSetAttribute(second, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                HQS_CUDA_TRY(launch_pdl(first, dim3(adjoint ? GG : n, maxchunk, count), th, sm, st, tab, zc));
+                HQS_CUDA_TRY(launch_pdl(second, dim3(adjoint ? n : GG, maxchunk, count), th, sm, st, tab, zc));
+                HQS_CUDA_TRY(cudaGetLastError());
+                return HQS_OK;
+            });
         }
     });
 }

@@ -124,11 +124,12 @@ int launch_fwd(hqs_plan_s* p, const float2* x, float2* y, cudaStream_t s);
 int launch_adj(hqs_plan_s* p, const float2* y, float2* x, cudaStream_t s);
 int launch_adj_axpy(hqs_plan_s* p, const float2* y, float zc, const float2* z, float2* x, cudaStream_t s);
 // batched operators (csrc/nufft.cu): per-plan pieces and the lower-half passes of
-// a group of plans (G = 2n, 16-coil chunks) in one launch per pass
+// a group of plans (one grid size G = 2n and lines per CTA) in one launch per pass
 bool plan_half_passes(const hqs_plan_s* p);
+int plan_half_lines(const hqs_plan_s* p);
 size_t half_args_bytes();
 void fill_half_args(const hqs_plan_s* p, const float2* x, float2* xo, const float2* z, void* dst);
-int launch_half_group(int G, int n, int maxchunk, int count, const void* d_tab, int adjoint, float zc,
+int launch_half_group(int G, int n, int lines, int maxchunk, int count, const void* d_tab, int adjoint, float zc,
                       cudaStream_t s);
 int launch_spread(hqs_plan_s* p, const float2* y, cudaStream_t s);
 int launch_interp(hqs_plan_s* p, float2* y, cudaStream_t s);

@@ -180,58 +180,6 @@ HQS_DEV float2 toep_epilogue(float2 v, int64_t e, const float2* __restrict__ pve
     return v;
 }
 
-// Sums over the LINES lanes of a line group (low lane bits) of CNT values per lane at
-// once, halving the values a lane carries at each exchange while there are several:
-// 15 exchanges for 16 values over 16 lanes against 64 for one butterfly per value; the
-// order of the sum is fixed.  Afterwards lane j holds in w[0 .. PER) the totals of the
-// values j PER + k (PER = CNT / LINES >= 1), or in w[0] that of value j >> SH, shared by
-// 2^SH lanes (CNT < LINES).
-template <int CNT, int LINES> HQS_DEV void lanes_sum(float2* w, int lane) {
-    int c = CNT;
-#pragma unroll
-    for (int bit = LINES / 2; bit > 0; bit >>= 1) {
-        if (c > 1) {
-            c >>= 1;
-            const bool up = (lane & bit) != 0;
-#pragma unroll
-            for (int k = 0; k < CNT / 2; ++k) {
-                if (k >= c) continue;
-                const float2 give = sel(up, w[k], w[k + c]), keep = sel(up, w[k + c], w[k]);
-                w[k] = make_float2(keep.x + __shfl_xor_sync(0xffffffffu, give.x, bit),
-                                   keep.y + __shfl_xor_sync(0xffffffffu, give.y, bit));
-            }
-        } else {
-            w[0] = make_float2(w[0].x + __shfl_xor_sync(0xffffffffu, w[0].x, bit),
-                               w[0].y + __shfl_xor_sync(0xffffffffu, w[0].y, bit));
-        }
-    }
-}
-template <int CNT, int LINES, class F> HQS_DEV void lanes_sum_each(float2* w, int lane, F&& f) {
-    lanes_sum<CNT, LINES>(w, lane);
-    if constexpr (CNT >= LINES) {
-        constexpr int PER = CNT / LINES;
-#pragma unroll
-        for (int k = 0; k < PER; ++k) f(lane * PER + k, w[k]);
-    } else {
-        constexpr int REP = LINES / CNT;
-        if ((lane & (REP - 1)) == 0) f(lane / REP, w[0]);
-    }
-}
-
-// Inverse tail of a row of coils (line = coil) with the weighted coil sum fused:
-// put(ix, sum_l conj(S_l[ix]) v_l[ix]) once for each pixel ix < n of the row.  sv: the
-// lane's maps at its 4 SUB outputs (index 4 b + q), zero for lanes without a coil.
-template <int N, int LINES, class PUT>
-HQS_DEV void fft16_tail_coilsum(const float2* s, const Lane16& T, const float2* sv, PUT&& put) {
-    constexpr int R = Fft16<N>::R, CNT = 4 * Fft16<N>::SUB;
-    constexpr int C1 = CNT >= 16 ? 16 : CNT, C2 = CNT - C1;   // 16 + 4 at 640, 16 + 8 at 768
-    float2 w[CNT];
-    fft16_tail<N, LINES>(s, T, [&](int b, int q, int, float2 v) { w[4 * b + q] = cmulc(sv[4 * b + q], v); });
-    auto out = [&](int j, float2 v) { put(T.tp + 8 * (j >> 2) + R * (4 * T.par + (j & 3)), v); };
-    lanes_sum_each<C1, LINES>(w, T.line, out);
-    if constexpr (C2 > 0) lanes_sum_each<C2, LINES>(w + C1, T.line, [&](int j, float2 v) { out(C1 + j, v); });
-}
-
 // P3: row iy: IFFT along x, keep n, sum_l conj(S_l) . over the chunk's coils.
 // One chunk: epilogue and store here (returns the thread's partial); several
 // chunks: the raw chunk sum goes to A.chunk[ch] for k_toep_chunk_epilogue.
