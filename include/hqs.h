@@ -81,8 +81,8 @@ typedef struct {
     int64_t npoints;          /* M */
     double  kb_beta;          /* Kaiser-Bessel shape parameter */
     size_t  device_bytes;     /* device memory held by the plan */
-    int     nsub;             /* spreading work items (tile-owned spreading) */
-    int     tile;             /* spreading tile edge on the grid */
+    int     nsub;             /* CTAs of the tile-owned spreading */
+    int     tile;             /* edge of the bins the points are sorted in */
 } hqs_plan_info;
 
 typedef struct {
@@ -133,7 +133,7 @@ HQS_API int hqs_forward(hqs_plan plan, const hqs_c64* x, hqs_c64* y, void* strea
 
 /* --------------------------------------------------------- adjoint (a3) */
 /* x = A^H y (Sec. 3.4 uses A^H), the exact transpose of hqs_forward:
- * KB spreading (each grid tile accumulated in shared memory by the CTAs
+ * KB spreading (each grid tile accumulated in registers by the warps
  * that own it and written once: no atomics, a fixed summation order, so the
  * result is bitwise repeatable), inverse FFT, deapodisation, coil
  * combination with conj(S_l).  y: (L, M); x: (ny, nx). */
@@ -410,7 +410,7 @@ HQS_API const char* hqs_status_string(int status);
 /* Tuning knobs (no counterpart in the paper), set per plan by the autotuner:
  *   HQS_TUNE_FUSED_GRID  cap on the persistent solve's CTAs (0 = all resident)
  *   HQS_TUNE_PC_LINES    preconditioner rows/columns per work item (1..16)
- *   HQS_TUNE_SPREAD_TILE spreading tile edge (8, 16 or 32): re-bins the
+ *   HQS_TUNE_SPREAD_TILE edge of the point bins (8, 16 or 32): re-bins the
  *                        plan's points (hqs_plan_retile on the default stream)
  * and one test hook for the failure path of the persistent solve:
  *   HQS_TUNE_DEBUG_BARRIER_SKIP  1 arms it for the next HQS_SOLVE_FUSED solve
@@ -425,7 +425,7 @@ HQS_API const char* hqs_status_string(int status);
 #define HQS_TUNE_SPREAD_TILE  3
 #define HQS_TUNE_DEBUG_BARRIER_SKIP 4
 HQS_API int hqs_plan_set_tuning(hqs_plan plan, int key, int value);
-/* Re-sorts the plan's points into tile x tile spreading bins (8, 16, 32);
+/* Re-sorts the plan's points into tile x tile bins (8, 16, 32);
  * BLOCKING on `stream`.  The result of hqs_adjoint does not depend on the tile
  * beyond float rounding order. */
 HQS_API int hqs_plan_retile(hqs_plan plan, int tile, void* stream);

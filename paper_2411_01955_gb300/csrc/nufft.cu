@@ -315,361 +315,287 @@ HQS_HALF_KERNELS(adj_cols_h)
 HQS_HALF_KERNELS(adj_rows_h)
 #undef HQS_HALF_KERNELS
 
-template <int W>
+// Type-2 interpolation: LPP lanes per sorted point, lane q owning VEC coils of a chunk
+// (two as one 16-byte load where the coil count is even), the weights from the plan's
+// table, the results straight to the caller's (coil, point) order (a sorted copy and a
+// kernel to put it in order cost 8 us more).  Bound: latency of the L2 and L1 gathers of
+// W^2 grid values of a point's coils, so the registers go to loads in flight (3 CTAs per
+// SM with 85 registers: a 320^2 x 16-coil forward at W 6 55 us; with 128 registers 48).
+template <int VEC> struct Coils;
+template <> struct Coils<2> {
+    float2 a, b;
+    HQS_DEV void zero() { a = b = make_float2(0.f, 0.f); }
+    HQS_DEV void fma_load(const float2* p, float w) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+        a = cfma_r(make_float2(v.x, v.y), w, a);
+        b = cfma_r(make_float2(v.z, v.w), w, b);
+    }
+    HQS_DEV void fma(const Coils& v, float w) {
+        a = cfma_r(v.a, w, a);
+        b = cfma_r(v.b, w, b);
+    }
+    HQS_DEV void put(float2* y, int64_t M) const {
+        y[0] = a;
+        y[M] = b;
+    }
+};
+template <> struct Coils<1> {
+    float2 a;
+    HQS_DEV void zero() { a = make_float2(0.f, 0.f); }
+    HQS_DEV void fma_load(const float2* p, float w) { a = cfma_r(__ldg(p), w, a); }
+    HQS_DEV void fma(const Coils& v, float w) { a = cfma_r(v.a, w, a); }
+    HQS_DEV void put(float2* y, int64_t) const { y[0] = a; }
+};
+template <int W, int VEC, int LPP>
 __global__ void __launch_bounds__(256) k_interp(const float2* __restrict__ Gh, const int4* __restrict__ pts,
-                                                const int* __restrict__ perm, int M, int G, int L,
-                                                float beta, float2* __restrict__ y) {
+                                                const float* __restrict__ kbw, const int* __restrict__ perm, int M,
+                                                int G, int L, float2* __restrict__ y) {
     HQS_PDL_ENTRY();
-    const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4);
-    const int h = threadIdx.x & 15;
-    const int base = threadIdx.x & 16;
-    const bool valid = j < M;
-    const int4 pt = valid ? pts[j] : make_int4(0, 0, 0, 0);
-    const float dx = __int_as_float(pt.z), dy = __int_as_float(pt.w);
-    float wm = 0.f;
-    if (valid && h < 2 * W) wm = kb_phi(h < W ? dx - (float)h : dy - (float)(h - W), (float)W, beta);
-    float wx[W], wy[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        wx[w] = __shfl_sync(0xffffffffu, wm, base + w);
-        wy[w] = __shfl_sync(0xffffffffu, wm, base + W + w);
-    }
-    if (!valid) return;
-    int gxs[W];
-#pragma unroll
-    for (int b = 0; b < W; ++b) {
-        int gx = pt.x + b;
-        gxs[b] = gx >= G ? gx - G : gx;
-    }
-    const int dst = perm[j];
-    for (int l = h; l < L; l += 16) {
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            int gy = pt.y + a;
-            if (gy >= G) gy -= G;
-            const float2* row = Gh + (int64_t)gy * G * L + l;
-            float2 ra = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int b = 0; b < W; ++b) {
-                const float2 g = __ldg(row + (int64_t)gxs[b] * L);
-                ra.x = fmaf(wx[b], g.x, ra.x);
-                ra.y = fmaf(wx[b], g.y, ra.y);
-            }
-            acc.x = fmaf(wy[a], ra.x, acc.x);
-            acc.y = fmaf(wy[a], ra.y, acc.y);
-        }
-        y[(int64_t)l * M + dst] = acc;
-    }
-}
-
-// Type-2 interpolation for 16-coil chunks: 8 lanes per point, lane q owning coils
-// (2q, 2q+1) of a chunk, so one float4 load per lane reads a tap's 16 coils as one
-// 128-byte line; the 2W weights come from the plan's table; the result goes to the
-// sorted order, coil-innermost (one 128-byte store per point and chunk), and
-// k_y_from_sorted puts it in the caller's (coil, point) order.
-template <int W>
-__global__ void __launch_bounds__(256) k_interp16(const float2* __restrict__ Gh, const int4* __restrict__ pts,
-                                                  const float* __restrict__ kbw, int M, int G, int L,
-                                                  float2* __restrict__ ys) {
-    HQS_PDL_ENTRY();
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t j = t >> 3;
-    const int q = threadIdx.x & 7;
+    const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LPP;
+    const int q = threadIdx.x % LPP;
     if (j >= M) return;
     const int4 pt = pts[j];
-    float wx[W], wy[W];
+    const int dst = perm[j];
+    float wx[8], wy[8];
+    const float4* kw = reinterpret_cast<const float4*>(kbw + j * 24);
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
-        wx[w] = __ldg(kbw + j * 2 * W + w);
-        wy[w] = __ldg(kbw + j * 2 * W + W + w);
+    for (int h = 0; h < (W + 3) / 4; ++h) {
+        const float4 v = __ldg(kw + h);
+        wx[4 * h] = v.x, wx[4 * h + 1] = v.y, wx[4 * h + 2] = v.z, wx[4 * h + 3] = v.w;
+    }
+#pragma unroll
+    for (int h = 0; h < (W + 1) / 2; ++h) {
+        const float4 v = __ldg(kw + 2 + h);
+        wy[2 * h] = v.x, wy[2 * h + 1] = v.z;
     }
     int gxs[W];
 #pragma unroll
     for (int b = 0; b < W; ++b) {
         const int gx = pt.x + b;
-        gxs[b] = gx >= G ? gx - G : gx;
+        gxs[b] = (gx >= G ? gx - G : gx) * L;
     }
-    for (int l0 = 0; l0 < L; l0 += 16) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int l = q * VEC; l < L; l += LPP * VEC) {
+        Coils<VEC> acc;
+        acc.zero();
 #pragma unroll
         for (int a = 0; a < W; ++a) {
             int gy = pt.y + a;
             if (gy >= G) gy -= G;
-            const float4* row = reinterpret_cast<const float4*>(Gh + (int64_t)gy * G * L + l0) + q;
-            float4 ra = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float2* row = Gh + (int64_t)gy * G * L + l;
+            Coils<VEC> ra;
+            ra.zero();
 #pragma unroll
-            for (int b = 0; b < W; ++b) {
-                const float4 g = __ldg(row + (int64_t)gxs[b] * (L / 2));
-                ra.x = fmaf(wx[b], g.x, ra.x);
-                ra.y = fmaf(wx[b], g.y, ra.y);
-                ra.z = fmaf(wx[b], g.z, ra.z);
-                ra.w = fmaf(wx[b], g.w, ra.w);
-            }
-            acc.x = fmaf(wy[a], ra.x, acc.x);
-            acc.y = fmaf(wy[a], ra.y, acc.y);
-            acc.z = fmaf(wy[a], ra.z, acc.z);
-            acc.w = fmaf(wy[a], ra.w, acc.w);
+            for (int b = 0; b < W; ++b) ra.fma_load(row + gxs[b], wx[b]);
+            acc.fma(ra, wy[a]);
         }
-        reinterpret_cast<float4*>(ys + j * L + l0)[q] = acc;
+        acc.put(y + (int64_t)l * M + dst, M);
     }
 }
 
 // ---------------------------------------------------------------- adjoint
-// k-space data to the sorted point order, coil-innermost: ys[invperm[m]][l] =
-// y[l][m].  A CTA stages kSortPts caller-order points of every coil (coalesced
-// rows of y) in shared memory and writes each point's L-coil line contiguously.
-constexpr int kSortPts = 64;
-__global__ void __launch_bounds__(256) k_y_to_sorted(const float2* __restrict__ y, const int* __restrict__ invperm,
-                                                     int M, int L, float2* __restrict__ ys) {
-    HQS_PDL_ENTRY();
-    extern __shared__ float2 sy[];   // [kSortPts][L + 1]
-    const int m0 = blockIdx.x * kSortPts;
-    const int np = min(kSortPts, M - m0);
-    for (int e = threadIdx.x; e < L * kSortPts; e += blockDim.x) {
-        const int l = e / kSortPts, q = e - l * kSortPts;
-        if (q < np) sy[q * (L + 1) + l] = y[(int64_t)l * M + m0 + q];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < np * L; e += blockDim.x) {
-        const int q = e / L, l = e - q * L;
-        ys[(int64_t)invperm[m0 + q] * L + l] = sy[q * (L + 1) + l];
+// Tile-owned type-1 spreading: each 8 x 8 tile of the grid is written once, with plain
+// stores, by the warps that own it (no atomics on data, no memset, a fixed order of the
+// sums).  The plan lists the points that touch each tile (2.7 tiles a point at W 6) with
+// the offset of their first tap.  Lane (x, coil group) keeps the 8 rows of its cell
+// column for CPL coils in registers, so a point costs its value times the lane's x
+// weight once, then one packed multiply-add per exact y tap and coil, the rows selected
+// by a switch on the point's y offset (registers need static names).  The weights and
+// k-space values of 16 points at a time go to the warp's own shared memory with
+// cp.async while the 16 before are added: a warp needs no barrier.
+// A tile of at most HQS_SPREAD_LIGHT points belongs to one warp, eight such tiles to a
+// CTA; a heavier one to whole CTAs of up to 8 HQS_SPREAD_LIGHT points each, whose warps' tiles are summed through shared
+// memory, and, where there are several CTAs, through partial tiles in slot order by the
+// last to arrive.
+// Bound: latency of a point's shared-memory reads and switch, and of the list, weight and
+// value reads per tile.  320^2 x 16 coils, 32,768 spiral points: a whole adjoint 85.5 ->
+// 62.1 us (384^2 x 13 coils, 56,064 radial points: 145 -> 94.8) against CTAs that scanned
+// the neighbouring bins' points; light tiles of up to 32, 64, 128, 256 points: 64.7, 62.1,
+// 75.0, 103.5 us; without reading the next point ahead 66.1.
+constexpr int kTile = 8;
+constexpr int kSpreadBatch = 16;
+template <int CPL> constexpr int spread_slot() { return 96 + 4 * CPL * (int)sizeof(float2); }
+template <int CPL> constexpr size_t spread_smem() {
+    // point slots of 8 warps, or their 8 tiles while a heavy tile is summed
+    constexpr size_t a = (size_t)8 * 2 * kSpreadBatch * spread_slot<CPL>();
+    constexpr size_t b = (size_t)8 * kTile * kTile * 4 * CPL * sizeof(float2);
+    return a > b ? a : b;
+}
+template <int W, int CPL, int OY>
+HQS_DEV void spread_rows(float2 (&acc)[kTile][CPL], const char* sp, const float2* u) {
+    const float4* wy = reinterpret_cast<const float4*>(sp + 32);
+#pragma unroll
+    for (int b = 0; b < W; ++b) {
+        if (OY + b < 0 || OY + b >= kTile) continue;
+        const float4 w4 = wy[b >> 1];
+        const float2 w = (b & 1) ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) acc[(OY + b) & (kTile - 1)][c] = cfma2(u[c], w, acc[(OY + b) & (kTile - 1)][c]);
     }
 }
-
-// The reverse copy for the forward operator: y[l][m] = ys[invperm[m]][l], each
-// point's L-coil line read contiguously, each coil's kSortPts points written as one run.
-__global__ void __launch_bounds__(256) k_y_from_sorted(const float2* __restrict__ ys, const int* __restrict__ invperm,
-                                                       int M, int L, float2* __restrict__ y) {
-    HQS_PDL_ENTRY();
-    extern __shared__ float2 sy[];   // [kSortPts][L + 1]
-    const int m0 = blockIdx.x * kSortPts;
-    const int np = min(kSortPts, M - m0);
-    for (int e = threadIdx.x; e < np * L; e += blockDim.x) {
-        const int q = e / L, l = e - q * L;
-        sy[q * (L + 1) + l] = ys[(int64_t)invperm[m0 + q] * L + l];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < L * kSortPts; e += blockDim.x) {
-        const int l = e / kSortPts, q = e - l * kSortPts;
-        if (q < np) y[(int64_t)l * M + m0 + q] = sy[q * (L + 1) + l];
+// CPL values of a lane to d: pairs as 16-byte stores, or the first n singly
+template <int CPL> HQS_DEV void put_coils(float2* d, const float2* v, int n, bool pairs) {
+    if (CPL >= 2 && pairs && n >= CPL) {
+#pragma unroll
+        for (int c = 0; c + 1 < CPL; c += 2)
+            reinterpret_cast<float4*>(d)[c / 2] = make_float4(v[c].x, v[c].y, v[c + 1].x, v[c + 1].y);
+    } else {
+#pragma unroll
+        for (int c = 0; c < CPL; ++c)
+            if (c < n) d[c] = v[c];
     }
 }
-
-// Tile-owned type-1 spreading.  One CTA per item of a TT x TT tile of the
-// grid: the item's candidates (points [c0, c1) of the tile's 3 x 3
-// neighbouring bins, taken in a fixed order; a point's W taps reach at most
-// one bin to either side because TT >= W/2) that touch the tile are staged in
-// shared memory, in candidate order, with their plan-time Kaiser-Bessel
-// weights, their first tap relative to the tile and their k-space values.
-// Warp w owns the tile rows w (mod 8); for one row and a chunk of LCS coils a
-// lane owns the (cell, coil) pairs p = lane + 32 k of the row and keeps their
-// sums in registers while it walks the staged points in order, so no two
-// threads ever update one cell and every cell is summed in the same order.
-// The row is then written once with plain stores: to the grid when the tile
-// has one item, else to the item's partial slot, and the last of the tile's
-// items to arrive sums the slots in slot order into the grid.  No atomics on
-// data and no memset of the grid.
-constexpr int kSpreadWarps = 8;
-// FULL16: every coil chunk has exactly 16 coils (L a multiple of 16).  Then lane
-// (h, l) = (lane / 16, lane % 16) owns coil l of the cells x = h + 2 k of a row,
-// and each staged point's x weights over the tile row are tabulated once
-// (wrow[i][h][k], zero outside the footprint), so a cell update is one
-// multiply-add pair on registers.
-template <int W, int TT, bool FULL16>
-__global__ void __launch_bounds__(256) k_spread_tiles(const float2* __restrict__ ys, const int4* __restrict__ pts,
-                                                      const float* __restrict__ kbw, const int2* __restrict__ tile_nb,
-                                                      const int4* __restrict__ items, const int2* __restrict__ tinfo,
-                                                      unsigned* __restrict__ tickets, float2* __restrict__ partial,
-                                                      int G, int L, int LCS, int nbx, float2* __restrict__ grid) {
+template <int W, int CPL>
+__global__ void __launch_bounds__(256, 2)
+    k_spread(const float2* __restrict__ y, const float* __restrict__ kbw, const int4* __restrict__ list,
+             const int4* __restrict__ ctas, const int4* __restrict__ light, const int2* __restrict__ tinfo,
+             unsigned* __restrict__ tickets, float2* __restrict__ partial, int64_t M, int nbx, int G, int L,
+             float2* __restrict__ grid) {
     HQS_PDL_ENTRY();
-    constexpr int CAND = HQS_SPREAD_CAND;
-    constexpr int NK = (TT * 16 + 31) / 32;   // (cell, coil) pairs of a row per lane, LCS <= 16
+    constexpr int T = kTile, CL = 4 * CPL, SLOT = spread_slot<CPL>(), NB = kSpreadBatch;
+    static_assert(T == 8 && W <= 8 && NB == 16, "one point per half-warp of copies, eight steps a batch");
     extern __shared__ float4 smem4[];
-    float2* sval = reinterpret_cast<float2*>(smem4);              // [CAND][LCS]
-    float* swt = reinterpret_cast<float*>(sval + CAND * LCS);      // [CAND][2W]
-    int2* soff = reinterpret_cast<int2*>(swt + CAND * 2 * W);      // [CAND]: first tap - tile origin (x, y)
-    int* sidx = reinterpret_cast<int*>(soff + CAND);               // [CAND]: sorted point index
-    float* wrow = reinterpret_cast<float*>(sidx + CAND);           // FULL16: [CAND][2][TT / 2]
-    __shared__ int2 nbs[10];
-    __shared__ int npts, wcount[kSpreadWarps], last;
-    const int4 it = items[blockIdx.x];
-    const int t = it.x, tx = t % nbx, ty = t / nbx;
-    const int x0 = tx * TT, y0 = ty * TT;
+    __shared__ int last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // the tile's distinct neighbouring bins from the plan: (first point, candidate
-    // prefix) in candidate order, entry 9 = (bins, candidates)
-    if (threadIdx.x < 10) nbs[threadIdx.x] = tile_nb[(int64_t)t * 10 + threadIdx.x];
+    const int xl = lane & 7, cq = lane >> 3;
+    const int l0 = blockIdx.y * CL, lc = min(CL, L - l0);
+    // (tile, first entry, end entry, partial slot or -1), or (-1, first light tile, end, -)
+    const int4 it = ctas[blockIdx.x];
+    const bool heavy = it.x >= 0;
+    int tile = it.x, e0 = 0, e1 = 0;
+    if (heavy) {   // this warp's eighth of the entries
+        const int n = it.z - it.y;
+        e0 = it.y + n * warp / 8;
+        e1 = it.y + n * (warp + 1) / 8;
+    } else if (it.y + warp < it.z) {
+        const int4 t = light[it.y + warp];
+        tile = t.x;
+        e0 = t.y;
+        e1 = t.z;
+    }
+    char* sw = reinterpret_cast<char*>(smem4) + (size_t)warp * 2 * NB * SLOT;
+    float2 acc[T][CPL];
+#pragma unroll
+    for (int r = 0; r < T; ++r)
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) acc[r][c] = make_float2(0.f, 0.f);
+    auto entry = [&](int e) { return lane < NB && e + lane < e1 ? __ldg(list + e + lane) : make_int4(0, 0, 0, 0); };
+    auto copy = [&](const int4& ent, int n, int buf) {
+        const int q = lane & 15;
+#pragma unroll
+        for (int s = 0; s < NB / 2; ++s) {
+            const int i = 2 * s + (lane >> 4);
+            const int j = __shfl_sync(0xffffffffu, ent.x, i), m = __shfl_sync(0xffffffffu, ent.y, i);
+            if (i >= n) continue;
+            char* d = sw + (buf * NB + i) * SLOT;
+            if (q < 6) cp_async16(d + 16 * q, kbw + (int64_t)j * 24 + 4 * q);
+            if (q < lc) cp_async8(d + 96 + 8 * q, y + (int64_t)(l0 + q) * M + m);
+        }
+        cp_async_commit();
+    };
+    int4 cur = entry(e0), nxt = entry(e0 + NB);
+    copy(cur, e1 - e0, 0);
+    for (int e = e0, buf = 0; e < e1; e += NB, buf ^= 1) {
+        const int4 nn = entry(e + 2 * NB);
+        copy(nxt, e1 - e - NB, buf ^ 1);   // empty after the last batch
+        cp_async_wait_group<1>();
+        __syncwarp();
+        const int n = min(NB, e1 - e);
+        // the next point's offset, x weight and values are read while this one is added
+        const int vl = 96 + cq * CPL * (int)sizeof(float2);
+        const char* sp = sw + buf * NB * SLOT;
+        int off = __shfl_sync(0xffffffffu, cur.z, 0);
+        float wx;
+        float2 v[CPL];
+        auto fetch = [&](const char* p) {
+            const int bx = xl - ((off & 255) - 16);
+            const bool in = (unsigned)bx < (unsigned)W;
+            wx = *reinterpret_cast<const float*>(p + (in ? 4 * bx : 0));
+            wx = in ? wx : 0.f;
+            if constexpr (CPL == 4) {
+                const float4 v0 = *reinterpret_cast<const float4*>(p + vl), v1 = *reinterpret_cast<const float4*>(p + vl + 16);
+                v[0] = make_float2(v0.x, v0.y), v[1] = make_float2(v0.z, v0.w);
+                v[2] = make_float2(v1.x, v1.y), v[3] = make_float2(v1.z, v1.w);
+            } else {
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) v[c] = reinterpret_cast<const float2*>(p + vl)[c];
+            }
+        };
+        fetch(sp);
+        for (int i = 0; i < n; ++i, sp += SLOT) {
+            const int oy = (off >> 8) - 16;
+            float2 u[CPL];
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) u[c] = cmul_r(v[c], wx);
+            if (i + 1 < n) {
+                off = __shfl_sync(0xffffffffu, cur.z, i + 1);
+                fetch(sp + SLOT);
+            }
+            switch (oy) {
+#define HQS_ROWS(OY)                                                 \
+    case OY:                                                         \
+        if constexpr (OY > -W) spread_rows<W, CPL, OY>(acc, sp, u);  \
+        break;
+                HQS_ROWS(-7) HQS_ROWS(-6) HQS_ROWS(-5) HQS_ROWS(-4) HQS_ROWS(-3)
+                HQS_ROWS(-2) HQS_ROWS(-1) HQS_ROWS(0) HQS_ROWS(1) HQS_ROWS(2)
+                HQS_ROWS(3) HQS_ROWS(4) HQS_ROWS(5) HQS_ROWS(6) HQS_ROWS(7)
+#undef HQS_ROWS
+            }
+        }
+        __syncwarp();
+        cur = nxt;
+        nxt = nn;
+    }
+    cp_async_wait_all();
+    const int ncoil = lc - cq * CPL;   // coils of this lane that exist (may be <= 0)
+    const bool pairs = L % 2 == 0;
+    const int64_t grow = (int64_t)G * L;
+    auto cell = [&](int r) {
+        return grid + ((int64_t)((tile / nbx) * T + r) * G + (tile % nbx) * T + xl) * L + l0 + cq * CPL;
+    };
+    if (!heavy) {
+        if (tile < 0) return;
+        float2* g = cell(0);
+#pragma unroll
+        for (int r = 0; r < T; ++r) put_coils<CPL>(g + r * grow, acc[r], ncoil, pairs);
+        return;
+    }
+    // the CTA's sum: every warp's tile to shared memory, then warp w adds row w in warp order
     __syncthreads();
-    // stage the candidates that touch the tile, in candidate order (CAND == blockDim)
-    {
-        const int c = it.y + threadIdx.x;
-        bool ov = false;
-        int j = 0, ox = 0, oy = 0;
-        if (c < it.z) {
-            const int nnb = nbs[9].x;
-            int k = 0;
-            while (k + 1 < nnb && nbs[k + 1].y <= c) ++k;
-            j = nbs[k].x + (c - nbs[k].y);
-            const int4 pt = pts[j];
-            // first tap relative to the tile, on the periodic grid: in [0, TT) when the
-            // taps start inside the tile, in [-(W-1), 0) when they start left of it
-            ox = pt.x - x0;
-            oy = pt.y - y0;
-            if (ox < 0) ox += G;
-            if (oy < 0) oy += G;
-            if (ox >= TT) ox -= G;
-            if (oy >= TT) oy -= G;
-            ov = ox > -W && oy > -W;
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, ov);
-        if (lane == 0) wcount[warp] = __popc(bal);
-        __syncthreads();
-        int base = 0;
-        for (int w = 0; w < warp; ++w) base += wcount[w];
-        if (threadIdx.x == 0) {
-            int tot = 0;
-            for (int w = 0; w < kSpreadWarps; ++w) tot += wcount[w];
-            npts = tot;
-        }
-        if (ov) {
-            const int pos = base + __popc(bal & ((1u << lane) - 1u));
-            soff[pos] = make_int2(ox, oy);
-            sidx[pos] = j;
-        }
-        __syncthreads();
+    // (element c of a lane at [warp][row][c][lane], so a warp's accesses are contiguous)
+    float2* st = reinterpret_cast<float2*>(smem4);
+#pragma unroll
+    for (int r = 0; r < T; ++r)
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) st[((warp * T + r) * CPL + c) * 32 + lane] = acc[r][c];
+    __syncthreads();
+    float2 sum[CPL];
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) sum[c] = make_float2(0.f, 0.f);
+    for (int w = 0; w < 8; ++w)
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) sum[c] = cadd(sum[c], st[((w * T + warp) * CPL + c) * 32 + lane]);
+    if (it.w < 0) {
+        put_coils<CPL>(cell(warp), sum, ncoil, pairs);
+        return;
     }
-    const int np = npts;
-    for (int e = threadIdx.x; e < np * 2 * W; e += blockDim.x) {
-        const int i = e / (2 * W), h = e - i * (2 * W);
-        swt[e] = __ldg(kbw + (int64_t)sidx[i] * 2 * W + h);
-    }
-    if constexpr (FULL16) {
-        // the first chunk's values load together with the weights (one latency round)
-        for (int e = threadIdx.x; e < np * 16; e += blockDim.x) {
-            const int i = e >> 4, ll = e & 15;
-            sval[i * 16 + ll] = __ldg(ys + (int64_t)sidx[i] * L + ll);
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < np * TT; e += blockDim.x) {
-            const int i = e / TT, x = e - i * TT;
-            int b = x - soff[i].x;
-            b += b < 0 ? G : 0;
-            wrow[i * TT + (x & 1) * (TT / 2) + (x >> 1)] = (unsigned)b < (unsigned)W ? swt[i * 2 * W + b] : 0.f;
-        }
-        const int h = lane >> 4, l = lane & 15;
-        for (int l0 = 0; l0 < L; l0 += 16) {
-            if (l0 > 0) {   // later 16-coil chunks
-                for (int e = threadIdx.x; e < np * 16; e += blockDim.x) {
-                    const int i = e >> 4, ll = e & 15;
-                    sval[i * 16 + ll] = __ldg(ys + (int64_t)sidx[i] * L + l0 + ll);
-                }
-            }
-            __syncthreads();
-            float2* dst = it.w < 0 ? grid : partial + (int64_t)it.w * TT * TT * L;
-            for (int r = warp; r < TT; r += kSpreadWarps) {
-                float2 acc[TT / 2];
+    const int64_t slot = (int64_t)gridDim.y * T * T * CL;
+    float2* pc = partial + ((int64_t)blockIdx.y * T * T + warp * T + xl) * CL + cq * CPL;
+    put_coils<CPL>(pc + it.w * slot, sum, CPL, true);
+    __threadfence();
+    __syncthreads();
+    const int2 ti = tinfo[tile];
+    unsigned* ticket = tickets + (int64_t)tile * gridDim.y + blockIdx.y;
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == (unsigned)(ti.x - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
 #pragma unroll
-                for (int k = 0; k < TT / 2; ++k) acc[k] = make_float2(0.f, 0.f);
-                for (int i = 0; i < np; ++i) {
-                    int a = r - soff[i].y;
-                    a += a < 0 ? G : 0;
-                    if ((unsigned)a >= (unsigned)W) continue;
-                    const float wy = swt[i * 2 * W + W + a];
-                    float2 v = sval[i * 16 + l];
-                    v.x *= wy;
-                    v.y *= wy;
-                    const float4* wr = reinterpret_cast<const float4*>(wrow + i * TT + h * (TT / 2));
+    for (int c = 0; c < CPL; ++c) sum[c] = make_float2(0.f, 0.f);
+    for (int k = 0; k < ti.x; ++k)
 #pragma unroll
-                    for (int k4 = 0; k4 < TT / 8; ++k4) {
-                        const float4 w4 = wr[k4];
-                        const float wk[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            acc[4 * k4 + q].x = fmaf(wk[q], v.x, acc[4 * k4 + q].x);
-                            acc[4 * k4 + q].y = fmaf(wk[q], v.y, acc[4 * k4 + q].y);
-                        }
-                    }
-                }
-                const int64_t rowo = it.w < 0 ? ((int64_t)(y0 + r) * G + x0) * L : (int64_t)r * TT * L;
-#pragma unroll
-                for (int k = 0; k < TT / 2; ++k) dst[rowo + (int64_t)(h + 2 * k) * L + l0 + l] = acc[k];
-            }
-            __syncthreads();
-        }
-    }
-    for (int l0 = 0; !FULL16 && l0 < L; l0 += LCS) {
-        const int lc = min(LCS, L - l0);
-        for (int e = threadIdx.x; e < np * lc; e += blockDim.x) {
-            const int i = e / lc, l = e - i * lc;
-            sval[i * LCS + l] = __ldg(ys + (int64_t)sidx[i] * L + l0 + l);
-        }
-        __syncthreads();
-        const int npair = TT * lc;
-        int px[NK], pl[NK];
-#pragma unroll
-        for (int k = 0; k < NK; ++k) {
-            const int pp = lane + 32 * k;
-            px[k] = pp / lc;
-            pl[k] = pp - px[k] * lc;
-        }
-        float2* dst = it.w < 0 ? grid : partial + (int64_t)it.w * TT * TT * L;
-        for (int r = warp; r < TT; r += kSpreadWarps) {
-            float2 acc[NK];
-#pragma unroll
-            for (int k = 0; k < NK; ++k) acc[k] = make_float2(0.f, 0.f);
-            for (int i = 0; i < np; ++i) {
-                const int2 o = soff[i];
-                // the point's row tap for this row (the wrap matters only when the tile is
-                // the whole grid: there a footprint can leave its right edge and re-enter)
-                int a = r - o.y;
-                a += a < 0 ? G : 0;
-                if ((unsigned)a >= (unsigned)W) continue;
-                const float wy = swt[i * 2 * W + W + a];
-#pragma unroll
-                for (int k = 0; k < NK; ++k) {
-                    int b = px[k] - o.x;
-                    b += b < 0 ? G : 0;
-                    const int bc = min(max(b, 0), W - 1);
-                    float w = swt[i * 2 * W + bc];
-                    w = ((unsigned)b < (unsigned)W) ? w * wy : 0.f;
-                    const float2 v = sval[i * LCS + pl[k]];
-                    acc[k].x = fmaf(w, v.x, acc[k].x);
-                    acc[k].y = fmaf(w, v.y, acc[k].y);
-                }
-            }
-            const int64_t rowo = it.w < 0 ? ((int64_t)(y0 + r) * G + x0) * L : (int64_t)r * TT * L;
-#pragma unroll
-            for (int k = 0; k < NK; ++k)
-                if (lane + 32 * k < npair) dst[rowo + (int64_t)px[k] * L + l0 + pl[k]] = acc[k];
-        }
-        __syncthreads();
-    }
-    if (it.w >= 0) {
-        // the last item of the tile to arrive sums the partial slots in order
-        __threadfence();
-        __syncthreads();
-        const int2 ti = tinfo[t];
-        if (threadIdx.x == 0) last = atomicAdd(&tickets[t], 1u) == (unsigned)(ti.x - 1);
-        __syncthreads();
-        if (last) {
-            __threadfence();
-            const int64_t slot = (int64_t)TT * TT * L;
-            const float2* p0 = partial + (int64_t)ti.y * slot;
-            for (int e = threadIdx.x; e < TT * TT * L; e += blockDim.x) {
-                float2 acc = __ldcg(p0 + e);
-                for (int c = 1; c < ti.x; ++c) {
-                    const float2 v = __ldcg(p0 + c * slot + e);
-                    acc.x += v.x;
-                    acc.y += v.y;
-                }
-                const int l = e % L, cell = e / L;
-                const int r = cell / TT, cx = cell - r * TT;
-                grid[((int64_t)(y0 + r) * G + x0 + cx) * L + l] = acc;
-            }
-            if (threadIdx.x == 0) tickets[t] = 0u;
-        }
-    }
+        for (int c = 0; c < CPL; ++c) sum[c] = cadd(sum[c], __ldcg(pc + (ti.y + k) * slot + c));
+    put_coils<CPL>(cell(warp), sum, ncoil, pairs);
+    if (threadIdx.x == 0) *ticket = 0u;
 }
 
 // Column gx: IFFT along y of the spread grid, keep the image rows -> V[iy][gx][l].
@@ -869,86 +795,95 @@ static int adj_fft_impl(hqs_plan_s* p, float2* x, float zc, const float2* z, cud
 template <int W>
 static int interp_impl(hqs_plan_s* p, float2* y, cudaStream_t st) {
     if (p->M == 0) return HQS_OK;
-    if (p->L % 16 == 0) {
-        const int64_t threads8 = p->M * 8;
-        HQS_CUDA_TRY(launch_pdl(k_interp16<W>, dim3((unsigned)ceil_div64(threads8, 256)), dim3(256), 0, st, p->grid,
-                                p->pts, p->spread.kbw, (int)p->M, p->G, p->L, p->spread.ysort));
-        const size_t smy = (size_t)kSortPts * (p->L + 1) * sizeof(float2);
-        HQS_CUDA_TRY(launch_pdl(k_y_from_sorted, dim3((unsigned)ceil_div64(p->M, kSortPts)), dim3(256), smy, st,
-                                p->spread.ysort, p->invperm, (int)p->M, p->L, y));
+    auto go = [&]<int VEC, int LPP>() -> int {
+        HQS_CUDA_TRY(launch_pdl(k_interp<W, VEC, LPP>, dim3((unsigned)ceil_div64(p->M * LPP, 256)), dim3(256), 0, st,
+                                p->grid, p->pts, p->spread.kbw, p->perm, (int)p->M, p->G, p->L, y));
         HQS_CUDA_TRY(cudaGetLastError());
         return HQS_OK;
-    }
-    const int64_t threads = p->M * 16;
-    HQS_CUDA_TRY(launch_pdl(k_interp<W>, dim3((unsigned)ceil_div64(threads, 256)), dim3(256), 0, st, p->grid, p->pts,
-                            p->perm, (int)p->M, p->G, p->L, (float)p->beta, y));
-    HQS_CUDA_TRY(cudaGetLastError());
-    return HQS_OK;
+    };
+    // lanes per point: as many as the coils fill (pairs of coils need an even count)
+    if (p->L % 2 == 0) return p->L > 4 ? go.template operator()<2, 8>() : go.template operator()<2, 2>();
+    return p->L > 4 ? go.template operator()<1, 16>() : go.template operator()<1, 4>();
 }
 
-// Kaiser-Bessel weights of every sorted point: kbw[j][h] = phi(dx_j - h),
-// kbw[j][W + h] = phi(dy_j - h), h < W (a plan-time table of the spreading).
+// Kaiser-Bessel weights of the sorted points, 24 floats each: x taps [8], y taps as
+// pairs [8][2] (the operand of packed multiply-adds); zero beyond W.
 __global__ void k_point_weights(const int4* __restrict__ pts, int M, int W, float beta, float* __restrict__ kbw) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= (int64_t)M * 2 * W) return;
-    const int j = (int)(e / (2 * W)), h = (int)(e - (int64_t)j * 2 * W);
+    if (e >= (int64_t)M * 16) return;
+    const int j = (int)(e >> 4), h = (int)(e & 15), b = h & 7;
     const int4 pt = pts[j];
-    const float t = h < W ? __int_as_float(pt.z) - (float)h : __int_as_float(pt.w) - (float)(h - W);
-    kbw[e] = kb_phi(t, (float)W, beta);
+    const float t = __int_as_float(h < 8 ? pt.z : pt.w) - (float)b;
+    const float w = b < W ? kb_phi(t, (float)W, beta) : 0.f;
+    float* o = kbw + (int64_t)j * 24;
+    if (h < 8) o[b] = w;
+    else o[8 + 2 * b] = o[9 + 2 * b] = w;
 }
 
 int launch_point_weights(hqs_plan_s* p, cudaStream_t st) {
     if (p->M == 0) return HQS_OK;
-    const int64_t cnt = p->M * 2 * p->W;
-    k_point_weights<<<(unsigned)ceil_div64(cnt, 256), 256, 0, st>>>(p->pts, (int)p->M, p->W, (float)p->beta,
-                                                                     p->spread.kbw);
+    k_point_weights<<<(unsigned)ceil_div64(p->M * 16, 256), 256, 0, st>>>(p->pts, (int)p->M, p->W, (float)p->beta,
+                                                                          p->spread.kbw);
     HQS_CUDA_TRY(cudaGetLastError());
     return HQS_OK;
 }
 
-// coils per chunk of the tile-owned spreading (shared tile TT^2 x LCS)
-inline int spread_lcs(int tile, int L) {
-    (void)tile;
-    const int nch = ceil_div(L, 16);
-    return ceil_div(L, nch);
+// The tiles (up to two per axis) that a point's footprint touches: f(tile, offsets).
+template <class F> HQS_DEV void touched_tiles(int4 p, int W, int G, F&& f) {
+    constexpr int T = kTile;
+    const int i0[2] = {p.x, p.y};
+    int t[2][2], o[2][2], n[2];
+    for (int a = 0; a < 2; ++a) {
+        int e = i0[a] + W - 1;
+        e -= e >= G ? G : 0;
+        t[a][0] = i0[a] / T;
+        o[a][0] = i0[a] - t[a][0] * T;
+        t[a][1] = e / T;
+        const int d = i0[a] - t[a][1] * T;
+        o[a][1] = d > 0 ? d - G : d;   // taps that wrap start before cell 0
+        n[a] = t[a][1] != t[a][0] ? 2 : 1;
+    }
+    for (int b = 0; b < n[1]; ++b)
+        for (int a = 0; a < n[0]; ++a) f(t[1][b] * (G / T) + t[0][a], (o[0][a] + 16) | ((o[1][b] + 16) << 8));
+}
+__global__ void k_tile_count(const int4* __restrict__ pts, int M, int W, int G, int* __restrict__ counts) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < M) touched_tiles(pts[j], W, G, [&](int t, int) { atomicAdd(&counts[t], 1); });
+}
+__global__ void k_tile_fill(const int4* __restrict__ pts, const int* __restrict__ perm, int M, int W, int G,
+                            int* __restrict__ cursor, int4* __restrict__ list) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < M)
+        touched_tiles(pts[j], W, G,
+                      [&](int t, int off) { list[atomicAdd(&cursor[t], 1)] = make_int4(j, perm[j], off, 0); });
 }
 
-inline size_t spread_smem(int W, int lcs, int tile) {
-    return (size_t)HQS_SPREAD_CAND * lcs * sizeof(float2) + (size_t)HQS_SPREAD_CAND * 2 * W * sizeof(float) +
-           (size_t)HQS_SPREAD_CAND * (sizeof(int2) + sizeof(int)) + (size_t)HQS_SPREAD_CAND * tile * sizeof(float);
-}
-
-int launch_y_to_sorted(const float2* y, const int* inv, int64_t M, int L, float2* ysort, cudaStream_t st) {
-    if (M == 0) return HQS_OK;
-    const size_t smy = (size_t)kSortPts * (L + 1) * sizeof(float2);
-    HQS_CUDA_TRY(launch_pdl(k_y_to_sorted, dim3((unsigned)ceil_div64(M, kSortPts)), dim3(256), smy, st, y, inv, (int)M, L,
-                            ysort));
+int launch_tile_count(const hqs_plan_s* p, int* counts, cudaStream_t st) {
+    if (p->M > 0) k_tile_count<<<(unsigned)ceil_div64(p->M, 256), 256, 0, st>>>(p->pts, (int)p->M, p->W, p->G, counts);
+    HQS_CUDA_TRY(cudaGetLastError());
     return HQS_OK;
 }
-
-template <int W, int TT>
-static int spread_tiles_impl(hqs_plan_s* p, const float2* y, cudaStream_t st) {
-    const int lcs = spread_lcs(TT, p->L);
-    const bool full16 = p->L % 16 == 0;
-    const size_t sm = spread_smem(W, lcs, full16 ? TT : 0);
-    auto kern = full16 ? k_spread_tiles<W, TT, true> : k_spread_tiles<W, TT, false>;
-    HQS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    if (const int rc = launch_y_to_sorted(y, p->invperm, p->M, p->L, p->spread.ysort, st); rc != HQS_OK) return rc;
-    HQS_CUDA_TRY(launch_pdl(kern, dim3(p->spread.nitems), dim3(256), sm, st, p->spread.ysort, p->pts, p->spread.kbw,
-                            p->spread.tile_nb, p->spread.items, p->spread.tile_info, p->spread.tickets,
-                            p->spread.partial, p->G, p->L, lcs, p->nbx, p->grid));
+int launch_tile_fill(const hqs_plan_s* p, int* cursor, int4* list, cudaStream_t st) {
+    if (p->M > 0)
+        k_tile_fill<<<(unsigned)ceil_div64(p->M, 256), 256, 0, st>>>(p->pts, p->perm, (int)p->M, p->W, p->G, cursor,
+                                                                     list);
     HQS_CUDA_TRY(cudaGetLastError());
     return HQS_OK;
 }
 
 template <int W>
 static int spread_impl(hqs_plan_s* p, const float2* y, cudaStream_t st) {
-    switch (p->tile) {
-        case 8: return spread_tiles_impl<W, 8>(p, y, st);
-        case 16: return spread_tiles_impl<W, 16>(p, y, st);
-        case 32: return spread_tiles_impl<W, 32>(p, y, st);
-        default: return HQS_ERR_INVALID_ARG;
-    }
+    const int cpl = spread_cpl(p->L), nch = ceil_div(p->L, 4 * cpl);
+    const hqs_plan_s::Spread& S = p->spread;
+    auto go = [&]<int CPL>() -> int {
+        constexpr size_t sm = spread_smem<CPL>();
+        HQS_CUDA_TRY(cudaFuncSetAttribute(k_spread<W, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        HQS_CUDA_TRY(launch_pdl(k_spread<W, CPL>, dim3(S.nctas, nch), dim3(256), sm, st, y, S.kbw, S.list, S.ctas, S.light,
+                                S.tile_info, S.tickets, S.partial, p->M, p->G / kTile, p->G, p->L, p->grid));
+        HQS_CUDA_TRY(cudaGetLastError());
+        return HQS_OK;
+    };
+    return cpl == 1 ? go.template operator()<1>() : (cpl == 2 ? go.template operator()<2>() : go.template operator()<4>());
 }
 
 template <class F> static int dispatch_w(int W, F&& f) {

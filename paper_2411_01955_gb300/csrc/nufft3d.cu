@@ -406,6 +406,27 @@ __global__ void __launch_bounds__(256, 2) k_interp3(const float2* __restrict__ G
 // against 2630 and a 41 us memset with patches of 4 coils added by atomics (a whole
 // adjoint 2824 -> 1013 us; units of one point and 256-point batches: 1297 us).
 #define HQS3_ITEM 256
+// k-space data to the sorted point order, coil-innermost: ys[inv[m]][l] = y[l][m].  A CTA
+// stages kSortPts caller-order points of every coil (coalesced rows of y) in shared
+// memory and writes each point's L-coil line contiguously.
+constexpr int kSortPts = 64;
+__global__ void __launch_bounds__(256) k_y_to_sorted(const float2* __restrict__ y, const int* __restrict__ inv,
+                                                     int64_t M, int L, float2* __restrict__ ys) {
+    extern __shared__ float4 smem4[];
+    float2* sy = reinterpret_cast<float2*>(smem4);   // [kSortPts][L + 1]
+    const int64_t m0 = (int64_t)blockIdx.x * kSortPts;
+    const int np = (int)min((int64_t)kSortPts, M - m0);
+    for (int e = threadIdx.x; e < L * kSortPts; e += blockDim.x) {
+        const int l = e / kSortPts, q = e - l * kSortPts;
+        if (q < np) sy[q * (L + 1) + l] = y[(int64_t)l * M + m0 + q];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < np * L; e += blockDim.x) {
+        const int q = e / L, l = e - q * L;
+        ys[(int64_t)inv[m0 + q] * L + l] = sy[q * (L + 1) + l];
+    }
+}
+
 constexpr int kBatch3 = 32;    // units staged at once (one per lane of the plane test)
 // bytes of one point's slot: 32 weights, CL values
 template <int CPL> constexpr int spread3_slot() { return 128 + 4 * CPL * (int)sizeof(float2); }
@@ -1327,9 +1348,6 @@ int spread3_unit(const Points3& pts, const int G[3], double beta, float2* grid, 
     return HQS_OK;
 }
 
-// coils per lane of the tile-owned spreading (4 lanes share a cell)
-int spread3_cpl(int L) { return L <= 4 ? 1 : (L <= 8 ? 2 : 4); }
-
 // The plan's points in footprint order, their weights, the interpolation's units and the
 // spreading's items, from the points in bin order (host offsets pts.off).
 int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
@@ -1418,7 +1436,7 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
         std::stable_sort(items.begin(), items.end(),
                          [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
         p->nitems = (int)items.size();
-        const int cl = 4 * spread3_cpl(p->L), nch = ceil_div(p->L, cl);
+        const int cl = 4 * spread_cpl(p->L), nch = ceil_div(p->L, cl);
         if ((rc = alloc3(p, &p->items, items.size())) != HQS_OK) break;
         if ((rc = alloc3(p, &p->tinfo, tinfo.size())) != HQS_OK) break;
         if ((rc = alloc3(p, &p->tickets, (size_t)nbins * nch)) != HQS_OK) break;
@@ -1435,8 +1453,10 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
 
 // Spread the k-space data y onto the plan's grid (every cell written).
 int spread3(hqs_plan3d_s* p, const float2* y, float2* grid, cudaStream_t s) {
-    TRY3(launch_y_to_sorted(y, p->inv, p->M, p->L, p->ysort, s));
-    const int cpl = spread3_cpl(p->L), nch = ceil_div(p->L, 4 * cpl);
+    if (p->M > 0)
+        k_y_to_sorted<<<(unsigned)ceil_div64(p->M, kSortPts), 256, (size_t)kSortPts * (p->L + 1) * sizeof(float2), s>>>(
+            y, p->inv, p->M, p->L, p->ysort);
+    const int cpl = spread_cpl(p->L), nch = ceil_div(p->L, 4 * cpl);
     return dispatch_w3(p->W, [&]<int WW>() {
         auto go = [&]<int CPL>() {
             const size_t sm = spread3_smem<CPL>();

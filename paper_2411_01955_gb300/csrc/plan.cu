@@ -113,11 +113,6 @@ __global__ void k_point_scatter(const int4* __restrict__ raw, const int* __restr
     perm[pos] = j;
 }
 
-__global__ void k_invert_perm(const int* __restrict__ perm, int M, int* __restrict__ inv) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < M) inv[perm[j]] = j;
-}
-
 // Toeplitz kernel c[py][px] = Npix^-1 sum_j exp(+i (kx_j dx + ky_j dy)), d the
 // circulant offset of position p, as a complex GEMM Ey^T Ex whose operands are
 // generated in shared memory.  Phases are formed in turns from the split
@@ -300,6 +295,24 @@ static void plan_free(hqs_plan_s* p) {
     delete p;
 }
 
+// The range of accepted plans: the partial tiles of tile x tile bins, one for every 256
+// points of a bin's distinct neighbours where there are more than 256, stay within 1 GiB.
+static int spread_limit(const hqs_plan_s* p, const std::vector<int>& hc) {
+    const int T = p->tile, nbx = p->G / T, m = std::min(nbx, 3);
+    int64_t slots = 0;
+    for (int t = 0; t < nbx * nbx; ++t) {
+        int64_t cand = 0;
+        for (int a = 0; a < m; ++a)
+            for (int b = 0; b < m; ++b) {
+                const int by = (t / nbx + a - (m == 3) + nbx) % nbx, bx = (t % nbx + b - (m == 3) + nbx) % nbx;
+                cand += hc[by * nbx + bx];
+            }
+        const int64_t k = ceil_div64(cand, 256);
+        if (k > 1) slots += k;
+    }
+    return slots * T * T * p->L * (int64_t)sizeof(float2) > ((int64_t)1 << 30) ? HQS_ERR_UNSUPPORTED : HQS_OK;
+}
+
 static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user, cudaStream_t s) {
     const int n = p->n, L = p->L, G = p->G, n2 = p->n2;
     const int M = (int)p->M;
@@ -315,9 +328,7 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
     HQS_TRY(dev_alloc(p, &p->apod, (size_t)n));
     HQS_TRY(dev_alloc(p, &p->pts, (size_t)std::max(M, 1)));
     HQS_TRY(dev_alloc(p, &p->perm, (size_t)std::max(M, 1)));
-    HQS_TRY(dev_alloc(p, &p->invperm, (size_t)std::max(M, 1)));
-    HQS_TRY(dev_alloc(p, &p->spread.ysort, (size_t)std::max(M, 1) * L));
-    HQS_TRY(dev_alloc(p, &p->spread.kbw, (size_t)std::max(M, 1) * 2 * p->W));
+    HQS_TRY(dev_alloc(p, &p->spread.kbw, (size_t)std::max(M, 1) * 24));
     HQS_TRY(dev_alloc(p, &p->khat, (size_t)n2 * n2));
     HQS_TRY(dev_alloc(p, &p->lam, (size_t)n * n));
     HQS_TRY(dev_alloc(p, &p->grid, (size_t)G * G * L));
@@ -429,12 +440,10 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
             rc = HQS_ERR_CUDA;
             break;
         }
-        if (M > 0) {
-            k_point_scatter<<<ceil_div(M, 256), 256, 0, s>>>(raw, bin, M, counts, p->pts, p->perm);
-            k_invert_perm<<<ceil_div(M, 256), 256, 0, s>>>(p->perm, M, p->invperm);
-        }
+        if ((rc = spread_limit(p, hc)) != HQS_OK) break;
+        if (M > 0) k_point_scatter<<<ceil_div(M, 256), 256, 0, s>>>(raw, bin, M, counts, p->pts, p->perm);
         if ((rc = launch_point_weights(p, s)) != HQS_OK) break;
-        if ((rc = spread_build(p, hc, s)) != HQS_OK) break;
+        if ((rc = spread_build(p, s)) != HQS_OK) break;
 
         // Toeplitz kernel, its FFT (Khat, real, scaled by 1/n2^2) and the density symbol
         dim3 gg(ceil_div(n2, 64), ceil_div(n2, 64));
@@ -502,7 +511,10 @@ int plan_create_internal(hqs_plan* out, const float* traj, int64_t M, int ny, in
     return HQS_OK;
 }
 
-// Re-binning of the already sorted points for another spreading tile size.
+static int tile_counts(hqs_plan_s* p, int* cursor, std::vector<int>& cnt, cudaStream_t s);
+static int tile_list(hqs_plan_s* p, int* cursor, const std::vector<int>& cnt, int4* list, cudaStream_t s);
+
+// Re-binning of the already sorted points for another bin size.
 __global__ void k_rebin(const int4* __restrict__ pts, int M, int G, int W, int TB, int nbx,
                         int* __restrict__ bin, int* __restrict__ counts) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -533,14 +545,15 @@ extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     const int M = (int)p->M;
     const int nbx = p->G / tile, nbins = nbx * nbx;
-    int *bin = nullptr, *counts = nullptr, *perm2 = nullptr;
+    int *bin = nullptr, *counts = nullptr, *perm2 = nullptr, *cursor = nullptr;
     int4* pts2 = nullptr;
     int rc = HQS_OK;
     const int old_tile = p->tile, old_nbx = p->nbx;
     do {
         const int Mp = std::max(M, 1);
         if (cudaMalloc(&bin, Mp * sizeof(int)) || cudaMalloc(&counts, nbins * sizeof(int)) ||
-            cudaMalloc(&perm2, Mp * sizeof(int)) || cudaMalloc(&pts2, Mp * sizeof(int4))) {
+            cudaMalloc(&perm2, Mp * sizeof(int)) || cudaMalloc(&pts2, Mp * sizeof(int4)) ||
+            cudaMalloc(&cursor, (size_t)(p->G / 8) * (p->G / 8) * sizeof(int))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -558,10 +571,9 @@ extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
             rc = HQS_ERR_CUDA;
             break;
         }
-        // items for the new tile first: if they cannot be built the points stay as they are
         p->tile = tile;
         p->nbx = nbx;
-        if ((rc = spread_build(p, hc, s)) != HQS_OK) {
+        if ((rc = spread_limit(p, hc)) != HQS_OK) {
             p->tile = old_tile;
             p->nbx = old_nbx;
             break;
@@ -572,10 +584,14 @@ extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
             rc = HQS_ERR_CUDA;
             break;
         }
-        if (M > 0) k_invert_perm<<<ceil_div(M, 256), 256, 0, s>>>(p->perm, M, p->invperm);
         if ((rc = launch_point_weights(p, s)) != HQS_OK) break;
+        // the tiles' lists name points by their place in the sorted order
+        std::vector<int> cnt;
+        if ((rc = tile_counts(p, cursor, cnt, s)) != HQS_OK) break;
+        if ((rc = tile_list(p, cursor, cnt, p->spread.list, s)) != HQS_OK) break;
         if (cudaStreamSynchronize(s)) { rc = HQS_ERR_CUDA; break; }
     } while (0);
+    cudaFree(cursor);
     cudaFree(bin);
     cudaFree(counts);
     cudaFree(perm2);
@@ -585,95 +601,105 @@ extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
 
 // ------------------------------------------------ tile-owned spreading items
 void spread_free(hqs_plan_s* p) {
-    cudaFree(p->spread.items);
-    cudaFree(p->spread.tile_info);
-    cudaFree(p->spread.tile_nb);
-    cudaFree(p->spread.tickets);
-    cudaFree(p->spread.partial);
-    p->spread.items = nullptr;
-    p->spread.tile_info = nullptr;
-    p->spread.tile_nb = nullptr;
-    p->spread.tickets = nullptr;
-    p->spread.partial = nullptr;
-    p->bytes -= p->spread.bytes;
-    p->spread.bytes = 0;
-    p->spread.nitems = p->spread.nslots = 0;
+    hqs_plan_s::Spread& S = p->spread;
+    for (void* v : {(void*)S.list, (void*)S.ctas, (void*)S.light, (void*)S.tile_info, (void*)S.tickets, (void*)S.partial})
+        cudaFree(v);
+    p->bytes -= S.bytes;
+    float* kbw = S.kbw;
+    S = hqs_plan_s::Spread();
+    S.kbw = kbw;
 }
 
-// Every tile of p->tile x p->tile grid cells gets items of at most
-// HQS_SPREAD_CAND candidates: the points of its distinct neighbouring bins
-// (3 x 3, fewer when the grid has fewer than 3 bins per axis).  A tile with
-// more candidates gets several items, each with a partial slot.
-int spread_build(hqs_plan_s* p, const std::vector<int>& hc, cudaStream_t s) {
-    const int T = p->tile, nbx = p->G / T, nbins = nbx * nbx, L = p->L;
-    if ((int)hc.size() != nbins) return HQS_ERR_INVALID_ARG;
-    std::vector<int> off(nbins + 1, 0);
-    for (int b = 0; b < nbins; ++b) off[b + 1] = off[b] + hc[b];
-    auto distinct = [&](int t, int* out) {
-        int c = 0;
-        for (int d = -1; d <= 1; ++d) {
-            const int v = (t + d + nbx) % nbx;
-            bool seen = false;
-            for (int k = 0; k < c; ++k) seen |= out[k] == v;
-            if (!seen) out[c++] = v;
-        }
-        return c;
-    };
-    std::vector<int4> items;
-    std::vector<int2> info(nbins), nbt((size_t)nbins * 10, make_int2(0, 0));
-    int slots = 0;
-    for (int t = 0; t < nbins; ++t) {
-        int xs[3], ys[3];
-        const int cx = distinct(t % nbx, xs), cy = distinct(t / nbx, ys);
-        int cand = 0, k = 0;
-        for (int a = 0; a < cy; ++a)
-            for (int b = 0; b < cx; ++b, ++k) {
-                const int bin = ys[a] * nbx + xs[b];
-                nbt[(size_t)t * 10 + k] = make_int2(off[bin], cand);
-                cand += hc[bin];
-            }
-        nbt[(size_t)t * 10 + 9] = make_int2(k, cand);
-        const int nch = std::max(1, ceil_div(cand, HQS_SPREAD_CAND));
-        const int first = nch > 1 ? slots : -1;
-        if (nch > 1) slots += nch;
-        info[t] = make_int2(nch, first);
-        for (int k = 0; k < nch; ++k)
-            items.push_back(make_int4(t, k * HQS_SPREAD_CAND, std::min((k + 1) * HQS_SPREAD_CAND, cand),
-                                      nch > 1 ? first + k : -1));
+// points that touch each 8 x 8 tile of the grid, into `cnt` (cursor: device scratch, one
+// int per tile); the counts do not depend on the order of the points
+static int tile_counts(hqs_plan_s* p, int* cursor, std::vector<int>& cnt, cudaStream_t s) {
+    const int nt = (p->G / 8) * (p->G / 8);
+    cnt.resize(nt);
+    HQS_CUDA_TRY(cudaMemsetAsync(cursor, 0, nt * sizeof(int), s));
+    HQS_TRY(launch_tile_count(p, cursor, s));
+    HQS_CUDA_TRY(cudaMemcpyAsync(cnt.data(), cursor, nt * sizeof(int), cudaMemcpyDeviceToHost, s));
+    HQS_CUDA_TRY(cudaStreamSynchronize(s));
+    return HQS_OK;
+}
+// the list itself, tile by tile in the order of `cnt`
+static int tile_list(hqs_plan_s* p, int* cursor, const std::vector<int>& cnt, int4* list, cudaStream_t s) {
+    std::vector<int> off(cnt.size());
+    int acc = 0;
+    for (size_t t = 0; t < cnt.size(); ++t) {
+        off[t] = acc;
+        acc += cnt[t];
     }
-    // heaviest items first: the long ones start at once instead of at the end
-    std::stable_sort(items.begin(), items.end(),
-                     [](const int4& u, const int4& v) { return u.z - u.y > v.z - v.y; });
-    const size_t slot_elems = (size_t)T * T * L;
-    if ((size_t)slots * slot_elems * sizeof(float2) > ((size_t)1 << 30)) return HQS_ERR_UNSUPPORTED;
+    HQS_CUDA_TRY(cudaMemcpyAsync(cursor, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+    HQS_TRY(launch_tile_fill(p, cursor, list, s));
+    HQS_CUDA_TRY(cudaStreamSynchronize(s));
+    return HQS_OK;
+}
+
+// Lists the points of every 8 x 8 tile and deals the tiles to CTAs: tiles of more than
+// HQS_SPREAD_LIGHT points first, heaviest CTAs in front, 8 HQS_SPREAD_LIGHT points at
+// most to a CTA (several CTAs of one tile have partial slots); then the light tiles,
+// fullest first, eight to a CTA.
+int spread_build(hqs_plan_s* p, cudaStream_t s) {
+    const int nbx = p->G / 8, nt = nbx * nbx;
+    const int cl = 4 * spread_cpl(p->L), nch = ceil_div(p->L, cl);
+    int* cursor = nullptr;
+    HQS_CUDA_TRY(cudaMalloc(&cursor, nt * sizeof(int)));
     hqs_plan_s::Spread nw;
-    nw.nitems = (int)items.size();
-    nw.nslots = slots;
-    nw.ysort = p->spread.ysort;
     nw.kbw = p->spread.kbw;
-    int rc = HQS_OK;
-    if (cudaMalloc(&nw.items, items.size() * sizeof(int4)) ||
-        cudaMalloc(&nw.tile_info, nbins * sizeof(int2)) || cudaMalloc(&nw.tickets, nbins * sizeof(unsigned)) ||
-        cudaMalloc(&nw.tile_nb, (size_t)nbins * 10 * sizeof(int2)) ||
-        (slots > 0 && cudaMalloc(&nw.partial, slots * slot_elems * sizeof(float2)))) {
-        rc = HQS_ERR_OOM;
-    } else if (cudaMemcpyAsync(nw.items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, s) ||
-               cudaMemcpyAsync(nw.tile_info, info.data(), nbins * sizeof(int2), cudaMemcpyHostToDevice, s) ||
-               cudaMemcpyAsync(nw.tile_nb, nbt.data(), (size_t)nbins * 10 * sizeof(int2), cudaMemcpyHostToDevice, s) ||
-               cudaMemsetAsync(nw.tickets, 0, nbins * sizeof(unsigned), s) || cudaStreamSynchronize(s)) {
-        rc = HQS_ERR_CUDA;
-    }
+    auto build = [&]() -> int {
+        std::vector<int> cnt;
+        HQS_TRY(tile_counts(p, cursor, cnt, s));
+        int64_t total = 0;
+        for (int c : cnt) total += c;
+        if (total > 0x7fffffffLL) return HQS_ERR_UNSUPPORTED;
+        std::vector<int4> heavy, light;
+        std::vector<int2> info(nt, make_int2(0, 0));
+        int slots = 0, off = 0;
+        for (int t = 0; t < nt; ++t) {
+            const int n = cnt[t], k = ceil_div(n, 8 * HQS_SPREAD_LIGHT);
+            if (n <= HQS_SPREAD_LIGHT) {
+                light.push_back(make_int4(t, off, off + n, 0));
+            } else {
+                info[t] = make_int2(k, slots);
+                for (int i = 0; i < k; ++i)
+                    heavy.push_back(make_int4(t, off + (int)((int64_t)n * i / k), off + (int)((int64_t)n * (i + 1) / k),
+                                              k > 1 ? slots + i : -1));
+                if (k > 1) slots += k;
+            }
+            off += n;
+        }
+        auto more = [](const int4& u, const int4& v) { return u.z - u.y > v.z - v.y; };
+        std::stable_sort(heavy.begin(), heavy.end(), more);
+        std::stable_sort(light.begin(), light.end(), more);
+        std::vector<int4> ctas = heavy;
+        for (int i = 0; i < (int)light.size(); i += 8)
+            ctas.push_back(make_int4(-1, i, std::min(i + 8, (int)light.size()), -1));
+        nw.nctas = (int)ctas.size();
+        const size_t nl = std::max<size_t>(off, 1), ng = std::max<size_t>(light.size(), 1);
+        const size_t np = (size_t)std::max(slots, 1) * nch * 64 * cl;
+        HQS_CUDA_TRY(cudaMalloc(&nw.list, nl * sizeof(int4)));
+        HQS_CUDA_TRY(cudaMalloc(&nw.ctas, ctas.size() * sizeof(int4)));
+        HQS_CUDA_TRY(cudaMalloc(&nw.light, ng * sizeof(int4)));
+        HQS_CUDA_TRY(cudaMalloc(&nw.tile_info, nt * sizeof(int2)));
+        HQS_CUDA_TRY(cudaMalloc(&nw.tickets, (size_t)nt * nch * sizeof(unsigned)));
+        HQS_CUDA_TRY(cudaMalloc(&nw.partial, np * sizeof(float2)));
+        nw.bytes = (nl + ctas.size() + ng) * sizeof(int4) + nt * sizeof(int2) + (size_t)nt * nch * sizeof(unsigned) +
+                   np * sizeof(float2);
+        HQS_CUDA_TRY(cudaMemcpyAsync(nw.ctas, ctas.data(), ctas.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+        HQS_CUDA_TRY(cudaMemcpyAsync(nw.light, light.data(), light.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+        HQS_CUDA_TRY(cudaMemcpyAsync(nw.tile_info, info.data(), nt * sizeof(int2), cudaMemcpyHostToDevice, s));
+        HQS_CUDA_TRY(cudaMemsetAsync(nw.tickets, 0, (size_t)nt * nch * sizeof(unsigned), s));
+        return tile_list(p, cursor, cnt, nw.list, s);
+    };
+    const int rc = build();
+    cudaFree(cursor);
     if (rc != HQS_OK) {
-        cudaFree(nw.items);
-        cudaFree(nw.tile_info);
-        cudaFree(nw.tile_nb);
-        cudaFree(nw.tickets);
-        cudaFree(nw.partial);
+        for (void* v : {(void*)nw.list, (void*)nw.ctas, (void*)nw.light, (void*)nw.tile_info, (void*)nw.tickets,
+                        (void*)nw.partial})
+            cudaFree(v);
         return rc;
     }
     spread_free(p);
-    nw.bytes = items.size() * sizeof(int4) + nbins * (11 * sizeof(int2) + sizeof(unsigned)) +
-               slots * slot_elems * sizeof(float2);
     p->spread = nw;
     p->bytes += nw.bytes;
     return HQS_OK;
@@ -692,7 +718,7 @@ extern "C" int hqs_plan_get_info(hqs_plan p, hqs_plan_info* info) {
     info->npoints = p->M;
     info->kb_beta = p->beta;
     info->device_bytes = p->bytes;
-    info->nsub = p->spread.nitems;
+    info->nsub = p->spread.nctas;
     info->tile = p->tile;
     return HQS_OK;
 }

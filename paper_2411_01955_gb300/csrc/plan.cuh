@@ -11,7 +11,7 @@
 #endif
 #define HQS_MAX_LC HQS_KLINES  // coils per chunk in the FFT passes
 #define HQS_MAX_BLOCKS 2048    // partial-sum slots per reduction (and >= 3 x 256 for the FCG dots)
-#define HQS_SPREAD_CAND 256    // candidate points per tile-owned spreading item
+#define HQS_SPREAD_LIGHT 64    // points of a grid tile that one warp spreads; heavier tiles take whole CTAs
 #define HQS_TRACE_MAX 4096     // phase-trace stamps kept per persistent solve
 
 // CG scalars kept on the device so that the solve never needs the host
@@ -57,21 +57,20 @@ struct hqs_plan_s {
     float* apod = nullptr;      // [n] 1/phihat((i - n/2)/G)
     int4* pts = nullptr;        // sorted points: (i0x, i0y, bits(dx), bits(dy)), i0 in [0, G)
     int* perm = nullptr;        // sorted -> caller index
-    int* invperm = nullptr;     // caller index -> sorted position
-    // tile-owned spreading (adjoint): every grid tile of tile x tile cells is
-    // written by the CTAs of its items; candidates are the points of the 3 x 3
-    // neighbouring bins, taken in chunks of <= HQS_SPREAD_CAND
+    // tile-owned spreading (adjoint): every 8 x 8 tile of the grid is written by the warps
+    // that own it, from the list of the points that touch it
     struct Spread {
-        int4* items = nullptr;         // (tile, first candidate, end candidate, partial slot or -1)
-        int2* tile_info = nullptr;     // [nbins] (chunks, first partial slot)
-        int2* tile_nb = nullptr;       // [nbins][10]: (first point, candidate prefix) of each distinct
-                                       // neighbouring bin in candidate order, entry 9 = (bins, candidates)
-        unsigned* tickets = nullptr;   // [nbins] arrival counts of multi-chunk tiles (reset by the last)
-        float2* partial = nullptr;     // [slots][tile * tile * L] partial tiles of multi-chunk tiles
-        float2* ysort = nullptr;       // [M][L] k-space data in sorted order, coil-innermost
-        float* kbw = nullptr;          // [M][2W] Kaiser-Bessel weights of the sorted points (x taps, y taps)
-        int nitems = 0, nslots = 0;
-        size_t bytes = 0;              // device bytes of the arrays above but ysort
+        int4* list = nullptr;          // tile by tile: (sorted point, caller index, offset of the first tap
+                                       // from the tile's origin + 16 in one byte per axis, 0)
+        int4* ctas = nullptr;          // (tile, first entry, end entry, partial slot or -1), or, for eight
+                                       // light tiles, (-1, first, end, -1) in `light`
+        int4* light = nullptr;         // (tile, first entry, end entry, 0)
+        int2* tile_info = nullptr;     // [tiles] (CTAs, first partial slot) of tiles with several CTAs
+        unsigned* tickets = nullptr;   // [tiles][coil chunks] arrival counts of those (reset by the last)
+        float2* partial = nullptr;     // [slots][coil chunks][64][coils of a chunk] their partial tiles
+        float* kbw = nullptr;          // [M][24] Kaiser-Bessel weights of the sorted points
+        int nctas = 0;
+        size_t bytes = 0;              // device bytes of the arrays above but kbw
     } spread;
     float* khat = nullptr;      // [n2][n2] transposed (khat[kx][ky]), includes 1/n2^2
     float* lam = nullptr;       // [n][n] density symbol
@@ -133,14 +132,15 @@ int launch_half_group(int G, int n, int lines, int maxchunk, int count, const vo
                       cudaStream_t s);
 int launch_spread(hqs_plan_s* p, const float2* y, cudaStream_t s);
 int launch_interp(hqs_plan_s* p, float2* y, cudaStream_t s);
-// ysort[inv[m]][l] = y[l][m] (csrc/nufft.cu)
-int launch_y_to_sorted(const float2* y, const int* inv, int64_t M, int L, float2* ysort, cudaStream_t s);
 int launch_adj_chunks(hqs_plan_s* p, float2* x, float zc, const float2* z, cudaStream_t s);
 int launch_toeplitz(hqs_plan_s* p, const float2* x, float2* out, cudaStream_t s);
 int launch_fft2d(const hqs_plan_s* p, float2* data, int N, bool inverse, cudaStream_t s);
 int launch_precond(hqs_plan_s* p, float a, float b, const float2* r, float2* z, cudaStream_t s);
-// (re)builds the tile-owned spreading items for p->tile from the per-bin point
-// counts (host) and the sorted points; blocking
-int spread_build(hqs_plan_s* p, const std::vector<int>& counts, cudaStream_t s);
+// coils per lane of the tile-owned spreading (4 lanes share a grid cell)
+inline int spread_cpl(int L) { return L <= 4 ? 1 : (L <= 8 ? 2 : 4); }
+// (re)builds the spreading lists from the sorted points; blocking
+int spread_build(hqs_plan_s* p, cudaStream_t s);
+int launch_tile_count(const hqs_plan_s* p, int* counts, cudaStream_t s);
+int launch_tile_fill(const hqs_plan_s* p, int* cursor, int4* list, cudaStream_t s);
 int launch_point_weights(hqs_plan_s* p, cudaStream_t s);   // spread.kbw from the sorted points
 void spread_free(hqs_plan_s* p);
