@@ -946,7 +946,7 @@ struct hqs_batch_s {
     // batched forward / adjoint: the lower-half passes' argument tables of the slices
     // that take them, grouped by grid size (rebuilt when the pointers change)
     struct HalfGroup {
-        int G, n, lines, maxchunk, first, count;
+        int G, n, lines, maxchunk, maxcoils, first, count;
     };
     void* d_half[2] = {nullptr, nullptr};   // [0] forward, [1] adjoint
     std::vector<HalfGroup> half_groups[2];
@@ -1340,13 +1340,14 @@ static int half_tables(hqs_batch_s* b, int dir, const float2* const* xin, float2
     for (int i = 0; i < b->ns; ++i) {
         const hqs_plan_s* p = b->plans[i];
         if (done[i] || !plan_half_passes(p)) continue;
-        hqs_batch_s::HalfGroup g{p->G, p->n, plan_half_lines(p), 0, slot, 0};
+        hqs_batch_s::HalfGroup g{p->G, p->n, plan_half_lines(p), 0, 0, slot, 0};
         for (int j = i; j < b->ns; ++j) {
             const hqs_plan_s* q = b->plans[j];
             if (done[j] || !plan_half_passes(q) || q->G != p->G || plan_half_lines(q) != g.lines) continue;
             fill_half_args(q, xin ? xin[j] : nullptr, xout ? xout[j] : nullptr, z ? z[j] : nullptr,
                            host.data() + sz * slot);
             g.maxchunk = std::max(g.maxchunk, q->nchunk);
+            g.maxcoils = std::max(g.maxcoils, q->L);
             ++g.count;
             ++slot;
             done[j] = 1;
@@ -1379,7 +1380,7 @@ extern "C" int hqs_batch_adjoint_axpy(hqs_batch b, const hqs_c64* const* y, floa
     }
     const size_t sz = half_args_bytes();
     for (const auto& g : b->half_groups[1])
-        HQS_TRY_RC(launch_half_group(g.G, g.n, g.lines, g.maxchunk, g.count,
+        HQS_TRY_RC(launch_half_group(g.G, g.n, g.lines, g.maxchunk, g.maxcoils, g.count,
                                      static_cast<unsigned char*>(b->d_half[1]) + sz * g.first, 1, zc, st));
     for (int i = 0; i < b->ns; ++i)
         if (plan_half_passes(b->plans[i])) HQS_TRY_RC(launch_adj_chunks(b->plans[i], X[i], zc, Z ? Z[i] : nullptr, st));
@@ -1396,7 +1397,7 @@ extern "C" int hqs_batch_forward(hqs_batch b, const hqs_c64* const* x, hqs_c64* 
     HQS_TRY_RC(half_tables(b, 0, Xin, nullptr, nullptr, st));
     const size_t sz = half_args_bytes();
     for (const auto& g : b->half_groups[0])
-        HQS_TRY_RC(launch_half_group(g.G, g.n, g.lines, g.maxchunk, g.count,
+        HQS_TRY_RC(launch_half_group(g.G, g.n, g.lines, g.maxchunk, g.maxcoils, g.count,
                                      static_cast<unsigned char*>(b->d_half[0]) + sz * g.first, 0, 0.f, st));
     for (int i = 0; i < b->ns; ++i) {
         hqs_plan_s* p = b->plans[i];

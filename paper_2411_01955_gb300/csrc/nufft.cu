@@ -179,26 +179,30 @@ HQS_DEV void half_forward(float2* s, const float2* twg, int lines, LD&& ld, ST&&
     }
 }
 
+// The forward passes take chunks of LINES coils, at most 8 for the two-stage transforms
+// (their lines do not meet, see toep_impl in toeplitz.cu; 320^2 x 16 coils forward 48.0 ->
+// 44.1 us).  The adjoint's columns, which load a whole line per thread at once, are slower
+// that way (384^2 x 13 coils adjoint 94.7 -> 102 us) and keep the plan's chunks.
 template <int G, int LINES> HQS_DEV void fwd_rows_h_item(const HalfArgs& A, int iy, int ch, float2* s) {
-    const int n = A.n, L = A.L, l0 = ch * A.LC;
+    const int n = A.n, L = A.L, l0 = ch * LINES;
     const float ay = A.apod[iy] * A.scale;
     const float2* xr = A.x + (int64_t)iy * n;
     const float2* sm = A.smaps + (int64_t)iy * n * L + l0;
     const float* apod = A.apod;
     float2* dst = A.work + (int64_t)iy * G * L + l0;
     half_forward<G, LINES>(
-        s, A.tw, min(A.LC, L - l0),
+        s, A.tw, min(LINES, L - l0),
         [&](int line, int q) { return cscale(cmul(__ldg(sm + (int64_t)q * L + line), __ldg(xr + q)), ay * __ldg(apod + q)); },
         [&](int line, int k, float2 v) { dst[(int64_t)k * L + line] = v; });
 }
 
 template <int G, int LINES> HQS_DEV void fwd_cols_h_item(const HalfArgs& A, int gx, int ch, float2* s) {
-    const int L = A.L, l0 = ch * A.LC;
+    const int L = A.L, l0 = ch * LINES;
     const int64_t rs = (int64_t)G * L;
     const float2* col = A.work + (int64_t)gx * L + l0;
     float2* dst = A.grid + (int64_t)gx * L + l0;
     half_forward<G, LINES>(
-        s, A.tw, min(A.LC, L - l0), [&](int line, int q) { return __ldg(col + q * rs + line); },
+        s, A.tw, min(LINES, L - l0), [&](int line, int q) { return __ldg(col + q * rs + line); },
         [&](int line, int k, float2 v) { dst[k * rs + line] = v; });
 }
 
@@ -292,7 +296,7 @@ template <int G, int LINES> HQS_DEV void adj_rows_h_item(const HalfArgs& A, int 
 
 // single slice: grid (rows or columns, chunks); batched: grid (rows or columns,
 // largest chunk count, slices), the slice's arguments from a device table
-#define HQS_HALF_KERNELS(NAME)                                                                                \
+#define HQS_HALF_KERNELS(NAME, CHUNKS)                                                                              \
     template <int G, int LINES>                                                                               \
     __global__ void __launch_bounds__(half_threads<G, LINES>(), 512 / half_threads<G, LINES>()) k_##NAME(HalfArgs A) { \
         HQS_PDL_ENTRY();                                                                                      \
@@ -306,13 +310,13 @@ template <int G, int LINES> HQS_DEV void adj_rows_h_item(const HalfArgs& A, int 
         extern __shared__ __align__(16) float2 s[];                                                           \
         HalfArgs A = tab[blockIdx.z];                                                                         \
         A.zc = zc;                                                                                            \
-        if ((int)blockIdx.y >= A.nchunk) return;                                                              \
+        if ((int)blockIdx.y >= (CHUNKS ? A.nchunk : (A.L + LINES - 1) / LINES)) return;                          \
         NAME##_item<G, LINES>(A, blockIdx.x, blockIdx.y, s);                                                  \
     }
-HQS_HALF_KERNELS(fwd_rows_h)
-HQS_HALF_KERNELS(fwd_cols_h)
-HQS_HALF_KERNELS(adj_cols_h)
-HQS_HALF_KERNELS(adj_rows_h)
+HQS_HALF_KERNELS(fwd_rows_h, false)
+HQS_HALF_KERNELS(fwd_cols_h, false)
+HQS_HALF_KERNELS(adj_cols_h, true)
+HQS_HALF_KERNELS(adj_rows_h, true)
 #undef HQS_HALF_KERNELS
 
 // Type-2 interpolation: LPP lanes per sorted point, lane q owning VEC coils of a chunk
@@ -701,6 +705,8 @@ inline bool half_passes(const hqs_plan_s* p) {
 }
 // lines per CTA of these passes: the smallest of 4, 8, 16 that holds the coil chunk
 inline int half_lines(const hqs_plan_s* p) { return p->G >= 128 && p->LC <= 8 ? (p->LC <= 4 ? 4 : 8) : kLines; }
+// lines per CTA of the passes whose lines do not meet
+template <int G, int LINES> constexpr int half_free_lines() { return fft16_ok<G>() && LINES > 8 ? 8 : LINES; }
 template <int G, class F> static int dispatch_half(int lines, F&& f) {
     if constexpr (fft16_ok<G>()) {
         if (lines == 4) return f.template operator()<4>();
@@ -737,13 +743,14 @@ static int fwd_fft_impl(hqs_plan_s* p, const float2* x, cudaStream_t st) {
     if constexpr (G % 2 == 0 && G != 16 && G != 320 && G != 384) {   // twice a supported image
         if (half_passes(p))
             return dispatch_half<G>(half_lines(p), [&]<int LN>() -> int {
-                constexpr int ht = half_threads<G, LN>();
-                constexpr size_t hs = half_smem<G, LN>();
-                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h<G, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
-                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h<G, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
+                constexpr int LI = half_free_lines<G, LN>(), ht = half_threads<G, LI>();
+                constexpr size_t hs = half_smem<G, LI>();
+                const int nc = ceil_div(p->L, LI);
+                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h<G, LI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
+                HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h<G, LI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs));
                 const HalfArgs A = half_args(p, x, nullptr, 0.f, nullptr);
-                HQS_CUDA_TRY(launch_pdl(k_fwd_rows_h<G, LN>, dim3(p->n, p->nchunk), ht, hs, st, A));
-                HQS_CUDA_TRY(launch_pdl(k_fwd_cols_h<G, LN>, dim3(G, p->nchunk), ht, hs, st, A));
+                HQS_CUDA_TRY(launch_pdl(k_fwd_rows_h<G, LI>, dim3(p->n, nc), ht, hs, st, A));
+                HQS_CUDA_TRY(launch_pdl(k_fwd_cols_h<G, LI>, dim3(G, nc), ht, hs, st, A));
                 HQS_CUDA_TRY(cudaGetLastError());
                 return HQS_OK;
             });
@@ -923,23 +930,32 @@ void fill_half_args(const hqs_plan_s* p, const float2* x, float2* xo, const floa
 
 // `count` plans with grid G = 2n and `lines` lines per CTA whose arguments are the
 // consecutive HalfArgs at d_tab: the forward's row and column passes (adjoint 0)
-// or the adjoint's column and row passes (adjoint 1), grid (lines, chunks, plans)
-int launch_half_group(int G, int n, int lines, int maxchunk, int count, const void* d_tab, int adjoint, float zc,
+// or the adjoint's column and row passes (adjoint 1), grid (lines, chunks, plans);
+// maxchunk, maxcoils: the largest chunk and coil count among them
+int launch_half_group(int G, int n, int lines, int maxchunk, int maxcoils, int count, const void* d_tab, int adjoint, float zc,
                       cudaStream_t st) {
     return dispatch_fft_size(G, [&]<int GG>() -> int {
         if constexpr (GG == 16 || GG == 320 || GG == 384) {
             return HQS_ERR_UNSUPPORTED;
         } else {
             return dispatch_half<GG>(lines, [&]<int LN>() -> int {
-                constexpr int th = half_threads<GG, LN>();
-                constexpr size_t sm = half_smem<GG, LN>();
                 const HalfArgs* tab = static_cast<const HalfArgs*>(d_tab);
-                auto first = adjoint ? k_adj_cols_h_b<GG, LN> : k_fwd_rows_h_b<GG, LN>;
-                auto second = adjoint ? k_adj_rows_h_b<GG, LN> : k_fwd_cols_h_b<GG, LN>;
-                HQS_CUDA_TRY(cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                HQS_CUDA_TRY(cudaFuncSetAttribute(second, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                HQS_CUDA_TRY(launch_pdl(first, dim3(adjoint ? GG : n, maxchunk, count), th, sm, st, tab, zc));
-                HQS_CUDA_TRY(launch_pdl(second, dim3(adjoint ? n : GG, maxchunk, count), th, sm, st, tab, zc));
+                if (adjoint) {
+                    constexpr int th = half_threads<GG, LN>();
+                    constexpr size_t sm = half_smem<GG, LN>();
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_cols_h_b<GG, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows_h_b<GG, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(launch_pdl(k_adj_cols_h_b<GG, LN>, dim3(GG, maxchunk, count), th, sm, st, tab, zc));
+                    HQS_CUDA_TRY(launch_pdl(k_adj_rows_h_b<GG, LN>, dim3(n, maxchunk, count), th, sm, st, tab, zc));
+                } else {
+                    constexpr int LI = half_free_lines<GG, LN>(), th = half_threads<GG, LI>();
+                    constexpr size_t sm = half_smem<GG, LI>();
+                    const int nc = ceil_div(maxcoils, LI);
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h_b<GG, LI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h_b<GG, LI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(launch_pdl(k_fwd_rows_h_b<GG, LI>, dim3(n, nc, count), th, sm, st, tab, zc));
+                    HQS_CUDA_TRY(launch_pdl(k_fwd_cols_h_b<GG, LI>, dim3(GG, nc, count), th, sm, st, tab, zc));
+                }
                 HQS_CUDA_TRY(cudaGetLastError());
                 return HQS_OK;
             });

@@ -128,7 +128,7 @@ bool plan_half_passes(const hqs_plan_s* p);
 int plan_half_lines(const hqs_plan_s* p);
 size_t half_args_bytes();
 void fill_half_args(const hqs_plan_s* p, const float2* x, float2* xo, const float2* z, void* dst);
-int launch_half_group(int G, int n, int lines, int maxchunk, int count, const void* d_tab, int adjoint, float zc,
+int launch_half_group(int G, int n, int lines, int maxchunk, int maxcoils, int count, const void* d_tab, int adjoint, float zc,
                       cudaStream_t s);
 int launch_spread(hqs_plan_s* p, const float2* y, cudaStream_t s);
 int launch_interp(hqs_plan_s* p, float2* y, cudaStream_t s);
