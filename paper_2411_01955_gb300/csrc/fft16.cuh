@@ -108,14 +108,18 @@ template <int LINES> HQS_DEV float2 swap_pair(float2 v) {
 // Every thread of the CTA calls it (the loads of threads without a line read the
 // caller's clamped line); no barrier inside.  ROT: output k times i^k (the image's
 // centring, i^(kk + 16 m) = i^kk, folded into the lane factors).
-template <int N, int LINES, bool ROT = false, class LD> HQS_DEV void fft16_head(float2* s, const Lane16& T, LD&& ld) {
+// fft16_head_load and fft16_head_do are its two halves, for callers that load ahead.
+template <int N, class LD> HQS_DEV void fft16_head_load(float2 (&o)[Fft16<N>::SUB][4], const Lane16& T, LD&& ld) {
     constexpr int R = Fft16<N>::R, SUB = Fft16<N>::SUB;
-    const bool odd = T.par != 0;
-    float2 o[SUB][4];
 #pragma unroll
     for (int b = 0; b < SUB; ++b)
 #pragma unroll
         for (int q = 0; q < 4; ++q) o[b][q] = ld(T.tp + 8 * b + R * (4 * T.par + q));
+}
+template <int N, int LINES, bool ROT = false>
+HQS_DEV void fft16_head_do(float2* s, const Lane16& T, const float2 (&o)[Fft16<N>::SUB][4]) {
+    constexpr int SUB = Fft16<N>::SUB;
+    const bool odd = T.par != 0;
     // lane factors of the sums and differences: w16^(par q) and (-1)^par w16^((2 + par) q)
     float2 ca[4], cb[4];
 #pragma unroll
@@ -155,6 +159,12 @@ template <int N, int LINES, bool ROT = false, class LD> HQS_DEV void fft16_head(
             dst[(4 * m + 2) * LINES] = f[m];
         }
     }
+}
+
+template <int N, int LINES, bool ROT = false, class LD> HQS_DEV void fft16_head(float2* s, const Lane16& T, LD&& ld) {
+    float2 o[Fft16<N>::SUB][4];
+    fft16_head_load<N>(o, T, ld);
+    fft16_head_do<N, LINES, ROT>(s, T, o);
 }
 
 // Inverse tail: the lane's 4 outputs of each of its SUB columns go to put(b, q, pos, v),
@@ -269,15 +279,17 @@ template <int CNT, int LINES, class F> HQS_DEV void lanes_sum_each(float2* w, in
 // Inverse tail of a row of coils (line = coil) with the weighted coil sum fused:
 // put(ix, sum_l conj(S_l[ix]) v_l[ix]) once for each pixel ix < n of the row.  sv: the
 // lane's maps at its 4 SUB outputs (index 4 b + q), zero for lanes without a coil.
-template <int N, int LINES, bool ROT = false, class PUT>
+// COILS < LINES: the lines are rows of COILS coils each, summed row by row.
+template <int N, int LINES, bool ROT = false, int COILS = LINES, class PUT>
 HQS_DEV void fft16_tail_coilsum(const float2* s, const Lane16& T, const float2* sv, PUT&& put) {
     constexpr int R = Fft16<N>::R, CNT = 4 * Fft16<N>::SUB;
     constexpr int C1 = CNT >= 16 ? 16 : CNT, C2 = CNT - C1;   // 16 + 4 at 640, 16 + 8 at 768
     float2 w[CNT];
     fft16_tail<N, LINES, ROT>(s, T, [&](int b, int q, int, float2 v) { w[4 * b + q] = cmulc(sv[4 * b + q], v); });
     auto out = [&](int j, float2 v) { put(T.tp + 8 * (j >> 2) + R * (4 * T.par + (j & 3)), v); };
-    lanes_sum_each<C1, LINES>(w, T.line, out);
-    if constexpr (C2 > 0) lanes_sum_each<C2, LINES>(w + C1, T.line, [&](int j, float2 v) { out(C1 + j, v); });
+    const int lane = T.line % COILS;
+    lanes_sum_each<C1, COILS>(w, lane, out);
+    if constexpr (C2 > 0) lanes_sum_each<C2, COILS>(w + C1, lane, [&](int j, float2 v) { out(C1 + j, v); });
 }
 
 }  // namespace hqs

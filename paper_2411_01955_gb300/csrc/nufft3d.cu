@@ -27,7 +27,7 @@
 #include <cstddef>
 #include <vector>
 
-#include "fft.cuh"
+#include "fft16.cuh"
 #include "plan.cuh"
 
 using namespace hqs;
@@ -43,7 +43,7 @@ struct Cg3 {
 };
 
 struct hqs_plan3d_s {
-    int device = 0;
+    int device = 0, nsm = 1;
     int n[3] = {0, 0, 0};     // nx, ny, nz
     int G[3] = {0, 0, 0};     // oversampled NUFFT grid (= 2n: also the Toeplitz grid)
     int L = 0, W = 0;
@@ -882,6 +882,232 @@ __global__ void k_pass3(LD ld, ST st, MID mid, int64_t nlines, int64_t B, const 
     }
 }
 
+// ---- passes over lines whose image (or block) is in the lower half, n = N/2 elements
+// Every operator pass is one of three: the forward transform of a line whose upper half
+// is zero, the inverse of which only the lower half is wanted, or the two with a factor
+// between them; the centred NUFFT passes are the same with the output (input) k rotated
+// by i^k (see nufft.cu).  They run on the two-stage transforms of fft16.cuh where those
+// cover the size (128 and 256 points here): one shared-memory round trip per transform.
+// Bound: instruction issue.
+// Their sizes fit 32 bits (at most 2^23 lines, strides of 2^23 elements): the line's
+// division and the element offsets are 32-bit operations, one wide multiply-add each (as
+// 64-bit ones they were a third of the passes' instructions).
+struct LinesI {
+    int64_t sA;
+    int sP;
+    LinesI(const Lines& g) : sA(g.sA), sP((int)g.sP) {}
+};
+struct LdRaw {
+    const float2* src;
+    LinesI g;
+    struct St { const float2* p; };
+    HQS_DEV St prepare(int a, int b) const { return {src + a * g.sA + b}; }
+    HQS_DEV float2 operator()(const St& t, int p) const { return t.p[(int64_t)p * g.sP]; }
+};
+// S_l x, row (z, y) of coil b
+struct LdCoilRow {
+    const float2* x;
+    const float2* S;
+    int nx, L;
+    struct St { const float2* xr; const float2* sr; };
+    HQS_DEV St prepare(int a, int b) const { return {x + (int64_t)a * nx, S + (int64_t)a * nx * L + b}; }
+    HQS_DEV float2 operator()(const St& t, int q) const { return cmul(t.sr[q * L], t.xr[q]); }
+};
+// S_l x / (phihat^3), row (z, y) of coil b
+struct LdImageRow {
+    const float2* x;
+    const float2* S;
+    const float *apx, *apy, *apz;
+    int nx, ny, L;
+    float scale;
+    struct St { const float2* xr; const float2* sr; float f; };
+    HQS_DEV St prepare(int a, int b) const {
+        const int z = a / ny, yy = a - z * ny;
+        return {x + (int64_t)a * nx, S + (int64_t)a * nx * L + b, scale * apz[z] * apy[yy]};
+    }
+    HQS_DEV float2 operator()(const St& t, int q) const { return cscale(cmul(t.sr[q * L], t.xr[q]), t.f * apx[q]); }
+};
+struct StRaw {
+    static constexpr int kCoils = 0;
+    float2* dst;
+    LinesI g;
+    struct St { float2* p; };
+    HQS_DEV St prepare(int a, int b) const { return {dst + a * g.sA + b}; }
+    HQS_DEV void put(const St& t, int pos, float2 v) const { t.p[(int64_t)pos * g.sP] = v; }
+};
+// conj(S) v per coil: P[(a*nx + o)*L + b]
+struct StCoilRow {
+    static constexpr int kCoils = 0;
+    float2* dst;
+    const float2* S;
+    int nx, L;
+    struct St { float2* d; const float2* s; };
+    HQS_DEV St prepare(int a, int b) const {
+        const int64_t e0 = (int64_t)a * nx * L + b;
+        return {dst + e0, S + e0};
+    }
+    HQS_DEV void put(const St& t, int o, float2 v) const { t.d[o * L] = cmulc(t.s[o * L], v); }
+};
+// The coil sum of StCoilSum on registers: CO coils (a power of two up to kLines), the
+// lines of a row adjacent lanes.
+template <int CO> struct StCoilSumRow {
+    static constexpr int kCoils = CO;
+    float2* out;
+    const float2* S;
+    const float2* z;
+    const float *apx, *apy, *apz;
+    int nx, ny;
+    float ca, cb;
+    struct St { const float2* s; float2* o; const float2* zr; float f; };
+    HQS_DEV St prepare(int a, int b) const {
+        float f = ca;
+        if (apx) {
+            const int zz = a / ny, yy = a - zz * ny;
+            f *= apz[zz] * apy[yy];
+        }
+        const int64_t e = (int64_t)a * nx;
+        return {S + e * CO + b, out + e, z ? z + e : nullptr, f};
+    }
+    HQS_DEV void put(const St& t, int o, float2 v) const {
+        float2 w = cscale(v, apx ? t.f * apx[o] : t.f);
+        if (t.zr) {
+            const float2 zv = t.zr[o];
+            w.x = fmaf(cb, zv.x, w.x);
+            w.y = fmaf(cb, zv.y, w.y);
+        }
+        t.o[o] = w;
+    }
+};
+
+// Khat between the z transforms: b = (ky*Tx + kx)*L + l
+struct MidKhatI {
+    const float* khat;
+    int plane, L;   // Ty * Tx
+    struct St { const float* k; };
+    HQS_DEV St prepare(int, int b) const { return {khat + (unsigned)b / (unsigned)L}; }
+    HQS_DEV float2 operator()(const St& t, int p, float2 v) const { return cmul_r(v, __ldg(t.k + (int64_t)p * plane)); }
+};
+
+enum { PASS_FWD = 0, PASS_INV = 1, PASS_PAIR = 2 };
+// CTAs per SM, and the persistent grid
+template <int N> constexpr int half3_ctas() { return N <= 128 ? 4 : 2; }
+// Persistent CTAs of 16 lines each round: a thread loads its share of the next round's
+// lines before it transforms this round's, so that loads are always in flight.  Two line
+// buffers in turn: a round's first writes need no barrier after the last one's reads.
+// 64^3 x 16 coils, 5 PCG iterations: 1632 us with 4 persistent CTAs per SM, 1708 with 3,
+// 1830 with one round per CTA, 1762 with the 8 x 16 stages of k_pass3.
+template <int N, int DIR, bool ROT, class LD, class ST, class MID>
+__global__ void __launch_bounds__(16 * kLines, half3_ctas<N>())
+    k_pass3h(LD ld, ST st, MID mid, int nlines, unsigned B, const float2* __restrict__ twg, const int* stop) {
+    if (stop && *stop) return;
+    extern __shared__ __align__(16) float2 smem[];
+    constexpr int R = Fft16<N>::R, SUB = Fft16<N>::SUB;
+    float2* tw = smem + 2 * N * kLines;
+    for (int c = threadIdx.x; c < N / 2; c += blockDim.x) cp_async16(tw + 2 * c, twg + 2 * c);
+    cp_async_wait_all();
+    const Lane16 T(kLines);
+    const int nround = (nlines + kLines - 1) / kLines;
+    float2 in[DIR == PASS_INV ? R / 4 : SUB][4];   // this round's loads, then the next one's
+    auto fetch = [&](int rd) {
+        // threads without a line read the round's first one and store nothing
+        const int l0 = rd * kLines, mine = l0 + T.line < nlines ? l0 + T.line : l0;
+        const int a = (int)((unsigned)mine / B);
+        const auto lds = ld.prepare(a, mine - a * (int)B);
+        if constexpr (DIR == PASS_INV) {
+#pragma unroll
+            for (int m = 0; m < R; ++m) in[m >> 2][m & 3] = ld(lds, T.t + 16 * m);
+        } else {
+            fft16_head_load<N>(in, T, [&](int q) { return ld(lds, q); });
+        }
+    };
+    int rd = blockIdx.x;
+    if (rd < nround) fetch(rd);
+    if constexpr (DIR == PASS_INV) __syncthreads();   // twiddles
+    for (int buf = 0; rd < nround; rd += gridDim.x, buf ^= 1) {
+        float2* s = smem + buf * N * kLines;
+        const int l0 = rd * kLines;
+        const bool act = l0 + T.line < nlines;
+        const int mine = act ? l0 + T.line : l0;
+        const int a = (int)((unsigned)mine / B), b = mine - a * (int)B;
+        const bool more = rd + (int)gridDim.x < nround;
+        float2 v[R];
+        if constexpr (DIR == PASS_INV) {
+#pragma unroll
+            for (int m = 0; m < R; ++m) v[m] = in[m >> 2][m & 3];
+            if (more) fetch(rd + (int)gridDim.x);
+        } else {
+            fft16_head_do<N, kLines, ROT && DIR == PASS_FWD>(s, T, in);
+            if (more) fetch(rd + (int)gridDim.x);
+            __syncthreads();
+            fft16_mid_read<N, kLines>(s, T, v);
+            fft16_mid_fwd<N>(T, tw, v);
+            if constexpr (DIR == PASS_FWD) {
+                const auto sts = st.prepare(a, b);
+                if (act) {
+#pragma unroll
+                    for (int m = 0; m < R; ++m) st.put(sts, T.t + 16 * m, v[m]);
+                }
+            } else {
+                const auto mds = mid.prepare(a, b);
+#pragma unroll
+                for (int m = 0; m < R; ++m) v[m] = mid(mds, T.t + 16 * m, v[m]);
+            }
+        }
+        if constexpr (DIR != PASS_FWD) {
+            fft16_mid_inv<N>(T, tw, v);
+            fft16_mid_write<N, kLines>(s, T, v);
+            const auto sts = st.prepare(a, b);
+            if constexpr (ST::kCoils > 0) {
+                float2 sv[4 * SUB];
+#pragma unroll
+                for (int k = 0; k < 4 * SUB; ++k) {
+                    sv[k] = sts.s[(T.tp + 8 * (k >> 2) + R * (4 * T.par + (k & 3))) * ST::kCoils];
+                    if (!act) sv[k] = make_float2(0.f, 0.f);
+                }
+                __syncthreads();
+                fft16_tail_coilsum<N, kLines, ROT, ST::kCoils>(s, T, sv, [&](int o, float2 w) {
+                    if (act) st.put(sts, o, w);
+                });
+            } else {
+                __syncthreads();
+                fft16_tail<N, kLines, ROT>(s, T, [&](int, int, int o, float2 w) {
+                    if (act) st.put(sts, o, w);
+                });
+            }
+        }
+    }
+}
+// whether the axis of N points takes these passes
+bool half3(int N) { return N == 128 || N == 256; }
+template <int DIR, bool ROT, class LD, class ST, class MID = NoMid>
+int run_half(const hqs_plan3d_s* p, int N, LD ld, ST st, int64_t nlines, int64_t B, cudaStream_t s, MID mid = MID{}) {
+    if (nlines <= 0) return HQS_OK;
+    const float2* tw = nullptr;
+    for (int i = 0; i < 9; ++i)
+        if (p->tw_sizes[i] == N) tw = p->tw + p->tw_offs[i] + N;
+    if (!tw || !half3(N)) return HQS_ERR_INVALID_ARG;
+    auto go = [&]<int NN>() -> int {
+        auto kern = k_pass3h<NN, DIR, ROT, LD, ST, MID>;
+        constexpr size_t sm = (size_t)(2 * NN * kLines + NN) * sizeof(float2);
+        HQS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        const int64_t nblk = std::min<int64_t>(ceil_div64(nlines, kLines), (int64_t)p->nsm * half3_ctas<NN>());
+        kern<<<(unsigned)nblk, 16 * kLines, sm, s>>>(ld, st, mid, (int)nlines, (unsigned)B, tw, p->stop);
+        HQS_CUDA_TRY(cudaGetLastError());
+        return HQS_OK;
+    };
+    return N == 128 ? go.template operator()<128>() : go.template operator()<256>();
+}
+// the last x pass with the coil sum on registers, for the coil counts that divide kLines
+template <bool ROT, class F> int with_coils(int L, F&& f) {
+    switch (L) {
+        case 1: return f.template operator()<1>();
+        case 2: return f.template operator()<2>();
+        case 4: return f.template operator()<4>();
+        case 8: return f.template operator()<8>();
+        default: return f.template operator()<16>();
+    }
+}
+
 template <class F> int dispatch3(int n, F&& f) { return dispatch_fft_size(n, std::forward<F>(f)); }
 
 const float2* tw3(const hqs_plan3d_s* p, int N) {
@@ -1499,18 +1725,28 @@ int fwd3(hqs_plan3d_s* p, const float2* x, float2* y, cudaStream_t s) {
     const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
     const int Gx = p->G[0], Gy = p->G[1], Gz = p->G[2], L = p->L;
     // x pass: [nz][ny][Gx][L] in bufA
+    if (half3(Gx)) {
+        TRY3((run_half<PASS_FWD, true>(p, Gx, LdImageRow{x, p->smaps, p->apod[0], p->apod[1], p->apod[2], nx, ny, L, p->scale},
+                                       StRaw{p->bufA, Lines{(int64_t)Gx * L, L}}, (int64_t)nz * ny * L, L, s)));
+    } else {
     TRY3((run_pass<false, false, false>(
         p, Gx, LdImageX{x, p->smaps, p->apod[0], p->apod[1], p->apod[2], nx, ny, Gx, L, p->scale},
         StLine{p->bufA, {(int64_t)Gx * L, L}, Gx, 0, Gx}, (int64_t)nz * ny * L, L, s)));
+    }
     // y pass: [nz][Gy][Gx][L] in bufB
-    const int64_t row = (int64_t)Gx * L;
-    TRY3((run_pass<false, false, false>(p, Gy, LdCentred{p->bufA, {(int64_t)ny * row, row}, ny, Gy},
-                                        StLine{p->bufB, {(int64_t)Gy * row, row}, Gy, 0, Gy},
-                                        (int64_t)nz * row, row, s)));
+    const int64_t row = (int64_t)Gx * L, plane = (int64_t)Gy * row;
+    const Lines ly{(int64_t)ny * row, row}, lY{plane, row}, lz{0, plane};
+    if (half3(Gy))
+        TRY3((run_half<PASS_FWD, true>(p, Gy, LdRaw{p->bufA, ly}, StRaw{p->bufB, lY}, (int64_t)nz * row, row, s)));
+    else
+        TRY3((run_pass<false, false, false>(p, Gy, LdCentred{p->bufA, ly, ny, Gy}, StLine{p->bufB, lY, Gy, 0, Gy},
+                                            (int64_t)nz * row, row, s)));
     // z pass: [Gz][Gy][Gx][L] in bufA
-    const int64_t plane = (int64_t)Gy * row;
-    TRY3((run_pass<false, false, false>(p, Gz, LdCentred{p->bufB, {0, plane}, nz, Gz},
-                                        StLine{p->bufA, {0, plane}, Gz, 0, Gz}, plane, plane, s)));
+    if (half3(Gz))
+        TRY3((run_half<PASS_FWD, true>(p, Gz, LdRaw{p->bufB, lz}, StRaw{p->bufA, lz}, plane, plane, s)));
+    else
+        TRY3((run_pass<false, false, false>(p, Gz, LdCentred{p->bufB, lz, nz, Gz}, StLine{p->bufA, lz, Gz, 0, Gz}, plane,
+                                            plane, s)));
     return interp3(p, p->bufA, y, s);
 }
 
@@ -1518,25 +1754,38 @@ int adj3(hqs_plan3d_s* p, const float2* y, float2* x, cudaStream_t s) {
     const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
     const int Gx = p->G[0], Gy = p->G[1], Gz = p->G[2], L = p->L;
     TRY3(spread3(p, y, p->bufA, s));
-    const int64_t row = (int64_t)Gx * L, plane = (int64_t)Gy * row;
+    const int64_t row = (int64_t)Gx * L, plane = (int64_t)Gy * row, nrow = (int64_t)nz * ny * L;
+    const Lines lx{row, L}, ly{(int64_t)ny * row, row}, lY{plane, row}, lz{0, plane};
     // z: [nz][Gy][Gx][L] in bufB
-    TRY3((run_pass<true, false, false>(p, Gz, LdLine{p->bufA, {0, plane}, Gz},
-                                       StLine{p->bufB, {0, plane}, nz, 1, Gz}, plane, plane, s)));
+    if (half3(Gz))
+        TRY3((run_half<PASS_INV, true>(p, Gz, LdRaw{p->bufA, lz}, StRaw{p->bufB, lz}, plane, plane, s)));
+    else
+        TRY3((run_pass<true, false, false>(p, Gz, LdLine{p->bufA, lz, Gz}, StLine{p->bufB, lz, nz, 1, Gz}, plane, plane, s)));
     // y: [nz][ny][Gx][L] in bufA
-    TRY3((run_pass<true, false, false>(p, Gy, LdLine{p->bufB, {plane, row}, Gy},
-                                       StLine{p->bufA, {(int64_t)ny * row, row}, ny, 1, Gy}, (int64_t)nz * row,
-                                       row, s)));
+    if (half3(Gy))
+        TRY3((run_half<PASS_INV, true>(p, Gy, LdRaw{p->bufB, lY}, StRaw{p->bufA, ly}, (int64_t)nz * row, row, s)));
+    else
+        TRY3((run_pass<true, false, false>(p, Gy, LdLine{p->bufB, lY, Gy}, StLine{p->bufA, ly, ny, 1, Gy}, (int64_t)nz * row,
+                                           row, s)));
     // x: conj(S_l) coil sum and deapodisation fused where the CTA holds whole rows,
     // else per coil into bufC and a separate sum
     if (kLines % L == 0) {
+        if (half3(Gx))
+            return with_coils<true>(L, [&]<int CO>() {
+                return run_half<PASS_INV, true>(p, Gx, LdRaw{p->bufA, lx},
+                                                StCoilSumRow<CO>{x, p->smaps, nullptr, p->apod[0], p->apod[1], p->apod[2], nx,
+                                                                 ny, p->scale, 0.f},
+                                                nrow, L, s);
+            });
         TRY3((run_pass<true, false, false>(
-            p, Gx, LdLine{p->bufA, {row, L}, Gx},
-            StCoilSum{x, p->smaps, nullptr, p->apod[0], p->apod[1], p->apod[2], nx, ny, L, 1, Gx, p->scale, 0.f},
-            (int64_t)nz * ny * L, L, s)));
+            p, Gx, LdLine{p->bufA, lx, Gx},
+            StCoilSum{x, p->smaps, nullptr, p->apod[0], p->apod[1], p->apod[2], nx, ny, L, 1, Gx, p->scale, 0.f}, nrow, L, s)));
         return HQS_OK;
     }
-    TRY3((run_pass<true, false, false>(p, Gx, LdLine{p->bufA, {row, L}, Gx},
-                                       StCoil{p->bufC, p->smaps, nx, L, 1, Gx}, (int64_t)nz * ny * L, L, s)));
+    if (half3(Gx))
+        TRY3((run_half<PASS_INV, true>(p, Gx, LdRaw{p->bufA, lx}, StCoilRow{p->bufC, p->smaps, nx, L}, nrow, L, s)));
+    else
+        TRY3((run_pass<true, false, false>(p, Gx, LdLine{p->bufA, lx, Gx}, StCoil{p->bufC, p->smaps, nx, L, 1, Gx}, nrow, L, s)));
     const int64_t nvox = (int64_t)nx * ny * nz;
     k_coil_sum3<<<vec_blocks(nvox), 256, 0, s>>>(p->bufC, L, nx, ny, nvox, p->apod[0], p->apod[1], p->apod[2],
                                                  p->scale, 0.f, nullptr, x, p->stop);
@@ -1548,30 +1797,46 @@ int adj3(hqs_plan3d_s* p, const float2* y, float2* x, cudaStream_t s) {
 int toep3(hqs_plan3d_s* p, const float2* x, float2* out, float ca, float cb, const float2* z, cudaStream_t s) {
     const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
     const int Tx = p->G[0], Ty = p->G[1], Tz = p->G[2], L = p->L;
-    const int64_t row = (int64_t)Tx * L, plane = (int64_t)Ty * row;
+    const int64_t row = (int64_t)Tx * L, plane = (int64_t)Ty * row, nrow = (int64_t)nz * ny * L, nyl = (int64_t)nz * row;
+    const Lines lx{row, L}, ly{(int64_t)ny * row, row}, lY{plane, row}, lz{0, plane};
     // x: [nz][ny][Tx][L] in bufA
-    TRY3((run_pass<false, true, false>(p, Tx, LdToepX{x, p->smaps, nx, L}, StLine{p->bufA, {row, L}, Tx, 0, Tx},
-                                       (int64_t)nz * ny * L, L, s)));
+    if (half3(Tx))
+        TRY3((run_half<PASS_FWD, false>(p, Tx, LdCoilRow{x, p->smaps, nx, L}, StRaw{p->bufA, lx}, nrow, L, s)));
+    else
+        TRY3((run_pass<false, true, false>(p, Tx, LdToepX{x, p->smaps, nx, L}, StLine{p->bufA, lx, Tx, 0, Tx}, nrow, L, s)));
     // y: [nz][Ty][Tx][L] in bufB
-    TRY3((run_pass<false, true, false>(p, Ty, LdLine{p->bufA, {(int64_t)ny * row, row}, ny},
-                                       StLine{p->bufB, {plane, row}, Ty, 0, Ty}, (int64_t)nz * row, row, s)));
+    if (half3(Ty))
+        TRY3((run_half<PASS_FWD, false>(p, Ty, LdRaw{p->bufA, ly}, StRaw{p->bufB, lY}, nyl, row, s)));
+    else
+        TRY3((run_pass<false, true, false>(p, Ty, LdLine{p->bufA, ly, ny}, StLine{p->bufB, lY, Ty, 0, Ty}, nyl, row, s)));
     // z: FFT, Khat, IFFT, rows z < nz, in place in bufB
-    TRY3((run_pass<true, true, true>(p, Tz, LdLine{p->bufB, {0, plane}, nz}, StLine{p->bufB, {0, plane}, nz, 0, Tz},
-                                     plane, plane, s, MidKhat{p->khat, (int64_t)Ty * Tx, L})));
+    const MidKhat mk{p->khat, (int64_t)Ty * Tx, L};
+    if (half3(Tz))
+        TRY3((run_half<PASS_PAIR, false>(p, Tz, LdRaw{p->bufB, lz}, StRaw{p->bufB, lz}, plane, plane, s, MidKhatI{p->khat, Ty * Tx, L})));
+    else
+        TRY3((run_pass<true, true, true>(p, Tz, LdLine{p->bufB, lz, nz}, StLine{p->bufB, lz, nz, 0, Tz}, plane, plane, s, mk)));
     // y inverse: [nz][ny][Tx][L] in bufA
-    TRY3((run_pass<true, false, true>(p, Ty, LdLine{p->bufB, {plane, row}, Ty},
-                                      StLine{p->bufA, {(int64_t)ny * row, row}, ny, 0, Ty}, (int64_t)nz * row, row,
-                                      s)));
+    if (half3(Ty))
+        TRY3((run_half<PASS_INV, false>(p, Ty, LdRaw{p->bufB, lY}, StRaw{p->bufA, ly}, nyl, row, s)));
+    else
+        TRY3((run_pass<true, false, true>(p, Ty, LdLine{p->bufB, lY, Ty}, StLine{p->bufA, ly, ny, 0, Ty}, nyl, row, s)));
     // x inverse with the conj(S_l) coil sum fused (whole rows per CTA), else per coil in bufC + sum
     if (kLines % L == 0) {
+        if (half3(Tx))
+            return with_coils<false>(L, [&]<int CO>() {
+                return run_half<PASS_INV, false>(
+                    p, Tx, LdRaw{p->bufA, lx}, StCoilSumRow<CO>{out, p->smaps, z, nullptr, nullptr, nullptr, nx, ny, ca, cb},
+                    nrow, L, s);
+            });
         TRY3((run_pass<true, false, true>(
-            p, Tx, LdLine{p->bufA, {row, L}, Tx},
-            StCoilSum{out, p->smaps, z, nullptr, nullptr, nullptr, nx, ny, L, 0, Tx, ca, cb},
-            (int64_t)nz * ny * L, L, s)));
+            p, Tx, LdLine{p->bufA, lx, Tx},
+            StCoilSum{out, p->smaps, z, nullptr, nullptr, nullptr, nx, ny, L, 0, Tx, ca, cb}, nrow, L, s)));
         return HQS_OK;
     }
-    TRY3((run_pass<true, false, true>(p, Tx, LdLine{p->bufA, {row, L}, Tx}, StCoil{p->bufC, p->smaps, nx, L, 0, Tx},
-                                      (int64_t)nz * ny * L, L, s)));
+    if (half3(Tx))
+        TRY3((run_half<PASS_INV, false>(p, Tx, LdRaw{p->bufA, lx}, StCoilRow{p->bufC, p->smaps, nx, L}, nrow, L, s)));
+    else
+        TRY3((run_pass<true, false, true>(p, Tx, LdLine{p->bufA, lx, Tx}, StCoil{p->bufC, p->smaps, nx, L, 0, Tx}, nrow, L, s)));
     const int64_t nvox = (int64_t)nx * ny * nz;
     k_coil_sum3<<<vec_blocks(nvox), 256, 0, s>>>(p->bufC, L, nx, ny, nvox, nullptr, nullptr, nullptr, ca, cb, z,
                                                  out, p->stop);
@@ -1737,7 +2002,7 @@ int plan3d_build(hqs_plan3d_s* p, const float* traj, const float2* smaps_user, c
                 if (!seen) {
                     p->tw_sizes[ns] = N;
                     p->tw_offs[ns] = total;
-                    total += N;
+                    total += 2 * N;
                     ++ns;
                 }
             }
@@ -1747,6 +2012,10 @@ int plan3d_build(hqs_plan3d_s* p, const float* traj, const float2* smaps_user, c
                 const double ang = -2.0 * M_PI * (double)m / (double)p->tw_sizes[k];
                 h[p->tw_offs[k] + m] = make_float2((float)cos(ang), (float)sin(ang));
             }
+        // the second table of each size: w_N^(i kk) at i * 16 + kk, for the two-stage passes
+        for (int k = 0; k < ns; ++k)
+            for (int m = 0; m < p->tw_sizes[k]; ++m)
+                h[p->tw_offs[k] + p->tw_sizes[k] + m] = h[p->tw_offs[k] + (m / 16) * (m % 16)];
         TRY3(alloc3(p, &p->tw, (size_t)total));
         HQS_CUDA_TRY(cudaMemcpyAsync(p->tw, h.data(), total * sizeof(float2), cudaMemcpyHostToDevice, s));
         HQS_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1794,6 +2063,7 @@ extern "C" int hqs_plan3d_create(hqs_plan3d* out, const float* traj, int64_t M, 
     auto* p = new (std::nothrow) hqs_plan3d_s;
     if (!p) return HQS_ERR_OOM;
     cudaGetDevice(&p->device);
+    cudaDeviceGetAttribute(&p->nsm, cudaDevAttrMultiProcessorCount, p->device);
     p->n[0] = nx;
     p->n[1] = ny;
     p->n[2] = nz;
