@@ -368,22 +368,6 @@ extern "C" int hqs_learned_precond_apply(hqs_plan p, float a, float b, const hqs
 // is a small stand-in built from the same convolution kernels).
 namespace {
 
-__global__ void k_denoise_split(const float2* __restrict__ v, int count, float inv_sigma, float* __restrict__ planar) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-        const float2 a = v[e];
-        planar[e] = a.x * inv_sigma;
-        planar[count + e] = a.y * inv_sigma;
-    }
-}
-
-__global__ void k_denoise_combine(const float2* __restrict__ v, const float* __restrict__ noise, int count,
-                                  float sigma, float2* __restrict__ out) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-        const float2 a = v[e];
-        out[e] = make_float2(fmaf(-sigma, noise[e], a.x), fmaf(-sigma, noise[count + e], a.y));
-    }
-}
-
 __global__ void k_copy_c64(const float2* __restrict__ a, float2* __restrict__ b, int count) {
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) b[e] = a[e];
 }
@@ -404,12 +388,7 @@ extern "C" int hqs_net_denoise(void* user, const hqs_c64* in, hqs_c64* out, int 
         HQS_CUDA_TRY(cudaGetLastError());
         return HQS_OK;
     }
-    HQS_TRY_RC(ensure_net_buffers(net, std::max(ny, nx)));
-    float* x = net->planar;
-    float* noise = net->planar + 2 * (size_t)count;
-    k_denoise_split<<<nb, 256, 0, st>>>(v, count, 1.f / sigma, x);
-    HQS_TRY_RC(net_forward(net, x, noise, 1, ny, nx, st));
-    k_denoise_combine<<<nb, 256, 0, st>>>(v, noise, count, sigma, o);
+    HQS_TRY_RC(net_denoise_run(net, v, o, ny, nx, sigma, st));
     HQS_CUDA_TRY(cudaGetLastError());
     return HQS_OK;
 }

@@ -32,4 +32,6 @@ struct hqs_net_s {
 
 int net_num_params();
 int net_forward(hqs_net_s* net, const float* x, float* out, int N, int H, int Wd, cudaStream_t st);
+// out = v - sigma net(v / sigma) on complex H x Wd images, sigma > 0; out may be v
+int net_denoise_run(hqs_net_s* net, const float2* v, float2* out, int H, int Wd, float sigma, cudaStream_t st);
 int net_check(hqs_net_s* net, cudaStream_t st);
