@@ -49,7 +49,8 @@ struct hqs_plan_s {
     int q_rows = 8;     // lines per CTA in the single-image FFT passes
     int fused_grid = 0; // cap on the persistent solver's CTAs (0: occupancy limit)
     bool nufft_only = false; // internal plans that only grid (no Toeplitz kernel, density symbol zero)
-    int pc_lines = 4;   // preconditioner lines per item in the persistent solver (1..16)
+    int pc_lines = 2;   // preconditioner lines per item in the persistent solver (1..16; one 320^2 slice,
+                        // 304 CTAs: 1, 2, 4 lines give a step of 5 iterations 781, 700, 717 us)
     int debug_barrier_skip = 0;  // test hook for the next persistent solve (HQS_TUNE_DEBUG_BARRIER_SKIP)
 
     // constant tables and plan data (device)
