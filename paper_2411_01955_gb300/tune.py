@@ -3,7 +3,7 @@
 Three knobs change how work is cut into launches, never what is computed
 (beyond float rounding order of atomics and sums):
 
-  spread_tile  edge of the shared-memory spreading tile of the adjoint (8, 16, 32)
+  spread_tile  edge of the bins the points are sorted in (8, 16, 32)
   pc_lines     rows/columns of the preconditioner FFT per work item of the
                persistent solve (1..16)
   fused_grid   cap on the persistent solve's CTAs (0 = every resident CTA)
@@ -30,7 +30,7 @@ FUSED_GRIDS = (0, 152, 228)
 @dataclass
 class Tuning:
     spread_tile: int = 16
-    pc_lines: int = 4
+    pc_lines: int = 2
     fused_grid: int = 0
 
 
