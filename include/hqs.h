@@ -297,8 +297,8 @@ HQS_API int hqs_learned_precond_apply(hqs_plan plan, float a, float b, const hqs
  * the built-in Gaussian smoothing with `user` pointing to hqs_gauss_params
  * (NULL: kappa 1.5, sigma0 = sigma[0]).  Resuming from k0 with x_{k0} gives
  * the same x_K as an uninterrupted run: the Toeplitz/CG iterations have no
- * atomics and fixed-order reductions; only A^H y (float atomics in the
- * spreading) may differ in the last bits between calls.
+ * atomics and fixed-order reductions, and A^H y is summed in an order fixed
+ * per plan; two plans of one trajectory may differ in its last bits.
  * The loop enqueues on `stream` and
  * calls the callback from the calling thread between outer iterations; each
  * DC step synchronises `stream` once per CG iteration (plain mode). */
@@ -379,9 +379,9 @@ HQS_API int hqs_batch_toeplitz_normal(hqs_batch batch, const hqs_c64* const* x, 
 /* Batched NUFFT operators (Eq. (1) and its adjoint, the same gridding as
  * hqs_forward / hqs_adjoint_axpy): y[i] = A_i x[i], and x[i] = A_i^H y[i] +
  * zc z[i] (z NULL, or z[i] NULL: no axpy term), for every slice i.  The
- * slices whose grid is 2n with 16-coil chunks run their row and column FFT
- * passes together, one launch per pass and grid size; spreading,
- * interpolation and the other slices' passes run per slice.  y[i]: (L_i, M_i),
+ * slices whose grid is 2n (at any coil count from 128 points on, with full
+ * 16-coil chunks below) run their row and column FFT passes together, one
+ * launch per pass, grid size and lines per CTA; spreading, interpolation and the other slices' passes run per slice.  y[i]: (L_i, M_i),
  * x[i], z[i]: (n_i, n_i), device complex64, caller-owned.  Enqueued on
  * `stream`; synchronises it first when the image pointers differ from the last
  * call.  Uses the plans' workspaces: calls on one batch (and on its plans) run
