@@ -559,6 +559,13 @@ int net_num_params() { return (int)layer_offset(4); }
 static int net_reserve(hqs_net_s* net, int N, int H, int Wd) {
     const size_t pix = (size_t)N * H * Wd;
     const size_t tiles = (size_t)N * ceil_div(H, CONV_TILE) * ceil_div(Wd, CONV_TILE);
+    if (N > net->cap_n) {   // one loss per sample, however small the samples
+        cudaFree(net->loss_n);
+        net->loss_n = nullptr;
+        net->cap_n = 0;
+        HQS_CUDA_TRY(cudaMalloc(&net->loss_n, (size_t)N * sizeof(double)));
+        net->cap_n = N;
+    }
     if (pix <= net->cap_pix && tiles <= net->cap_tiles) return HQS_OK;
     for (float*& b : net->act) {
         cudaFree(b);
@@ -567,19 +574,15 @@ static int net_reserve(hqs_net_s* net, int N, int H, int Wd) {
     cudaFree(net->dbuf[0]);
     cudaFree(net->dbuf[1]);
     cudaFree(net->part);
-    cudaFree(net->loss_n);
     net->dbuf[0] = net->dbuf[1] = net->part = nullptr;
-    net->loss_n = nullptr;
     for (int l = 0; l < 3; ++l) HQS_CUDA_TRY(cudaMalloc(&net->act[l], pix * HQS_NET_HIDDEN * sizeof(float)));
     HQS_CUDA_TRY(cudaMalloc(&net->act[3], pix * 2 * sizeof(float)));
     HQS_CUDA_TRY(cudaMalloc(&net->dbuf[0], pix * HQS_NET_HIDDEN * sizeof(float)));
     HQS_CUDA_TRY(cudaMalloc(&net->dbuf[1], pix * HQS_NET_HIDDEN * sizeof(float)));
     const size_t maxw = (size_t)HQS_NET_HIDDEN * HQS_NET_HIDDEN * 9 + HQS_NET_HIDDEN;
     HQS_CUDA_TRY(cudaMalloc(&net->part, tiles * maxw * sizeof(float)));
-    HQS_CUDA_TRY(cudaMalloc(&net->loss_n, (size_t)N * sizeof(double)));
     net->cap_pix = pix;
     net->cap_tiles = tiles;
-    net->cap_n = N;
     return HQS_OK;
 }
 

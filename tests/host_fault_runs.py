@@ -1,0 +1,52 @@
+"""Scenarios of tests/test_host_faults.py, each run in a process of its own:
+
+    python tests/host_fault_runs.py <stand-in .so> <library .so> <scenario>
+
+The stand-in replaces the CUDA runtime (fake_cudart.cpp), so device pointers are host memory
+and kernels do nothing; what is checked is the host code around them.
+"""
+import ctypes as C
+import sys
+
+OOM = -2
+VP, LONG = C.c_void_p, C.c_long
+
+
+class Fake:
+    def __init__(self, path):
+        self.lib = C.CDLL(path, mode=C.RTLD_GLOBAL)
+        for name, ret in [("fake_calls", LONG), ("fake_bad", LONG), ("fake_live", LONG), ("fake_bytes", C.c_size_t),
+                          ("fake_hash", C.c_ulonglong), ("fake_launches", C.c_char_p)]:
+            getattr(self.lib, name).restype = ret
+        self.lib.fake_fail_call.argtypes = self.lib.fake_fail_malloc.argtypes = [LONG]
+
+    def __getattr__(self, name):
+        return getattr(self.lib, "fake_" + name)
+
+    def device(self, nbytes):
+        p = VP()
+        assert self.lib.cudaMalloc(C.byref(p), C.c_size_t(nbytes)) == 0
+        return p
+
+
+def net_scratch_holds_the_samples(fake, hqs):
+    """One large image first, then many small ones with fewer pixels and tiles in all: the
+    per-sample losses need room for the second count."""
+    net = VP()
+    assert hqs.hqs_net_create(C.byref(net)) == 0
+    x = fake.device(2 * 256 * 256 * 4)
+    loss = C.c_double()
+    lr = C.c_float(1e-3)
+    assert hqs.hqs_net_train_step(net, x, x, 1, 256, 256, lr, C.byref(loss), None) == 0
+    assert hqs.hqs_net_train_step(net, x, x, 128, 4, 4, lr, C.byref(loss), None) == 0
+    assert fake.bad() == 0, "per-sample losses copied from beyond their buffer"
+    hqs.hqs_net_destroy(net)
+
+
+
+if __name__ == "__main__":
+    fake = Fake(sys.argv[1])
+    hqs = C.CDLL(sys.argv[2])
+    hqs.hqs_net_destroy.restype = hqs.hqs_plan_destroy.restype = hqs.hqs_plan3d_destroy.restype = None
+    globals()[sys.argv[3]](fake, hqs)
+    assert fake.bad() == 0
