@@ -567,6 +567,7 @@ static int net_reserve(hqs_net_s* net, int N, int H, int Wd) {
         net->cap_n = N;
     }
     if (pix <= net->cap_pix && tiles <= net->cap_tiles) return HQS_OK;
+    net->cap_pix = net->cap_tiles = 0;   // until every buffer is there again
     for (float*& b : net->act) {
         cudaFree(b);
         b = nullptr;

@@ -205,6 +205,7 @@ double fixed_sum(const std::vector<double>& h, int off, int n) {
 
 static int ensure_net_buffers(hqs_net_s* net, int n) {
     if (net->cap_img >= n) return HQS_OK;
+    net->cap_img = 0;   // until every buffer is there again
     cudaFree(net->zdc);
     cudaFree(net->planar);
     cudaFree(net->scal);

@@ -43,6 +43,54 @@ def net_scratch_holds_the_samples(fake, hqs):
     hqs.hqs_net_destroy(net)
 
 
+def net_scratch_after_failed_growth(fake, hqs):
+    """A growth that runs out of memory leaves no buffer behind; the next, smaller call has
+    to allocate what it needs (not launch on the pointers that were freed)."""
+    for k in range(1, 8):
+        net = VP()
+        assert hqs.hqs_net_create(C.byref(net)) == 0
+        x = fake.device(2 * 128 * 128 * 4)
+        base = fake.bytes()
+        assert hqs.hqs_net_forward(net, x, x, 1, 64, 64, None) == 0
+        fake.fail_malloc(k)
+        assert hqs.hqs_net_forward(net, x, x, 1, 128, 128, None) == OOM
+        fake.fail_malloc(-1)
+        fake.lib.cudaGetLastError()
+        assert hqs.hqs_net_forward(net, x, x, 1, 32, 32, None) == 0
+        # activations and gradients: 5 x 32 + 2 planes of the image
+        assert fake.bytes() - base >= (5 * 32 + 2) * 32 * 32 * 4, k
+        hqs.hqs_net_destroy(net)
+
+
+def make_plan(fake, hqs, n, M=300, L=4, W=4):
+    plan = VP()
+    traj, smaps = fake.device(M * 8), fake.device(L * n * n * 8)
+    assert hqs.hqs_plan_create(C.byref(plan), traj, C.c_int64(M), n, n, L, smaps, W, C.c_float(2.0), None) == 0
+    return plan
+
+
+def learned_scratch_after_failed_growth(fake, hqs):
+    """The same for the learned preconditioner's image buffers."""
+    small, mid, big = (make_plan(fake, hqs, n) for n in (32, 64, 128))
+    r = fake.device(128 * 128 * 8)
+    one = C.c_float(1.0)
+    for k in range(1, 4):
+        net = VP()
+        assert hqs.hqs_net_create(C.byref(net)) == 0
+        for p in (small, mid, big):
+            assert hqs.hqs_plan_set_net(p, net) == 0
+        # the network's own scratch at its largest, so that only the image buffers grow
+        assert hqs.hqs_net_forward(net, r, r, 1, 128, 128, None) == 0
+        base = fake.bytes()
+        assert hqs.hqs_learned_precond_apply(mid, one, one, r, r, None) == 0
+        fake.fail_malloc(k)
+        assert hqs.hqs_learned_precond_apply(big, one, one, r, r, None) == OOM
+        fake.fail_malloc(-1)
+        fake.lib.cudaGetLastError()
+        assert hqs.hqs_learned_precond_apply(small, one, one, r, r, None) == 0
+        assert fake.bytes() - base >= (2 + 4) * 32 * 32 * 4, k
+        hqs.hqs_net_destroy(net)
+
 
 if __name__ == "__main__":
     fake = Fake(sys.argv[1])

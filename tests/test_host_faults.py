@@ -27,3 +27,8 @@ def run(libs, scenario):
 
 def test_net_scratch_holds_the_samples(libs):
     run(libs, "net_scratch_holds_the_samples")
+
+
+@pytest.mark.parametrize("what", ["net", "learned"])
+def test_scratch_after_failed_growth(libs, what):
+    run(libs, what + "_scratch_after_failed_growth")
