@@ -1025,6 +1025,7 @@ extern "C" int hqs_batch_create(hqs_batch* out, hqs_plan* plans, int n, int max_
     b->plans.assign(plans, plans + n);
     auto fail = [&](int rc) {
         batch_free(b);
+        cudaGetLastError();   // see hqs_note_cuda_error
         return rc;
     };
     // slice table and item lists
@@ -1043,7 +1044,7 @@ extern "C" int hqs_batch_create(hqs_batch* out, hqs_plan* plans, int n, int max_
         S.A.chunk = nullptr;
         if (nch > 1) {
             float2* cb = nullptr;
-            if (cudaMalloc(&cb, (size_t)nch * p->n * p->n * sizeof(float2))) return fail(HQS_ERR_OOM);
+            if (hqs_malloc(&cb, (size_t)nch * p->n * p->n * sizeof(float2))) return fail(HQS_ERR_OOM);
             b->chunks.push_back(cb);
             S.A.chunk = cb;
         }
@@ -1074,21 +1075,21 @@ extern "C" int hqs_batch_create(hqs_batch* out, hqs_plan* plans, int n, int max_
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device) || per_sm < 1)
         return fail(HQS_ERR_CUDA);
     b->grid = per_sm * nsm;
-    if (cudaMalloc(&b->d_slices, n * sizeof(BatchSlice)) || cudaMalloc(&b->d_off, off.size() * sizeof(int)) ||
-        cudaMalloc(&b->d_mu, max_outer * sizeof(float)) ||
-        cudaMalloc(&b->d_taps, (size_t)max_outer * (2 * HQS_BATCH_MAXR + 1) * sizeof(float)) ||
-        cudaMalloc(&b->d_radius, max_outer * sizeof(int)) ||
-        cudaMalloc(&b->d_part, (size_t)BS_N * n * b->grid * sizeof(double)) ||
-        cudaMalloc(&b->d_res, n * sizeof(double)) || cudaMalloc(&b->d_bar, 2 * sizeof(unsigned)) ||
-        cudaMalloc(&b->d_err, sizeof(unsigned)) || cudaMallocHost(&b->h_mu, max_outer * sizeof(float)) ||
+    if (hqs_malloc(&b->d_slices, n * sizeof(BatchSlice)) || hqs_malloc(&b->d_off, off.size() * sizeof(int)) ||
+        hqs_malloc(&b->d_mu, max_outer * sizeof(float)) ||
+        hqs_malloc(&b->d_taps, (size_t)max_outer * (2 * HQS_BATCH_MAXR + 1) * sizeof(float)) ||
+        hqs_malloc(&b->d_radius, max_outer * sizeof(int)) ||
+        hqs_malloc(&b->d_part, (size_t)BS_N * n * b->grid * sizeof(double)) ||
+        hqs_malloc(&b->d_res, n * sizeof(double)) || hqs_malloc(&b->d_bar, 2 * sizeof(unsigned)) ||
+        hqs_malloc(&b->d_err, sizeof(unsigned)) || cudaMallocHost(&b->h_mu, max_outer * sizeof(float)) ||
         cudaMallocHost(&b->h_taps, (size_t)max_outer * (2 * HQS_BATCH_MAXR + 1) * sizeof(float)) ||
         cudaMallocHost(&b->h_radius, max_outer * sizeof(int)) ||
         cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking))
         return fail(HQS_ERR_OOM);
     b->dc_host = hs;
     b->ap_host = hs;
-    if (cudaMalloc(&b->d_slices_dc, n * sizeof(BatchSlice)) || cudaMalloc(&b->d_iters, n * sizeof(int)) ||
-        cudaMalloc(&b->d_status, n * sizeof(int)) || cudaMalloc(&b->d_slices_ap, n * sizeof(BatchSlice)))
+    if (hqs_malloc(&b->d_slices_dc, n * sizeof(BatchSlice)) || hqs_malloc(&b->d_iters, n * sizeof(int)) ||
+        hqs_malloc(&b->d_status, n * sizeof(int)) || hqs_malloc(&b->d_slices_ap, n * sizeof(BatchSlice)))
         return fail(HQS_ERR_OOM);
     if (cudaMemcpy(b->d_slices, hs.data(), n * sizeof(BatchSlice), cudaMemcpyHostToDevice) ||
         cudaMemcpy(b->d_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice))

@@ -106,7 +106,15 @@ template <bool INV> HQS_DEV float2 mul_mi(float2 a) {
         }                                                    \
     } while (0)
 
+// Keeps the message for hqs_status_string and clears the runtime's own record of the
+// error: left there, an allocation that failed would be taken for the failure of the next
+// launch that is checked.
 void hqs_note_cuda_error(cudaError_t e, const char* what, const char* file, int line);
+template <class T> static inline cudaError_t hqs_malloc(T** p, size_t bytes) {
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+    if (e != cudaSuccess) hqs_note_cuda_error(e, "cudaMalloc", __FILE__, __LINE__);
+    return e;
+}
 
 // Device error word bits (per plan), read back at sync points.
 #define HQS_DEVERR_TIMEOUT   1u

@@ -1498,14 +1498,14 @@ int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], 
         cudaFree(counts);
     };
     const int64_t Mp = std::max<int64_t>(M, 1);
-    if (cudaMalloc(&rawi, Mp * sizeof(int4)) || cudaMalloc(&rawd, Mp * sizeof(float4)) ||
-        cudaMalloc(&bin, Mp * sizeof(int)) || cudaMalloc(&counts, nbins * sizeof(int))) {
+    if (hqs_malloc(&rawi, Mp * sizeof(int4)) || hqs_malloc(&rawd, Mp * sizeof(float4)) ||
+        hqs_malloc(&bin, Mp * sizeof(int)) || hqs_malloc(&counts, nbins * sizeof(int))) {
         cleanup();
         return HQS_ERR_OOM;
     }
     int rc = HQS_OK;
     do {
-        if (cudaMalloc(&out->pti, Mp * sizeof(int4)) || cudaMalloc(&out->ptd, Mp * sizeof(float4))) {
+        if (hqs_malloc(&out->pti, Mp * sizeof(int4)) || hqs_malloc(&out->ptd, Mp * sizeof(float4))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -1528,7 +1528,7 @@ int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], 
         }
         offs[nbins] = acc;
         out->nsub = (int)subs.size();
-        if (cudaMalloc(&out->subs, std::max<size_t>(subs.size(), 1) * sizeof(int4))) {
+        if (hqs_malloc(&out->subs, std::max<size_t>(subs.size(), 1) * sizeof(int4))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -1594,8 +1594,8 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
     };
     int rc = HQS_OK;
     do {
-        if (cudaMalloc(&ptd, Mp * sizeof(float4)) || cudaMalloc(&ucnt, nbins * sizeof(int)) ||
-            cudaMalloc(&tcnt, nbins * sizeof(int)) || cudaMalloc(&binoff, (nbins + 1) * sizeof(int))) {
+        if (hqs_malloc(&ptd, Mp * sizeof(float4)) || hqs_malloc(&ucnt, nbins * sizeof(int)) ||
+            hqs_malloc(&tcnt, nbins * sizeof(int)) || hqs_malloc(&binoff, (nbins + 1) * sizeof(int))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -1907,7 +1907,7 @@ int build_khat(hqs_plan3d_s* p, const float* traj, cudaStream_t s) {
     do {
         const size_t g4 = (size_t)G4[0] * G4[1] * G4[2];
         const size_t m2 = (size_t)T[2] * G4[1] * G4[0];   // [2nz][4ny][4nx]
-        if (cudaMalloc(&grid, g4 * sizeof(float2)) || cudaMalloc(&mid, m2 * sizeof(float2))) {
+        if (hqs_malloc(&grid, g4 * sizeof(float2)) || hqs_malloc(&mid, m2 * sizeof(float2))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -1918,8 +1918,11 @@ int build_khat(hqs_plan3d_s* p, const float* traj, cudaStream_t s) {
                 const int d = q < hn ? q : q - T[a];
                 h[q] = (float)(1.0 / kb_phihat3((double)d / G4[a], Wk, bk));
             }
-            if (cudaMalloc(&ap[a], T[a] * sizeof(float)) ||
-                cudaMemcpyAsync(ap[a], h.data(), T[a] * sizeof(float), cudaMemcpyHostToDevice, s) ||
+            if (hqs_malloc(&ap[a], T[a] * sizeof(float))) {
+                rc = HQS_ERR_OOM;
+                break;
+            }
+            if (cudaMemcpyAsync(ap[a], h.data(), T[a] * sizeof(float), cudaMemcpyHostToDevice, s) ||
                 cudaStreamSynchronize(s)) {
                 rc = HQS_ERR_CUDA;
                 break;

@@ -20,6 +20,7 @@ static thread_local char g_last_cuda_error[256] = {0};
 void hqs_note_cuda_error(cudaError_t e, const char* what, const char* file, int line) {
     snprintf(g_last_cuda_error, sizeof(g_last_cuda_error), "%s:%d %s -> %s", file, line, what,
              cudaGetErrorString(e));
+    cudaGetLastError();
     if (getenv("HQS_VERBOSE")) fprintf(stderr, "[hqs] %s\n", g_last_cuda_error);
 }
 
@@ -415,10 +416,10 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
     int rc = HQS_OK;
     do {
         const int Mp = std::max(M, 1);
-        if (cudaMalloc(&raw, Mp * sizeof(int4)) || cudaMalloc(&bin, Mp * sizeof(int)) ||
-            cudaMalloc(&counts, nbins * sizeof(int)) || cudaMalloc(&phase, Mp * sizeof(float4)) ||
-            cudaMalloc(&cbuf, (size_t)n2 * n2 * sizeof(float2)) ||
-            cudaMalloc(&chan, (size_t)n * n * sizeof(float2))) {
+        if (hqs_malloc(&raw, Mp * sizeof(int4)) || hqs_malloc(&bin, Mp * sizeof(int)) ||
+            hqs_malloc(&counts, nbins * sizeof(int)) || hqs_malloc(&phase, Mp * sizeof(float4)) ||
+            hqs_malloc(&cbuf, (size_t)n2 * n2 * sizeof(float2)) ||
+            hqs_malloc(&chan, (size_t)n * n * sizeof(float2))) {
             rc = HQS_ERR_OOM;
             break;
         }
@@ -551,9 +552,9 @@ extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
     const int old_tile = p->tile, old_nbx = p->nbx;
     do {
         const int Mp = std::max(M, 1);
-        if (cudaMalloc(&bin, Mp * sizeof(int)) || cudaMalloc(&counts, nbins * sizeof(int)) ||
-            cudaMalloc(&perm2, Mp * sizeof(int)) || cudaMalloc(&pts2, Mp * sizeof(int4)) ||
-            cudaMalloc(&cursor, (size_t)(p->G / 8) * (p->G / 8) * sizeof(int))) {
+        if (hqs_malloc(&bin, Mp * sizeof(int)) || hqs_malloc(&counts, nbins * sizeof(int)) ||
+            hqs_malloc(&perm2, Mp * sizeof(int)) || hqs_malloc(&pts2, Mp * sizeof(int4)) ||
+            hqs_malloc(&cursor, (size_t)(p->G / 8) * (p->G / 8) * sizeof(int))) {
             rc = HQS_ERR_OOM;
             break;
         }

@@ -75,8 +75,8 @@ extern "C" int hqs_estimate_smaps(const float* traj, int64_t M, const hqs_c64* y
     hqs_plan plan = nullptr;
     int rc = HQS_OK;
     do {
-        if (cudaMalloc(&ones, (size_t)count * sizeof(float2)) || cudaMalloc(&yw, (size_t)M * sizeof(float2)) ||
-            cudaMalloc(&rss, (size_t)count * sizeof(float)) || cudaMalloc(&amax, sizeof(unsigned))) {
+        if (hqs_malloc(&ones, (size_t)count * sizeof(float2)) || hqs_malloc(&yw, (size_t)M * sizeof(float2)) ||
+            hqs_malloc(&rss, (size_t)count * sizeof(float)) || hqs_malloc(&amax, sizeof(unsigned))) {
             rc = HQS_ERR_OOM;
             break;
         }

@@ -20,7 +20,7 @@ std::map<const void*, std::string> names;
 std::string launches;
 cudaError_t last = cudaSuccess;
 long calls = 0, mallocs = 0, fail_call = -1, fail_malloc = -1, bad = 0;
-unsigned char serial = 0;
+int pattern = 0;
 
 cudaError_t result(cudaError_t e) {
     if (e != cudaSuccess) last = e;
@@ -65,6 +65,7 @@ extern "C" {
 // ------------------------------------------------------------ the tests' side
 void fake_fail_call(long k) { fail_call = k < 0 ? -1 : calls + k; }       // the k-th call from now
 void fake_fail_malloc(long k) { fail_malloc = k < 0 ? -1 : mallocs + k; }
+void fake_pattern(int byte) { pattern = byte; }   // contents of new blocks
 long fake_calls() { return calls; }
 long fake_bad() { return bad; }
 long fake_live() { return (long)blocks.size(); }
@@ -92,7 +93,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
     ++mallocs;
     if (mallocs == fail_malloc || fails()) return result(cudaErrorMemoryAllocation);
     char* c = static_cast<char*>(malloc(n ? n : 1));
-    memset(c, ++serial, n ? n : 1);
+    memset(c, pattern, n ? n : 1);
     blocks[c] = {n, false};
     *p = c;
     return cudaSuccess;
@@ -123,6 +124,11 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, 
 cudaError_t cudaMemset(void* d, int v, size_t n) { return fill(d, v, n); }
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { return fill(d, v, n); }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return fails() ? result(cudaErrorUnknown) : cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* st, unsigned) {
+    *st = nullptr;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t cudaGetLastError() {
     const cudaError_t e = last;

@@ -92,9 +92,53 @@ def learned_scratch_after_failed_growth(fake, hqs):
         hqs.hqs_net_destroy(net)
 
 
+def next_call_after_oom(fake, hqs):
+    """Every allocation of the creating calls fails once; the refusal must not be reported
+    again by the next call, which has nothing to do with it."""
+    good = make_plan(fake, hqs, 32)
+    img, ksp = fake.device(64 * 64 * 8), fake.device(64 * 1024 * 8)
+    traj, maps3 = fake.device(3 * 500 * 4), fake.device(2 * 16 ** 3 * 8)
+    two, zero, h = C.c_float(2.0), C.c_float(0.0), VP()
+
+    def plan():
+        return hqs.hqs_plan_create(C.byref(h), traj, C.c_int64(200), 32, 32, 4, ksp, 4, two, None)
+
+    def volume():
+        return hqs.hqs_plan3d_create(C.byref(h), traj, C.c_int64(200), 16, 16, 16, 2, maps3, 4, two, None)
+
+    def batch():
+        return hqs.hqs_batch_create(C.byref(h), (VP * 1)(plan64), 1, 4)
+
+    def retile():
+        return hqs.hqs_plan_retile(good, 16, None)
+
+    def smaps():
+        return hqs.hqs_estimate_smaps(traj, C.c_int64(200), ksp, None, 32, 2, 4, two, C.c_float(8.0), zero, img, None)
+
+    plan64 = make_plan(fake, hqs, 64)
+    destroy = {plan: hqs.hqs_plan_destroy, volume: hqs.hqs_plan3d_destroy, batch: hqs.hqs_batch_destroy}
+    for call in (plan, volume, batch, retile, smaps):
+        refused = 0
+        while True:
+            live = fake.live()
+            fake.fail_malloc(refused + 1)
+            rc = call()
+            fake.fail_malloc(-1)
+            if rc == 0:
+                break
+            refused += 1
+            assert rc == OOM and refused < 100, (call.__name__, rc)
+            assert fake.live() == live, (call.__name__, refused, "memory lost")
+            assert hqs.hqs_adjoint(good, ksp, img, None) == 0, (call.__name__, refused)
+        assert refused > 0, call.__name__
+        if call in destroy:
+            destroy[call](h)
+
+
 if __name__ == "__main__":
     fake = Fake(sys.argv[1])
     hqs = C.CDLL(sys.argv[2])
     hqs.hqs_net_destroy.restype = hqs.hqs_plan_destroy.restype = hqs.hqs_plan3d_destroy.restype = None
+    hqs.hqs_batch_destroy.restype = None
     globals()[sys.argv[3]](fake, hqs)
     assert fake.bad() == 0

@@ -32,3 +32,7 @@ def test_net_scratch_holds_the_samples(libs):
 @pytest.mark.parametrize("what", ["net", "learned"])
 def test_scratch_after_failed_growth(libs, what):
     run(libs, what + "_scratch_after_failed_growth")
+
+
+def test_next_call_after_oom(libs):
+    run(libs, "next_call_after_oom")
