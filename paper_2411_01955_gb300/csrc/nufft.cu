@@ -827,10 +827,9 @@ __global__ void k_point_weights(const int4* __restrict__ pts, int M, int W, floa
     else o[8 + 2 * b] = o[9 + 2 * b] = w;
 }
 
-int launch_point_weights(hqs_plan_s* p, cudaStream_t st) {
+int launch_point_weights(const hqs_plan_s* p, const int4* pts, float* kbw, cudaStream_t st) {
     if (p->M == 0) return HQS_OK;
-    k_point_weights<<<(unsigned)ceil_div64(p->M * 16, 256), 256, 0, st>>>(p->pts, (int)p->M, p->W, (float)p->beta,
-                                                                          p->spread.kbw);
+    k_point_weights<<<(unsigned)ceil_div64(p->M * 16, 256), 256, 0, st>>>(pts, (int)p->M, p->W, (float)p->beta, kbw);
     HQS_CUDA_TRY(cudaGetLastError());
     return HQS_OK;
 }
@@ -870,10 +869,9 @@ int launch_tile_count(const hqs_plan_s* p, int* counts, cudaStream_t st) {
     HQS_CUDA_TRY(cudaGetLastError());
     return HQS_OK;
 }
-int launch_tile_fill(const hqs_plan_s* p, int* cursor, int4* list, cudaStream_t st) {
+int launch_tile_fill(const hqs_plan_s* p, const int4* pts, const int* perm, int* cursor, int4* list, cudaStream_t st) {
     if (p->M > 0)
-        k_tile_fill<<<(unsigned)ceil_div64(p->M, 256), 256, 0, st>>>(p->pts, p->perm, (int)p->M, p->W, p->G, cursor,
-                                                                     list);
+        k_tile_fill<<<(unsigned)ceil_div64(p->M, 256), 256, 0, st>>>(pts, perm, (int)p->M, p->W, p->G, cursor, list);
     HQS_CUDA_TRY(cudaGetLastError());
     return HQS_OK;
 }

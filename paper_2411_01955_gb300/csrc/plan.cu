@@ -298,8 +298,8 @@ static void plan_free(hqs_plan_s* p) {
 
 // The range of accepted plans: the partial tiles of tile x tile bins, one for every 256
 // points of a bin's distinct neighbours where there are more than 256, stay within 1 GiB.
-static int spread_limit(const hqs_plan_s* p, const std::vector<int>& hc) {
-    const int T = p->tile, nbx = p->G / T, m = std::min(nbx, 3);
+static int spread_limit(const hqs_plan_s* p, const std::vector<int>& hc, int T) {
+    const int nbx = p->G / T, m = std::min(nbx, 3);
     int64_t slots = 0;
     for (int t = 0; t < nbx * nbx; ++t) {
         int64_t cand = 0;
@@ -441,9 +441,9 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
             rc = HQS_ERR_CUDA;
             break;
         }
-        if ((rc = spread_limit(p, hc)) != HQS_OK) break;
+        if ((rc = spread_limit(p, hc, p->tile)) != HQS_OK) break;
         if (M > 0) k_point_scatter<<<ceil_div(M, 256), 256, 0, s>>>(raw, bin, M, counts, p->pts, p->perm);
-        if ((rc = launch_point_weights(p, s)) != HQS_OK) break;
+        if ((rc = launch_point_weights(p, p->pts, p->spread.kbw, s)) != HQS_OK) break;
         if ((rc = spread_build(p, s)) != HQS_OK) break;
 
         // Toeplitz kernel, its FFT (Khat, real, scaled by 1/n2^2) and the density symbol
@@ -513,7 +513,8 @@ int plan_create_internal(hqs_plan* out, const float* traj, int64_t M, int ny, in
 }
 
 static int tile_counts(hqs_plan_s* p, int* cursor, std::vector<int>& cnt, cudaStream_t s);
-static int tile_list(hqs_plan_s* p, int* cursor, const std::vector<int>& cnt, int4* list, cudaStream_t s);
+static int tile_list(hqs_plan_s* p, const int4* pts, const int* perm, int* cursor, const std::vector<int>& cnt,
+                     int4* list, cudaStream_t s);
 
 // Re-binning of the already sorted points for another bin size.
 __global__ void k_rebin(const int4* __restrict__ pts, int M, int G, int W, int TB, int nbx,
@@ -539,6 +540,22 @@ __global__ void k_rebin_scatter(const int4* __restrict__ pts, const int* __restr
     perm_out[pos] = perm[j];
 }
 
+// The re-sorted points and what is made from them, into the plan: one launch, so that all
+// of the plan's point arrays change or none does.  They are replaced in place because a
+// recorded graph of a batch names them.
+__global__ void k_replace_points(int64_t M, int64_t nlist, const int4* __restrict__ pts2, const int* __restrict__ perm2,
+                                 const float4* __restrict__ kbw2, const int4* __restrict__ list2,
+                                 int4* __restrict__ pts, int* __restrict__ perm, float4* __restrict__ kbw,
+                                 int4* __restrict__ list) {
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t e = t0; e < M; e += st) {
+        pts[e] = pts2[e];
+        perm[e] = perm2[e];
+    }
+    for (int64_t e = t0; e < 6 * M; e += st) kbw[e] = kbw2[e];
+    for (int64_t e = t0; e < nlist; e += st) list[e] = list2[e];
+}
+
 extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
     if (!p || (tile != 8 && tile != 16 && tile != 32) || p->G % tile != 0 || 2 * tile < p->W)
         return HQS_ERR_INVALID_ARG;
@@ -547,56 +564,51 @@ extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
     const int M = (int)p->M;
     const int nbx = p->G / tile, nbins = nbx * nbx;
     int *bin = nullptr, *counts = nullptr, *perm2 = nullptr, *cursor = nullptr;
-    int4* pts2 = nullptr;
-    int rc = HQS_OK;
-    const int old_tile = p->tile, old_nbx = p->nbx;
-    do {
-        const int Mp = std::max(M, 1);
-        if (hqs_malloc(&bin, Mp * sizeof(int)) || hqs_malloc(&counts, nbins * sizeof(int)) ||
-            hqs_malloc(&perm2, Mp * sizeof(int)) || hqs_malloc(&pts2, Mp * sizeof(int4)) ||
-            hqs_malloc(&cursor, (size_t)(p->G / 8) * (p->G / 8) * sizeof(int))) {
-            rc = HQS_ERR_OOM;
-            break;
-        }
-        if (cudaMemsetAsync(counts, 0, nbins * sizeof(int), s)) { rc = HQS_ERR_CUDA; break; }
+    int4 *pts2 = nullptr, *list2 = nullptr;
+    float* kbw2 = nullptr;
+    auto build = [&]() -> int {
+        const size_t Mp = (size_t)std::max(M, 1);
+        HQS_CUDA_TRY(cudaMalloc(&bin, Mp * sizeof(int)));
+        HQS_CUDA_TRY(cudaMalloc(&counts, nbins * sizeof(int)));
+        HQS_CUDA_TRY(cudaMalloc(&perm2, Mp * sizeof(int)));
+        HQS_CUDA_TRY(cudaMalloc(&pts2, Mp * sizeof(int4)));
+        HQS_CUDA_TRY(cudaMalloc(&kbw2, Mp * 24 * sizeof(float)));
+        HQS_CUDA_TRY(cudaMalloc(&cursor, (size_t)(p->G / 8) * (p->G / 8) * sizeof(int)));
+        HQS_CUDA_TRY(cudaMemsetAsync(counts, 0, nbins * sizeof(int), s));
         if (M > 0) k_rebin<<<ceil_div(M, 256), 256, 0, s>>>(p->pts, M, p->G, p->W, tile, nbx, bin, counts);
-        std::vector<int> hc(nbins), offs(nbins);
-        if (cudaMemcpyAsync(hc.data(), counts, nbins * sizeof(int), cudaMemcpyDeviceToHost, s) ||
-            cudaStreamSynchronize(s)) { rc = HQS_ERR_CUDA; break; }
+        HQS_CUDA_TRY(cudaGetLastError());
+        std::vector<int> hc(nbins), offs(nbins), cnt;
+        HQS_CUDA_TRY(cudaMemcpyAsync(hc.data(), counts, nbins * sizeof(int), cudaMemcpyDeviceToHost, s));
+        HQS_CUDA_TRY(cudaStreamSynchronize(s));
+        HQS_TRY(spread_limit(p, hc, tile));
         int acc = 0;
         for (int b = 0; b < nbins; ++b) {
             offs[b] = acc;
             acc += hc[b];
         }
-        if (cudaMemcpyAsync(counts, offs.data(), nbins * sizeof(int), cudaMemcpyHostToDevice, s)) {
-            rc = HQS_ERR_CUDA;
-            break;
-        }
+        HQS_CUDA_TRY(cudaMemcpyAsync(counts, offs.data(), nbins * sizeof(int), cudaMemcpyHostToDevice, s));
+        if (M > 0) k_rebin_scatter<<<ceil_div(M, 256), 256, 0, s>>>(p->pts, p->perm, bin, M, counts, pts2, perm2);
+        HQS_CUDA_TRY(cudaGetLastError());
+        HQS_TRY(launch_point_weights(p, pts2, kbw2, s));
+        // the tiles' lists name points by their place in the sorted order
+        HQS_TRY(tile_counts(p, cursor, cnt, s));
+        int64_t total = 0;
+        for (int c : cnt) total += c;
+        HQS_CUDA_TRY(cudaMalloc(&list2, std::max<size_t>(total, 1) * sizeof(int4)));
+        HQS_TRY(tile_list(p, pts2, perm2, cursor, cnt, list2, s));
+        const int64_t most = std::max<int64_t>(6 * (int64_t)M, total);
+        k_replace_points<<<(unsigned)std::min<int64_t>(std::max<int64_t>(ceil_div64(most, 256), 1), 4096), 256, 0, s>>>(
+            M, total, pts2, perm2, reinterpret_cast<const float4*>(kbw2), list2, p->pts, p->perm,
+            reinterpret_cast<float4*>(p->spread.kbw), p->spread.list);
+        HQS_CUDA_TRY(cudaGetLastError());
         p->tile = tile;
         p->nbx = nbx;
-        if ((rc = spread_limit(p, hc)) != HQS_OK) {
-            p->tile = old_tile;
-            p->nbx = old_nbx;
-            break;
-        }
-        if (M > 0) k_rebin_scatter<<<ceil_div(M, 256), 256, 0, s>>>(p->pts, p->perm, bin, M, counts, pts2, perm2);
-        if (M > 0 && (cudaMemcpyAsync(p->pts, pts2, M * sizeof(int4), cudaMemcpyDeviceToDevice, s) ||
-                      cudaMemcpyAsync(p->perm, perm2, M * sizeof(int), cudaMemcpyDeviceToDevice, s))) {
-            rc = HQS_ERR_CUDA;
-            break;
-        }
-        if ((rc = launch_point_weights(p, s)) != HQS_OK) break;
-        // the tiles' lists name points by their place in the sorted order
-        std::vector<int> cnt;
-        if ((rc = tile_counts(p, cursor, cnt, s)) != HQS_OK) break;
-        if ((rc = tile_list(p, cursor, cnt, p->spread.list, s)) != HQS_OK) break;
-        if (cudaStreamSynchronize(s)) { rc = HQS_ERR_CUDA; break; }
-    } while (0);
-    cudaFree(cursor);
-    cudaFree(bin);
-    cudaFree(counts);
-    cudaFree(perm2);
-    cudaFree(pts2);
+        HQS_CUDA_TRY(cudaStreamSynchronize(s));
+        return HQS_OK;
+    };
+    const int rc = build();
+    for (void* v : {(void*)bin, (void*)counts, (void*)perm2, (void*)cursor, (void*)pts2, (void*)list2, (void*)kbw2})
+        cudaFree(v);
     return rc;
 }
 
@@ -622,8 +634,9 @@ static int tile_counts(hqs_plan_s* p, int* cursor, std::vector<int>& cnt, cudaSt
     HQS_CUDA_TRY(cudaStreamSynchronize(s));
     return HQS_OK;
 }
-// the list itself, tile by tile in the order of `cnt`
-static int tile_list(hqs_plan_s* p, int* cursor, const std::vector<int>& cnt, int4* list, cudaStream_t s) {
+// the list itself, tile by tile in the order of `cnt`, of points sorted as in pts and perm
+static int tile_list(hqs_plan_s* p, const int4* pts, const int* perm, int* cursor, const std::vector<int>& cnt,
+                     int4* list, cudaStream_t s) {
     std::vector<int> off(cnt.size());
     int acc = 0;
     for (size_t t = 0; t < cnt.size(); ++t) {
@@ -631,7 +644,7 @@ static int tile_list(hqs_plan_s* p, int* cursor, const std::vector<int>& cnt, in
         acc += cnt[t];
     }
     HQS_CUDA_TRY(cudaMemcpyAsync(cursor, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-    HQS_TRY(launch_tile_fill(p, cursor, list, s));
+    HQS_TRY(launch_tile_fill(p, pts, perm, cursor, list, s));
     HQS_CUDA_TRY(cudaStreamSynchronize(s));
     return HQS_OK;
 }
@@ -690,7 +703,7 @@ int spread_build(hqs_plan_s* p, cudaStream_t s) {
         HQS_CUDA_TRY(cudaMemcpyAsync(nw.light, light.data(), light.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
         HQS_CUDA_TRY(cudaMemcpyAsync(nw.tile_info, info.data(), nt * sizeof(int2), cudaMemcpyHostToDevice, s));
         HQS_CUDA_TRY(cudaMemsetAsync(nw.tickets, 0, (size_t)nt * nch * sizeof(unsigned), s));
-        return tile_list(p, cursor, cnt, nw.list, s);
+        return tile_list(p, p->pts, p->perm, cursor, cnt, nw.list, s);
     };
     const int rc = build();
     cudaFree(cursor);

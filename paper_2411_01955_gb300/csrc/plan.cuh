@@ -142,6 +142,6 @@ inline int spread_cpl(int L) { return L <= 4 ? 1 : (L <= 8 ? 2 : 4); }
 // (re)builds the spreading lists from the sorted points; blocking
 int spread_build(hqs_plan_s* p, cudaStream_t s);
 int launch_tile_count(const hqs_plan_s* p, int* counts, cudaStream_t s);
-int launch_tile_fill(const hqs_plan_s* p, int* cursor, int4* list, cudaStream_t s);
-int launch_point_weights(hqs_plan_s* p, cudaStream_t s);   // spread.kbw from the sorted points
+int launch_tile_fill(const hqs_plan_s* p, const int4* pts, const int* perm, int* cursor, int4* list, cudaStream_t s);
+int launch_point_weights(const hqs_plan_s* p, const int4* pts, float* kbw, cudaStream_t s);
 void spread_free(hqs_plan_s* p);

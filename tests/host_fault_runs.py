@@ -135,6 +135,36 @@ def next_call_after_oom(fake, hqs):
             destroy[call](h)
 
 
+class PlanInfo(C.Structure):
+    _fields_ = [("ny", C.c_int), ("nx", C.c_int), ("coils", C.c_int), ("kernel_width", C.c_int),
+                ("oversamp", C.c_float), ("grid", C.c_int), ("npoints", C.c_int64), ("kb_beta", C.c_double),
+                ("device_bytes", C.c_size_t), ("nsub", C.c_int), ("tile", C.c_int)]
+
+
+def retile_fails_whole(fake, hqs):
+    """Every call that hqs_plan_retile makes fails once: a refusal leaves the plan's arrays and
+    its bin size as they were."""
+    plan, info = make_plan(fake, hqs, 32), PlanInfo()
+    # new blocks look different, so that a copy into the plan's shows
+    fake.mark()
+    fake.pattern(0x5a)
+    before, live, k = fake.hash(), fake.live(), 0
+    while True:
+        k += 1
+        fake.clear_launches()
+        fake.fail_call(k)
+        rc = hqs.hqs_plan_retile(plan, 16, None)
+        fake.fail_call(-1)
+        assert hqs.hqs_plan_get_info(plan, C.byref(info)) == 0
+        replaced = b"k_replace_points" in fake.launches()
+        assert fake.live() == live and fake.hash() == before, (k, rc)
+        assert replaced == (info.tile == 16), (k, rc)
+        if replaced:
+            break
+        assert rc != 0 and k < 200
+    assert k > 10
+
+
 if __name__ == "__main__":
     fake = Fake(sys.argv[1])
     hqs = C.CDLL(sys.argv[2])

@@ -36,3 +36,7 @@ def test_scratch_after_failed_growth(libs, what):
 
 def test_next_call_after_oom(libs):
     run(libs, "next_call_after_oom")
+
+
+def test_retile_fails_whole(libs):
+    run(libs, "retile_fails_whole")
