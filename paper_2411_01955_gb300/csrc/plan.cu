@@ -296,24 +296,6 @@ static void plan_free(hqs_plan_s* p) {
     delete p;
 }
 
-// The range of accepted plans: the partial tiles of tile x tile bins, one for every 256
-// points of a bin's distinct neighbours where there are more than 256, stay within 1 GiB.
-static int spread_limit(const hqs_plan_s* p, const std::vector<int>& hc, int T) {
-    const int nbx = p->G / T, m = std::min(nbx, 3);
-    int64_t slots = 0;
-    for (int t = 0; t < nbx * nbx; ++t) {
-        int64_t cand = 0;
-        for (int a = 0; a < m; ++a)
-            for (int b = 0; b < m; ++b) {
-                const int by = (t / nbx + a - (m == 3) + nbx) % nbx, bx = (t % nbx + b - (m == 3) + nbx) % nbx;
-                cand += hc[by * nbx + bx];
-            }
-        const int64_t k = ceil_div64(cand, 256);
-        if (k > 1) slots += k;
-    }
-    return slots * T * T * p->L * (int64_t)sizeof(float2) > ((int64_t)1 << 30) ? HQS_ERR_UNSUPPORTED : HQS_OK;
-}
-
 static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user, cudaStream_t s) {
     const int n = p->n, L = p->L, G = p->G, n2 = p->n2;
     const int M = (int)p->M;
@@ -441,7 +423,6 @@ static int plan_build(hqs_plan_s* p, const float* traj, const float2* smaps_user
             rc = HQS_ERR_CUDA;
             break;
         }
-        if ((rc = spread_limit(p, hc, p->tile)) != HQS_OK) break;
         if (M > 0) k_point_scatter<<<ceil_div(M, 256), 256, 0, s>>>(raw, bin, M, counts, p->pts, p->perm);
         if ((rc = launch_point_weights(p, p->pts, p->spread.kbw, s)) != HQS_OK) break;
         if ((rc = spread_build(p, s)) != HQS_OK) break;
@@ -580,7 +561,6 @@ extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
         std::vector<int> hc(nbins), offs(nbins), cnt;
         HQS_CUDA_TRY(cudaMemcpyAsync(hc.data(), counts, nbins * sizeof(int), cudaMemcpyDeviceToHost, s));
         HQS_CUDA_TRY(cudaStreamSynchronize(s));
-        HQS_TRY(spread_limit(p, hc, tile));
         int acc = 0;
         for (int b = 0; b < nbins; ++b) {
             offs[b] = acc;
@@ -663,9 +643,15 @@ int spread_build(hqs_plan_s* p, cudaStream_t s) {
     auto build = [&]() -> int {
         std::vector<int> cnt;
         HQS_TRY(tile_counts(p, cursor, cnt, s));
-        int64_t total = 0;
-        for (int c : cnt) total += c;
-        if (total > 0x7fffffffLL) return HQS_ERR_UNSUPPORTED;
+        // the lists and the partial tiles below stay within 8 GiB (which also keeps the lists'
+        // entries in 31 bits): room for 2 10^8 points at W 6
+        int64_t total = 0, parts = 0;
+        for (int c : cnt) {
+            total += c;
+            parts += c > 8 * HQS_SPREAD_LIGHT ? ceil_div(c, 8 * HQS_SPREAD_LIGHT) : 0;
+        }
+        if (total * (int64_t)sizeof(int4) + parts * nch * 64 * cl * (int64_t)sizeof(float2) > (int64_t)8 << 30)
+            return HQS_ERR_UNSUPPORTED;
         std::vector<int4> heavy, light;
         std::vector<int2> info(nt, make_int2(0, 0));
         int slots = 0, off = 0;
