@@ -113,7 +113,8 @@ typedef struct { float kappa; float sigma0; } hqs_gauss_params;
  * the coil maps into the plan (coil-innermost), computes the Toeplitz kernel
  * t(d) = Npix^-1 sum_j exp(i k_j.d) of A^H A on the 2N grid with its FFT, and
  * the density symbol of the circulant CG preconditioner.
- *   traj         (M, 2) float32 device, radians per pixel
+ *   traj         (M, 2) float32 device, radians per pixel (any real value,
+ *                periodic in 2*pi)
  *   smaps        (coils, ny, nx) complex device; Sum_l |S_l|^2 need not be 1
  *   kernel_width W in [2, 8]; oversamp * ny must be a supported FFT size
  *   (supported n: 16, 32, 64, 128, 256, 320, 384 with oversamp 2; any

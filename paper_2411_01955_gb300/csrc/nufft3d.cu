@@ -125,6 +125,7 @@ __global__ void k_points3(const float* __restrict__ traj, int M, int Gx, int Gy,
         int ii = (int)i0;
         if (ii < 0) ii += Gs[ax];
         if (ii >= Gs[ax]) ii -= Gs[ax];
+        if ((unsigned)ii >= (unsigned)Gs[ax]) ii = 0;   // k not finite: the weights are 0
         i0v[ax] = ii;
         int c = ii + W / 2;
         if (c >= Gs[ax]) c -= Gs[ax];

@@ -80,12 +80,13 @@ __global__ void k_point_coords(const float* __restrict__ traj, int M, int G, int
     for (int ax = 0; ax < 2; ++ax) {
         const double k = (double)traj[2 * j + ax];
         double u = (k * (double)G) / (2.0 * 3.141592653589793);
-        if (u < 0.0) u += (double)G;
+        u -= G * floor(u / G);
         const double i0 = ceil(u - 0.5 * (double)W);
         const double d = u - i0;
         int ii = (int)i0;
         if (ii < 0) ii += G;
         if (ii >= G) ii -= G;
+        if ((unsigned)ii >= (unsigned)G) ii = 0;   // k not finite: the weights are 0
         i0v[ax] = ii;
         dv[ax] = (float)d;
         int c = ii + W / 2;
