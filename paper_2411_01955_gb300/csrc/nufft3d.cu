@@ -29,6 +29,7 @@
 
 #include "fft16.cuh"
 #include "plan.cuh"
+#include "spread3_items.cuh"
 
 using namespace hqs;
 
@@ -61,6 +62,7 @@ struct hqs_plan3d_s {
     int nunits = 0;
     int2* list = nullptr;     // the units touching each tile, tile by tile: (first point, offsets of the first
                               // tap from the tile's origin + 16 in one byte per axis, count in the top byte)
+    int64_t* tfirst = nullptr;   // [tiles] first entry of a tile's list
     int4* items = nullptr;    // spreading items: (tile, first entry, end entry, partial slot or -1)
     int nitems = 0;
     int2* tinfo = nullptr;    // [tiles] (items, first partial slot) of tiles with several items
@@ -277,12 +279,13 @@ __global__ void k_tile_count3(const int4* __restrict__ pti, const int2* __restri
     if (u < nunits) touched_tiles3(pti[units[u].x], W, Gx, Gy, Gz, [&](int t, int) { atomicAdd(&counts[t], 1); });
 }
 __global__ void k_tile_fill3(const int4* __restrict__ pti, const int2* __restrict__ units, int nunits, int W, int Gx,
-                             int Gy, int Gz, int* __restrict__ cursor, int2* __restrict__ list) {
+                             int Gy, int Gz, const int64_t* __restrict__ tfirst, int* __restrict__ cursor,
+                             int2* __restrict__ list) {
     const int u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= nunits) return;
     const int2 un = units[u];
     touched_tiles3(pti[un.x], W, Gx, Gy, Gz,
-                   [&](int t, int off) { list[atomicAdd(&cursor[t], 1)] = make_int2(un.x, off | (un.y << 24)); });
+                   [&](int t, int off) { list[tfirst[t] + atomicAdd(&cursor[t], 1)] = make_int2(un.x, off | (un.y << 24)); });
 }
 
 // ------------------------------------------------------ interpolation
@@ -466,7 +469,7 @@ HQS_DEV void spread_rows3(float2 (&acc)[HQS3_TILE][CPL], const char* sp, int n, 
 template <int W, int CPL>
 __global__ void __launch_bounds__(256, 2)
     k_spread3_tiles(const float2* __restrict__ ys, const float* __restrict__ kbw, const int2* __restrict__ list,
-                    const int4* __restrict__ items, const int2* __restrict__ tinfo, unsigned* __restrict__ tickets,
+                    const int64_t* __restrict__ tfirst, const int4* __restrict__ items, const int2* __restrict__ tinfo, unsigned* __restrict__ tickets,
                     float2* __restrict__ partial, int nbx, int nby, int Gx, int Gy, int L, float2* __restrict__ grid) {
     constexpr int T = HQS3_TILE, CL = 4 * CPL, U = HQS3_UNIT, SLOT = spread3_slot<CPL>();
     static_assert(T == 8 && W <= 8 && U == 4, "one plane per warp; two points per 32 lanes of copies");
@@ -487,9 +490,10 @@ __global__ void __launch_bounds__(256, 2)
     // batch r: entries r, r + nbat, r + 2 nbat, ... of the item, lane i holding the i-th
     // (0 beyond the item: no points, an offset that touches no plane)
     const int cnt = it.z - it.y, nbat = (cnt + kBatch3 - 1) / kBatch3;
+    list += tfirst[tile] + it.y;
     auto entry = [&](int r) {
         const int e = r + lane * nbat;
-        return r < nbat && e < cnt ? __ldg(list + it.y + e) : make_int2(0, 0);
+        return r < nbat && e < cnt ? __ldg(list + e) : make_int2(0, 0);
     };
     // this warp's share of a batch's copies: 4 entries, half a warp per point, lane q of
     // the half-warp 16 bytes of weights (q < 8) or of values (pairs of coils, or single
@@ -1627,7 +1631,7 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
             break;
         }
         k_units3<<<nbins, 256, 0, s>>>(p->pti, binoff, ucnt, W, Gx, Gy, Gz, p->units);
-        const unsigned ublk = (unsigned)ceil_div(nu, 256);
+        const unsigned ublk = (unsigned)ceil_div64(nu, 256);
         if (nu > 0) k_tile_count3<<<ublk, 256, 0, s>>>(p->pti, p->units, nu, W, Gx, Gy, Gz, tcnt);
         if (cudaMemcpyAsync(tc.data(), tcnt, nbins * sizeof(int), cudaMemcpyDeviceToHost, s) ||
             cudaStreamSynchronize(s)) {
@@ -1635,41 +1639,26 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
             break;
         }
         // spreading items, heaviest first: every tile's entries in pieces of HQS3_ITEM
-        std::vector<int4> items;
-        std::vector<int2> tinfo(nbins);
-        int slots = 0;
-        int64_t entries = 0;
-        for (int t = 0; t < nbins; ++t) {
-            const int64_t n = tc[t];
-            const int k = (int)std::max<int64_t>(1, ceil_div64(n, HQS3_ITEM));
-            tc[t] = (int)entries;
-            tinfo[t] = make_int2(k, k > 1 ? slots : -1);
-            for (int i = 0; i < k; ++i)
-                items.push_back(make_int4(t, (int)(entries + n * i / k), (int)(entries + n * (i + 1) / k),
-                                          k > 1 ? slots + i : -1));
-            if (k > 1) slots += k;
-            entries += n;
-        }
-        if (entries > 0x7fffffffLL) {
-            rc = HQS_ERR_INVALID_ARG;
-            break;
-        }
-        if ((rc = alloc3(p, &p->list, (size_t)entries)) != HQS_OK) break;
-        if (cudaMemcpyAsync(tcnt, tc.data(), nbins * sizeof(int), cudaMemcpyHostToDevice, s)) {
+        Spread3Items it = spread3_items(tc, HQS3_ITEM);
+        if ((rc = alloc3(p, &p->list, (size_t)it.entries)) != HQS_OK) break;
+        if ((rc = alloc3(p, &p->tfirst, it.first.size())) != HQS_OK) break;
+        if (cudaMemcpyAsync(p->tfirst, it.first.data(), it.first.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s) ||
+            cudaMemsetAsync(tcnt, 0, nbins * sizeof(int), s)) {
             rc = HQS_ERR_CUDA;
             break;
         }
-        if (nu > 0) k_tile_fill3<<<ublk, 256, 0, s>>>(p->pti, p->units, nu, W, Gx, Gy, Gz, tcnt, p->list);
-        std::stable_sort(items.begin(), items.end(),
+        if (nu > 0)
+            k_tile_fill3<<<ublk, 256, 0, s>>>(p->pti, p->units, nu, W, Gx, Gy, Gz, p->tfirst, tcnt, p->list);
+        std::stable_sort(it.items.begin(), it.items.end(),
                          [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
-        p->nitems = (int)items.size();
+        p->nitems = (int)it.items.size();
         const int cl = 4 * spread_cpl(p->L), nch = ceil_div(p->L, cl);
-        if ((rc = alloc3(p, &p->items, items.size())) != HQS_OK) break;
-        if ((rc = alloc3(p, &p->tinfo, tinfo.size())) != HQS_OK) break;
+        if ((rc = alloc3(p, &p->items, it.items.size())) != HQS_OK) break;
+        if ((rc = alloc3(p, &p->tinfo, it.tinfo.size())) != HQS_OK) break;
         if ((rc = alloc3(p, &p->tickets, (size_t)nbins * nch)) != HQS_OK) break;
-        if ((rc = alloc3(p, &p->partial, (size_t)slots * nch * kCells3 * cl)) != HQS_OK) break;
-        if (cudaMemcpyAsync(p->items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, s) ||
-            cudaMemcpyAsync(p->tinfo, tinfo.data(), tinfo.size() * sizeof(int2), cudaMemcpyHostToDevice, s) ||
+        if ((rc = alloc3(p, &p->partial, (size_t)it.slots * nch * kCells3 * cl)) != HQS_OK) break;
+        if (cudaMemcpyAsync(p->items, it.items.data(), it.items.size() * sizeof(int4), cudaMemcpyHostToDevice, s) ||
+            cudaMemcpyAsync(p->tinfo, it.tinfo.data(), it.tinfo.size() * sizeof(int2), cudaMemcpyHostToDevice, s) ||
             cudaMemsetAsync(p->tickets, 0, (size_t)nbins * nch * sizeof(unsigned), s) ||
             cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
             rc = HQS_ERR_CUDA;
@@ -1689,7 +1678,7 @@ int spread3(hqs_plan3d_s* p, const float2* y, float2* grid, cudaStream_t s) {
             const size_t sm = spread3_smem<CPL>();
             auto kern = k_spread3_tiles<WW, CPL>;
             HQS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-            kern<<<dim3(p->nitems, nch), 256, sm, s>>>(p->ysort, p->kbw, p->list, p->items, p->tinfo, p->tickets,
+            kern<<<dim3(p->nitems, nch), 256, sm, s>>>(p->ysort, p->kbw, p->list, p->tfirst, p->items, p->tinfo, p->tickets,
                                                       p->partial, p->nb[0], p->nb[1], p->G[0], p->G[1], p->L, grid);
             HQS_CUDA_TRY(cudaGetLastError());
             return HQS_OK;
@@ -1709,7 +1698,7 @@ int interp3(hqs_plan3d_s* p, const float2* grid, float2* y, cudaStream_t s) {
             // CTAs, 44 us with one)
             constexpr int NG = 256 / LPP;
             const int rounds = std::max(1, std::min(kInterpRounds, p->nunits / (NG * 2 * 152)));
-            k_interp3<WW, VEC, LPP><<<ceil_div(p->nunits, NG * rounds), 256, 0, s>>>(
+            k_interp3<WW, VEC, LPP><<<(unsigned)ceil_div64(p->nunits, NG * rounds), 256, 0, s>>>(
                 grid, p->pti, p->kbw, p->units, p->nunits, rounds, p->M, p->G[0], p->G[1], p->G[2], p->L, y);
             HQS_CUDA_TRY(cudaGetLastError());
             return HQS_OK;
