@@ -1,16 +1,18 @@
 """Autotuner for the per-plan launch shapes, with a JSON cache.
 
-Three knobs change how work is cut into launches, never what is computed
-(beyond float rounding order of atomics and sums):
+Three knobs change how work is ordered and cut into launches, never what is
+computed (beyond the float rounding order of sums):
 
-  spread_tile  edge of the bins the points are sorted in (8, 16, 32)
+  spread_tile  edge of the bins the points are sorted in (8, 16, 32): the order
+               in which the interpolation reads the grid and in which the
+               spreading's lists name the points of an 8 x 8 grid tile
   pc_lines     rows/columns of the preconditioner FFT per work item of the
                persistent solve (1..16)
   fused_grid   cap on the persistent solve's CTAs (0 = every resident CTA)
 
 `autotune(plan)` times each candidate with CUDA events on the plan's own
-operators (hqs_adjoint for the tile, a fixed-iteration persistent DC solve
-for the other two), keeps the fastest, applies it and stores it in the cache
+operators (a forward and an adjoint for the bins, which order both, and a
+fixed-iteration persistent DC solve for the other two), keeps the fastest, applies it and stores it in the cache
 under a key made of the device name and the problem shape, so the next plan of
 the same shape gets the winners without timing anything.
 """
@@ -65,9 +67,9 @@ def store_cache(path: str, key: str, t: Tuning) -> None:
 
 
 def valid_tiles(G: int, W: int) -> list[int]:
-    """Spreading tiles that divide the grid and are at least half the kernel
-    width (so a point's taps reach at most one neighbouring tile per side)."""
-    return [t for t in SPREAD_TILES if G % t == 0 and 2 * t >= W]
+    """Bin edges that divide the grid (any kernel width W: a bin orders the
+    points, it does not hold their taps)."""
+    return [t for t in SPREAD_TILES if G % t == 0]
 
 
 def pick(timings: dict) -> object:
@@ -98,11 +100,26 @@ def _time(fn, reps: int) -> float:
     return s.elapsed_time(e) / reps
 
 
+def time_bins(plan: L.Plan, tiles, x, y, out, reps: int) -> dict:
+    """Time of one forward (image x to k-space data y) and one adjoint (y to the
+    image out) with the points in bins of each edge."""
+    timings = {}
+
+    def both():
+        L.forward(plan, x, y)
+        L.adjoint(plan, y, out)
+
+    for tile in tiles:
+        L.plan_set_tuning(plan, L.HQS_TUNE_SPREAD_TILE, tile)
+        timings[tile] = _time(both, reps)
+    return timings
+
+
 def autotune(plan: L.Plan, cache_path: str | None = None, use_cache: bool = True,
              reps: int = 5, solve_iters: int = 10, solve_shapes: bool = True) -> Tuning:
     """Times the candidates on `plan` (or reads them from the cache), applies
     the winners to the plan and returns them.  solve_shapes=False tunes the
-    spreading tile only (for plans whose solves run in the batched kernel,
+    point bins only (for plans whose solves run in the batched kernel,
     which has its own work decomposition)."""
     import torch
     info = plan.info()
@@ -117,13 +134,9 @@ def autotune(plan: L.Plan, cache_path: str | None = None, use_cache: bool = True
             apply(plan, t)
             return t
     g = torch.Generator(device="cuda").manual_seed(0)
-    y = torch.randn((Lc, max(M, 1)), dtype=torch.complex64, device="cuda", generator=g)[:, :M].contiguous()
-    x = torch.empty((n, n), dtype=torch.complex64, device="cuda")
-    tile_t = {}
-    for tile in valid_tiles(G, W):
-        L.plan_set_tuning(plan, L.HQS_TUNE_SPREAD_TILE, tile)
-        tile_t[tile] = _time(lambda: L.adjoint(plan, y, x), reps)
-    best = Tuning(spread_tile=pick(tile_t))
+    y = torch.empty((Lc, max(M, 1)), dtype=torch.complex64, device="cuda")[:, :M].contiguous()
+    x = torch.randn((n, n), dtype=torch.complex64, device="cuda", generator=g)
+    best = Tuning(spread_tile=pick(time_bins(plan, valid_tiles(G, W), x, y, torch.empty_like(x), reps)))
     L.plan_set_tuning(plan, L.HQS_TUNE_SPREAD_TILE, best.spread_tile)
     if not solve_shapes:
         if use_cache:
