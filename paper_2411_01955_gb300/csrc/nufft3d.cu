@@ -68,7 +68,8 @@ struct hqs_plan3d_s {
     int2* tinfo = nullptr;    // [tiles] (items, first partial slot) of tiles with several items
     unsigned* tickets = nullptr;   // [tiles][coil chunks] arrivals (reset by the last)
     float2* partial = nullptr;     // [slots][coil chunks][512][4 CPL] partial tiles
-    float2* ysort = nullptr;       // [M][L] k-space data in sorted order, coil-innermost
+    float2* ysort = nullptr;       // [M][L] k-space data in sorted order, coil-innermost: in bufB, which the
+                                   // adjoint's passes need only after the spreading, where it has the room
     float* khat = nullptr;    // [2nz][2ny][2nx], includes 1 / (8 Nvox)
     float2* tw = nullptr;     // twiddle bank
     int tw_sizes[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -77,6 +78,7 @@ struct hqs_plan3d_s {
     float* lam = nullptr;     // [nz][ny][nx] Chan symbol of the density preconditioner
     float2* bufA = nullptr;   // 8 Nvox L
     float2* bufB = nullptr;   // 4 Nvox L
+    int64_t bufB_rows = 0;    // 4 Nvox
     float2* bufC = nullptr;   // Nvox L
     float2* cg_r = nullptr;
     float2* cg_p = nullptr;
@@ -1588,7 +1590,8 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
     TRY3(alloc3(p, &p->pti, Mp));
     TRY3(alloc3(p, &p->inv, Mp));
     TRY3(alloc3(p, &p->kbw, Mp * 32));
-    TRY3(alloc3(p, &p->ysort, Mp * p->L));
+    if (p->M <= p->bufB_rows) p->ysort = p->bufB;
+    else TRY3(alloc3(p, &p->ysort, Mp * p->L));
     float4* ptd = nullptr;
     int *binoff = nullptr, *ucnt = nullptr, *tcnt = nullptr;
     auto cleanup = [&]() {
@@ -1638,8 +1641,13 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
             rc = HQS_ERR_CUDA;
             break;
         }
-        // spreading items, heaviest first: every tile's entries in pieces of HQS3_ITEM
-        Spread3Items it = spread3_items(tc, HQS3_ITEM);
+        // spreading items, heaviest first: every tile's entries in pieces of HQS3_ITEM, or of
+        // more where the partial tiles would pass the larger of 128 MiB and one image per coil
+        // (192^3 x 16 coils, 2 10^7 points at random: 20 GiB in pieces of 256; none of 1024)
+        const int cl = 4 * spread_cpl(p->L), nch = ceil_div(p->L, cl);
+        const int64_t slot = (int64_t)nch * kCells3 * cl;
+        const int64_t room = std::max<int64_t>((int64_t)128 << 20, p->bufB_rows / 4 * p->L * (int64_t)sizeof(float2));
+        Spread3Items it = spread3_items_within(tc, HQS3_ITEM, room / (slot * (int64_t)sizeof(float2)));
         if ((rc = alloc3(p, &p->list, (size_t)it.entries)) != HQS_OK) break;
         if ((rc = alloc3(p, &p->tfirst, it.first.size())) != HQS_OK) break;
         if (cudaMemcpyAsync(p->tfirst, it.first.data(), it.first.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s) ||
@@ -1652,11 +1660,10 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
         std::stable_sort(it.items.begin(), it.items.end(),
                          [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
         p->nitems = (int)it.items.size();
-        const int cl = 4 * spread_cpl(p->L), nch = ceil_div(p->L, cl);
         if ((rc = alloc3(p, &p->items, it.items.size())) != HQS_OK) break;
         if ((rc = alloc3(p, &p->tinfo, it.tinfo.size())) != HQS_OK) break;
         if ((rc = alloc3(p, &p->tickets, (size_t)nbins * nch)) != HQS_OK) break;
-        if ((rc = alloc3(p, &p->partial, (size_t)it.slots * nch * kCells3 * cl)) != HQS_OK) break;
+        if ((rc = alloc3(p, &p->partial, (size_t)(it.slots * slot))) != HQS_OK) break;
         if (cudaMemcpyAsync(p->items, it.items.data(), it.items.size() * sizeof(int4), cudaMemcpyHostToDevice, s) ||
             cudaMemcpyAsync(p->tinfo, it.tinfo.data(), it.tinfo.size() * sizeof(int2), cudaMemcpyHostToDevice, s) ||
             cudaMemsetAsync(p->tickets, 0, (size_t)nbins * nch * sizeof(unsigned), s) ||
@@ -1967,7 +1974,8 @@ int plan3d_build(hqs_plan3d_s* p, const float* traj, const float2* smaps_user, c
     for (int a = 0; a < 3; ++a) TRY3(alloc3(p, &p->apod[a], (size_t)p->n[a]));
     TRY3(alloc3(p, &p->khat, (size_t)gvox));
     TRY3(alloc3(p, &p->bufA, (size_t)(gvox * L)));
-    TRY3(alloc3(p, &p->bufB, (size_t)(gvox / 2 * L)));
+    p->bufB_rows = gvox / 2;
+    TRY3(alloc3(p, &p->bufB, (size_t)(p->bufB_rows * L)));
     TRY3(alloc3(p, &p->bufC, (size_t)(nvox * L)));
     TRY3(alloc3(p, &p->cg_r, (size_t)nvox));
     TRY3(alloc3(p, &p->cg_p, (size_t)nvox));

@@ -16,7 +16,7 @@ struct Spread3Items {
 };
 
 // Every tile's entries in pieces of at most `item`, an empty tile one empty item.
-inline Spread3Items spread3_items(const std::vector<int>& counts, int item) {
+inline Spread3Items spread3_items(const std::vector<int>& counts, int64_t item) {
     Spread3Items out;
     out.first.resize(counts.size());
     out.tinfo.resize(counts.size());
@@ -30,5 +30,13 @@ inline Spread3Items spread3_items(const std::vector<int>& counts, int item) {
         if (k > 1) out.slots += k;
         out.entries += n;
     }
+    return out;
+}
+
+// The same with the smallest pieces, item or more by powers of two, whose partial tiles are
+// at most max_slots (pieces of a whole tile need none).
+inline Spread3Items spread3_items_within(const std::vector<int>& counts, int64_t item, int64_t max_slots) {
+    Spread3Items out = spread3_items(counts, item);
+    while (out.slots > max_slots) out = spread3_items(counts, item *= 2);
     return out;
 }
