@@ -463,8 +463,8 @@ HQS_API int hqs_debug_toeplitz_stage(hqs_plan plan, const hqs_c64* x, int precis
  * {8, 16, 32, 64, 128, 160, 192}; coils 1..64; kernel_width 4..8; oversamp
  * must be 2 (the NUFFT grid is then also the 2N Toeplitz grid).  Invalid
  * arguments return HQS_ERR_INVALID_ARG with *out = NULL.  The plan holds
- * about (14 L + 13) * 8 * nz*ny*nx bytes of device memory, 148 bytes per point
- * (coordinates, order, weights), 8 bytes for every unit of up to 4 points of one
+ * about (14 L + 13) * 8 * nz*ny*nx bytes of device memory, 116 bytes per point
+ * (68 at W 4: coordinates, order, weights), 8 bytes for every unit of up to 4 points of one
  * footprint and 8 more for every 8^3 grid tile that it touches (at most 8, 4.3 on
  * average at W 6), partial tiles of at most the larger of 128 MiB and
  * 8 L * nz*ny*nx bytes, and, with more than 4 points per voxel, 8 L bytes per

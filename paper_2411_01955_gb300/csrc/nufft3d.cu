@@ -57,7 +57,7 @@ struct hqs_plan3d_s {
     float* apod[3] = {nullptr, nullptr, nullptr};
     int4* pti = nullptr;      // sorted points: (i0x, i0y, i0z, caller index)
     int* inv = nullptr;       // caller index -> sorted position
-    float* kbw = nullptr;     // [M][32] Kaiser-Bessel weights of the sorted points (k_weights3)
+    float* kbw = nullptr;     // [M][3 taps3(W)] Kaiser-Bessel weights of the sorted points (k_weights3)
     int2* units = nullptr;    // runs of <= HQS3_UNIT sorted points of one footprint: (first, count)
     int nunits = 0;
     int2* list = nullptr;     // the units touching each tile, tile by tile: (first point, offsets of the first
@@ -241,19 +241,21 @@ __global__ void __launch_bounds__(256) k_units3(const int4* __restrict__ pti, co
             units[unit_off[blockIdx.x] + uo[c] + k] =
                 make_int2(b0 + first[c] + k * HQS3_UNIT, min(HQS3_UNIT, cnt[c] - k * HQS3_UNIT));
 }
-// Kaiser-Bessel weights of the sorted points, 32 floats (128 bytes) each: x taps [8],
-// z taps [8], y taps as pairs [8][2] (the operand of packed multiply-adds); zero beyond W.
+// Kaiser-Bessel weights of the sorted points: x taps, y taps, z taps, each of W padded with
+// zeros to a multiple of 4 (16-byte loads and copies).  The spreading makes the pair of
+// equal factors of a packed multiply-add from one tap: with the pairs in the table (128
+// bytes a point at any W in place of 96, 48 at W 4) a 64^3 x 16-coil adjoint took 973 us, so
+// 964.
+__host__ __device__ constexpr int taps3(int W) { return (W + 3) / 4 * 4; }
 __global__ void k_weights3(const float4* __restrict__ ptd, int64_t M, int W, float beta, float* __restrict__ kbw) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= M * 24) return;
-    const int64_t j = e / 24;
-    const int h = (int)(e - j * 24), b = h & 7;
+    const int W4 = taps3(W);
+    if (e >= M * 3 * W4) return;
+    const int64_t j = e / (3 * W4);
+    const int h = (int)(e - j * (3 * W4)), ax = h / W4, b = h - ax * W4;
     const float4 d = ptd[j];
-    const float t = (h < 8 ? d.x : (h < 16 ? d.z : d.y)) - (float)b;
-    const float w = b < W ? kb_phi3(t, (float)W, beta) : 0.f;
-    float* o = kbw + j * 32;
-    if (h < 16) o[h] = w;
-    else o[16 + 2 * b] = o[17 + 2 * b] = w;
+    const float t = (ax == 0 ? d.x : (ax == 1 ? d.y : d.z)) - (float)b;
+    kbw[e] = b < W ? kb_phi3(t, (float)W, beta) : 0.f;
 }
 
 // The tiles (up to two per axis) that a footprint touches: f(tile, offsets).
@@ -329,9 +331,10 @@ __global__ void __launch_bounds__(256, 2) k_interp3(const float2* __restrict__ G
                                                     const float* __restrict__ kbw, const int2* __restrict__ units,
                                                     int nunits, int rounds, int64_t M, int Gx, int Gy,
                                                     int Gz, int L, float2* __restrict__ y) {
-    constexpr int NG = 256 / LPP, U = HQS3_UNIT;
+    constexpr int NG = 256 / LPP, U = HQS3_UNIT, W4 = taps3(W);
     static_assert(U == 4, "one float4 of weights per tap");
-    __shared__ __align__(16) float swt[NG][17][U];   // y taps 0..7, z taps 8..15 by point (17: distinct banks)
+    // y taps, z taps by point (one more row: distinct banks)
+    __shared__ __align__(16) float swt[NG][2 * W4 + 1][U];
     const int g = threadIdx.x / LPP, q = threadIdx.x % LPP;
     for (int r = 0; r < rounds; ++r) {
         const int64_t u = ((int64_t)blockIdx.x * rounds + r) * NG + g;
@@ -340,15 +343,14 @@ __global__ void __launch_bounds__(256, 2) k_interp3(const float2* __restrict__ G
         const int4 p0 = pti[un.x];
         // weights of the unit's points; points beyond its count repeat the last one
         __syncwarp();
-        for (int e = q; e < 16 * U; e += LPP) {
+        for (int e = q; e < 2 * W4 * U; e += LPP) {
             const int k = e & 3, h = e >> 2;
-            const float* kw = kbw + (int64_t)(un.x + min(k, un.y - 1)) * 32;
-            swt[g][h][k] = __ldg(kw + (h < 8 ? 16 + 2 * h : h));
+            swt[g][h][k] = __ldg(kbw + (int64_t)(un.x + min(k, un.y - 1)) * (3 * W4) + W4 + h);
         }
         float wx[U][W];
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const float* kw = kbw + (int64_t)(un.x + min(k, un.y - 1)) * 32;
+            const float* kw = kbw + (int64_t)(un.x + min(k, un.y - 1)) * (3 * W4);
 #pragma unroll
             for (int b = 0; b < W; b += 4) {
                 const float4 v = __ldg(reinterpret_cast<const float4*>(kw + b));
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(256, 2) k_interp3(const float2* __restrict__ G
             for (int k = 0; k < U; ++k) acc[k].zero();
 #pragma unroll 1
             for (int c = 0; c < W; ++c) {
-                const float4 wz = *reinterpret_cast<const float4*>(swt[g][8 + c]);
+                const float4 wz = *reinterpret_cast<const float4*>(swt[g][W4 + c]);
                 const float2* plane = Gh + (int64_t)wrap(p0.z + c, Gz) * Gy * Gx * L + l;
 #pragma unroll
                 for (int a = 0; a < W; ++a) {
@@ -434,16 +436,17 @@ __global__ void __launch_bounds__(256) k_y_to_sorted(const float2* __restrict__ 
 }
 
 constexpr int kBatch3 = 32;    // units staged at once (one per lane of the plane test)
-// bytes of one point's slot: 32 weights, CL values
-template <int CPL> constexpr int spread3_slot() { return 128 + 4 * CPL * (int)sizeof(float2); }
-template <int CPL> constexpr size_t spread3_smem() { return (size_t)2 * kBatch3 * HQS3_UNIT * spread3_slot<CPL>(); }
+// bytes of one point's slot: the weights, CL values
+template <int W> constexpr int spread3_vals() { return 12 * taps3(W); }
+template <int W, int CPL> constexpr int spread3_slot() { return spread3_vals<W>() + 4 * CPL * (int)sizeof(float2); }
+template <int W, int CPL> constexpr size_t spread3_smem() { return (size_t)2 * kBatch3 * HQS3_UNIT * spread3_slot<W, CPL>(); }
 // n points (slots from sp on): wxl the byte offset of the lane's x weight, or -32; wzl
 // that of the plane's z weight; vl that of the lane's values
 template <int W, int CPL, int OY>
 HQS_DEV void spread_rows3(float2 (&acc)[HQS3_TILE][CPL], const char* sp, int n, int wxl, int wzl, int vl) {
     constexpr int T = HQS3_TILE;
 #pragma unroll 1
-    for (int k = 0; k < n; ++k, sp += spread3_slot<CPL>()) {
+    for (int k = 0; k < n; ++k, sp += spread3_slot<W, CPL>()) {
         const float wx = *reinterpret_cast<const float*>(sp + (wxl & 31));
         const float t = (wxl < 0 ? 0.f : wx) * *reinterpret_cast<const float*>(sp + wzl);
         float2 u[CPL];
@@ -457,12 +460,13 @@ HQS_DEV void spread_rows3(float2 (&acc)[HQS3_TILE][CPL], const char* sp, int n, 
 #pragma unroll
             for (int c = 0; c < CPL; ++c) u[c] = cmul_r(reinterpret_cast<const float2*>(sp + vl)[c], t);
         }
-        const float4* wy = reinterpret_cast<const float4*>(sp + 64);
+        const float4* wy = reinterpret_cast<const float4*>(sp + 4 * taps3(W));
 #pragma unroll
         for (int b = 0; b < W; ++b) {
             if (OY + b < 0 || OY + b >= T) continue;
-            const float4 w4 = wy[b >> 1];
-            const float2 w = (b & 1) ? make_float2(w4.z, w4.w) : make_float2(w4.x, w4.y);
+            const float4 w4 = wy[b >> 2];
+            const float wb = (b & 3) == 0 ? w4.x : ((b & 3) == 1 ? w4.y : ((b & 3) == 2 ? w4.z : w4.w));
+            const float2 w = make_float2(wb, wb);
 #pragma unroll
             for (int c = 0; c < CPL; ++c) acc[(OY + b) & (T - 1)][c] = cfma2(u[c], w, acc[(OY + b) & (T - 1)][c]);
         }
@@ -473,7 +477,7 @@ __global__ void __launch_bounds__(256, 2)
     k_spread3_tiles(const float2* __restrict__ ys, const float* __restrict__ kbw, const int2* __restrict__ list,
                     const int64_t* __restrict__ tfirst, const int4* __restrict__ items, const int2* __restrict__ tinfo, unsigned* __restrict__ tickets,
                     float2* __restrict__ partial, int nbx, int nby, int Gx, int Gy, int L, float2* __restrict__ grid) {
-    constexpr int T = HQS3_TILE, CL = 4 * CPL, U = HQS3_UNIT, SLOT = spread3_slot<CPL>();
+    constexpr int T = HQS3_TILE, CL = 4 * CPL, U = HQS3_UNIT, SLOT = spread3_slot<W, CPL>(), VALS = spread3_vals<W>();
     static_assert(T == 8 && W <= 8 && U == 4, "one plane per warp; two points per 32 lanes of copies");
     extern __shared__ float4 smem4[];
     char* sbuf = reinterpret_cast<char*>(smem4);   // [2][kBatch3 U] point slots
@@ -498,7 +502,7 @@ __global__ void __launch_bounds__(256, 2)
         return r < nbat && e < cnt ? __ldg(list + e) : make_int2(0, 0);
     };
     // this warp's share of a batch's copies: 4 entries, half a warp per point, lane q of
-    // the half-warp 16 bytes of weights (q < 8) or of values (pairs of coils, or single
+    // the half-warp 16 bytes of weights (q < VALS / 16) or of values (pairs of coils, or single
     // ones where an odd coil count leaves rows on 8-byte boundaries)
     auto copy = [&](int2 ent, int buf) {
         const int q = lane & 15;
@@ -512,16 +516,16 @@ __global__ void __launch_bounds__(256, 2)
                 const int k = 2 * h + (lane >> 4);
                 if (k >= n) continue;
                 char* d = sbuf + (size_t)((buf * kBatch3 + e) * U + k) * SLOT;
-                if (q < 8) {
-                    cp_async16(d + 16 * q, kbw + (int64_t)(first + k) * 32 + 4 * q);
-                } else {
+                if (q < VALS / 16) {
+                    cp_async16(d + 16 * q, kbw + (int64_t)(first + k) * (VALS / 4) + 4 * q);
+                } else if (q >= 8) {
                     const float2* src = ys + (int64_t)(first + k) * L + l0;
                     const int c = 2 * (q - 8);
                     if (pairs && c < lc) {
-                        cp_async16(d + 128 + 8 * c, src + c);
+                        cp_async16(d + VALS + 8 * c, src + c);
                     } else if (!pairs) {
-                        if (c < lc) cp_async8(d + 128 + 8 * c, src + c);
-                        if (c + 1 < lc) cp_async8(d + 136 + 8 * c, src + c + 1);
+                        if (c < lc) cp_async8(d + VALS + 8 * c, src + c);
+                        if (c + 1 < lc) cp_async8(d + VALS + 8 + 8 * c, src + c + 1);
                     }
                 }
             }
@@ -544,8 +548,8 @@ __global__ void __launch_bounds__(256, 2)
             const char* sp = sbuf + (size_t)(((r & 1) * kBatch3 + b) * U) * SLOT;
             const int bx = xl - ((off & 255) - 16);
             const int wxl = (unsigned)bx < (unsigned)W ? 4 * bx : -32;   // -32: reads tap 0, counts as 0
-            const int wzl = 32 + 4 * (warp - (((off >> 16) & 255) - 16));
-            const int vl = 128 + cq * CPL * (int)sizeof(float2);
+            const int wzl = 8 * taps3(W) + 4 * (warp - (((off >> 16) & 255) - 16));
+            const int vl = VALS + cq * CPL * (int)sizeof(float2);
             const int n = off >> 24;
             switch (((off >> 8) & 255) - 16) {
 #define HQS3_ROWS(OY)                                                                  \
@@ -1589,7 +1593,7 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
     const size_t Mp = (size_t)std::max<int64_t>(p->M, 1);
     TRY3(alloc3(p, &p->pti, Mp));
     TRY3(alloc3(p, &p->inv, Mp));
-    TRY3(alloc3(p, &p->kbw, Mp * 32));
+    TRY3(alloc3(p, &p->kbw, Mp * 3 * taps3(W)));
     if (p->M <= p->bufB_rows) p->ysort = p->bufB;
     else TRY3(alloc3(p, &p->ysort, Mp * p->L));
     float4* ptd = nullptr;
@@ -1614,7 +1618,7 @@ int order_points(hqs_plan3d_s* p, const Points3& pts, cudaStream_t s) {
         }
         k_bin_sort3<<<nbins, 256, 0, s>>>(pts.pti, pts.ptd, binoff, W, Gx, Gy, Gz, p->pti, ptd, p->inv, ucnt);
         if (p->M > 0)
-            k_weights3<<<(unsigned)ceil_div64(p->M * 24, 256), 256, 0, s>>>(ptd, p->M, W, (float)p->beta, p->kbw);
+            k_weights3<<<(unsigned)ceil_div64(p->M * 3 * taps3(W), 256), 256, 0, s>>>(ptd, p->M, W, (float)p->beta, p->kbw);
         std::vector<int> uc(nbins), tc(nbins);
         if (cudaMemcpyAsync(uc.data(), ucnt, nbins * sizeof(int), cudaMemcpyDeviceToHost, s) ||
             cudaStreamSynchronize(s)) {
@@ -1682,7 +1686,7 @@ int spread3(hqs_plan3d_s* p, const float2* y, float2* grid, cudaStream_t s) {
     const int cpl = spread_cpl(p->L), nch = ceil_div(p->L, 4 * cpl);
     return dispatch_w3(p->W, [&]<int WW>() {
         auto go = [&]<int CPL>() {
-            const size_t sm = spread3_smem<CPL>();
+            const size_t sm = spread3_smem<WW, CPL>();
             auto kern = k_spread3_tiles<WW, CPL>;
             HQS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
             kern<<<dim3(p->nitems, nch), 256, sm, s>>>(p->ysort, p->kbw, p->list, p->tfirst, p->items, p->tinfo, p->tickets,

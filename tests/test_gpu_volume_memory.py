@@ -23,7 +23,7 @@ def test_points_cost_what_the_header_says(M, shared):
     for m in (0, M):
         plan = hq.plan3d_create(to_dev(k[:m]), (n, n, n), S, 6, 2.0)
         held.append(plan.info()["device_bytes"])
-    per_point = 148 + 8 * (1 + 8) + (0 if shared else 8 * L)
+    per_point = 116 + 8 * (1 + 8) + (0 if shared else 8 * L)
     # 64 KiB: work items and tickets of the 512 tiles
     assert held[1] - held[0] <= per_point * M + (128 << 20) + (64 << 10)
     x, y = to_dev(synth.phantom3d(1, (n, n, n))), to_dev(synth.complex_noise(3, (L, M)))
