@@ -473,7 +473,8 @@ HQS_API int hqs_plan3d_create(hqs_plan3d* out, const float* traj, int64_t M, int
                               int coils, const hqs_c64* smaps, int kernel_width, float oversamp,
                               void* stream);
 HQS_API void hqs_plan3d_destroy(hqs_plan3d plan);
-/* Host outputs (NULL skipped): point count, spreading sub-problems, device bytes held. */
+/* Host outputs (NULL skipped): point count, work items of the tile-owned spreading (CTAs
+ * per 4, 8 or 16 coils), device bytes held. */
 HQS_API int hqs_plan3d_get_info(hqs_plan3d plan, int64_t* npoints, int* nsub, size_t* device_bytes);
 
 /* y = A x by 3D gridding: apodise, zero-pad to the 2N grid, 3D FFT, W^3

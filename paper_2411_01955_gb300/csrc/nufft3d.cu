@@ -52,7 +52,6 @@ struct hqs_plan3d_s {
     int64_t M = 0;
     float scale = 1.f;        // Nvox^-1/2
     int nb[3] = {0, 0, 0};
-    int nsub = 0;
     float2* smaps = nullptr;  // [nz][ny][nx][L]
     float* apod[3] = {nullptr, nullptr, nullptr};
     int4* pti = nullptr;      // sorted points: (i0x, i0y, i0z, caller index)
@@ -1484,7 +1483,8 @@ bool size3_ok(int n) {
     return n >= 8 && n % 2 == 0 && fft_size_supported(2 * n) && fft_size_supported(4 * n);
 }
 
-// Sorted points and spreading sub-problems for grid G with kernel width W.
+// Points in bin order for grid G with kernel width W and, for the unit spreading, its
+// sub-problems.
 struct Points3 {
     int4* pti = nullptr;
     float4* ptd = nullptr;
@@ -1494,8 +1494,7 @@ struct Points3 {
     std::vector<int> off;   // [bins + 1] first point of each bin
 };
 
-int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], int W, Points3* out,
-                 cudaStream_t s) {
+int build_points(const float* traj, int64_t M, const int G[3], int W, bool with_subs, Points3* out, cudaStream_t s) {
     for (int a = 0; a < 3; ++a) out->nb[a] = G[a] / HQS3_TILE;
     const int nbins = out->nb[0] * out->nb[1] * out->nb[2];
     int4* rawi = nullptr;
@@ -1533,7 +1532,7 @@ int build_points(hqs_plan3d_s* p, const float* traj, int64_t M, const int G[3], 
         int acc = 0;
         for (int b = 0; b < nbins; ++b) {
             offs[b] = acc;
-            for (int st = 0; st < hc[b]; st += HQS3_MAXPTS)
+            for (int st = 0; with_subs && st < hc[b]; st += HQS3_MAXPTS)
                 subs.push_back(make_int4(b, acc + st, std::min(HQS3_MAXPTS, hc[b] - st), 0));
             acc += hc[b];
         }
@@ -1930,7 +1929,7 @@ int build_khat(hqs_plan3d_s* p, const float* traj, cudaStream_t s) {
             }
         }
         if (rc != HQS_OK) break;
-        if ((rc = build_points(p, traj, p->M, G4, Wk, &pts, s)) != HQS_OK) break;
+        if ((rc = build_points(traj, p->M, G4, Wk, true, &pts, s)) != HQS_OK) break;
         if ((rc = spread3_unit(pts, G4, bk, grid, s)) != HQS_OK) break;
         // z: [2nz][4ny][4nx] in mid (circulant crop)
         const int64_t row4 = G4[0], plane4 = (int64_t)G4[1] * G4[0];
@@ -2037,9 +2036,8 @@ int plan3d_build(hqs_plan3d_s* p, const float* traj, const float2* smaps_user, c
     HQS_CUDA_TRY(cudaGetLastError());
     {
         Points3 pts;   // bin order, freed once the footprint order is made
-        int rc = build_points(p, traj, p->M, p->G, p->W, &pts, s);
+        int rc = build_points(traj, p->M, p->G, p->W, false, &pts, s);
         for (int a = 0; a < 3; ++a) p->nb[a] = pts.nb[a];
-        p->nsub = pts.nsub;
         if (rc == HQS_OK) rc = order_points(p, pts, s);
         cudaFree(pts.pti);
         cudaFree(pts.ptd);
@@ -2247,7 +2245,7 @@ extern "C" int hqs_dc_solve3d(hqs_plan3d p, float a, float b, const hqs_c64* rhs
 extern "C" int hqs_plan3d_get_info(hqs_plan3d p, int64_t* npoints, int* nsub, size_t* device_bytes) {
     if (!p) return HQS_ERR_INVALID_ARG;
     if (npoints) *npoints = p->M;
-    if (nsub) *nsub = p->nsub;
+    if (nsub) *nsub = p->nitems;
     if (device_bytes) *device_bytes = p->bytes;
     return HQS_OK;
 }

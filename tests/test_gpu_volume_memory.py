@@ -33,3 +33,14 @@ def test_points_cost_what_the_header_says(M, shared):
     a = np.vdot(to_host(Ax), to_host(y))
     b = np.vdot(to_host(x), to_host(Ahy))
     assert abs(a - b) <= 1e-5 * np.linalg.norm(to_host(Ax)) * np.linalg.norm(to_host(y))
+
+
+def test_info_counts_the_spreading_items():
+    """One item for each of the 64 tiles of the 32^3 grid, and 4 more where 5,000 equal points (1,250 units
+    of 4, pieces of 256) lie in one tile."""
+    import paper_2411_01955_gb300 as hq
+    n = 16
+    S = to_dev(synth.coil_maps3d(2, (n, n, n), 1))
+    k = np.full((5000, 3), 5.5 * 2 * np.pi / (2 * n), dtype=np.float32)   # taps 4 .. 7 at W 4
+    for m, items in ((0, 64), (5000, 68)):
+        assert hq.plan3d_create(to_dev(k[:m]), (n, n, n), S, 4, 2.0).info()["nsub"] == items
