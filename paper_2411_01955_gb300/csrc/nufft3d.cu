@@ -1707,7 +1707,7 @@ int interp3(hqs_plan3d_s* p, const float2* grid, float2* y, cudaStream_t s) {
             // (a whole forward at 16 x 64 x 64 x 2 coils, 5,568 points: 97 us with 4 rounds on 11
             // CTAs, 44 us with one)
             constexpr int NG = 256 / LPP;
-            const int rounds = std::max(1, std::min(kInterpRounds, p->nunits / (NG * 2 * 152)));
+            const int rounds = std::max(1, std::min(kInterpRounds, p->nunits / (NG * 2 * p->nsm)));
             k_interp3<WW, VEC, LPP><<<(unsigned)ceil_div64(p->nunits, NG * rounds), 256, 0, s>>>(
                 grid, p->pti, p->kbw, p->units, p->nunits, rounds, p->M, p->G[0], p->G[1], p->G[2], p->L, y);
             HQS_CUDA_TRY(cudaGetLastError());
