@@ -118,8 +118,6 @@ template <class T> static inline cudaError_t hqs_malloc(T** p, size_t bytes) {
 
 // Device error word bits (per plan), read back at sync points.
 #define HQS_DEVERR_TIMEOUT   1u
-#define HQS_DEVERR_BREAKDOWN 2u
-#define HQS_DEVERR_BOUNDS    4u
 
 // Launch with programmatic stream serialisation: the kernel's CTAs may start
 // while the previous kernel of the stream finishes (the kernel begins with

@@ -23,10 +23,10 @@
 
 namespace {
 
-enum ConvMode { CONV_FWD = 0, CONV_FWD_RELU = 1, CONV_DGRAD_MASK = 2 };
+enum ConvMode { CONV_FWD_RELU, CONV_DGRAD_MASK };
 
 // CIN input channels -> COUT output channels on a 16x16 pixel tile.
-// CONV_FWD*: weights W[COUT][CIN][9], bias b[COUT].
+// CONV_FWD_RELU: weights W[COUT][CIN][9], bias b[COUT].
 // CONV_DGRAD_MASK: the layer's weights W[CIN][COUT][9] are read flipped and
 // transposed, no bias, output multiplied by (mask > 0).
 // CPLX (CIN 2): x is an interleaved complex image, its parts times `scale` the channels.
@@ -281,7 +281,7 @@ __device__ __forceinline__ void put_row(uint8_t* buf, const float (&v)[kTcPer][8
     }
 }
 
-// MODE as k_conv3x3 (CONV_FWD / CONV_FWD_RELU with bias, CONV_DGRAD_MASK with
+// MODE as k_conv3x3 (CONV_FWD_RELU with bias, CONV_DGRAD_MASK with
 // the layer's weights flipped and transposed and the ReLU mask of its input).
 // Work unit u = (sample, 128-column strip, run of `rows` output rows).
 template <int MODE>
@@ -587,7 +587,6 @@ static int net_reserve(hqs_net_s* net, int N, int H, int Wd) {
     return HQS_OK;
 }
 
-// forward; activations kept in net->act[0..3] (act[3] = output)
 // the two hidden layers: net->act[0] -> net->act[2]
 static int net_hidden(hqs_net_s* net, int N, int H, int Wd, cudaStream_t st) {
     const float* P = net->params;
@@ -604,6 +603,7 @@ static int net_hidden(hqs_net_s* net, int N, int H, int Wd, cudaStream_t st) {
     return HQS_OK;
 }
 
+// forward; activations kept in net->act[0..3] (act[3] = the output when out is NULL)
 int net_forward(hqs_net_s* net, const float* x, float* out, int N, int H, int Wd, cudaStream_t st) {
     HQS_TRY_RC(net_reserve(net, N, H, Wd));
     const float* P = net->params;

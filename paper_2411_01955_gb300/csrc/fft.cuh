@@ -523,11 +523,6 @@ template <int N> struct FftPair;
 #define FH(R, P) fft_stage_io<NN_, E_, R, P, false, ZIN_ && P == 1, false, P == 1, false>(s, t, act, tw, ld, nio, nio);
 #define FT(R, P) fft_stage_io<NN_, E_, R, P, true, false, HOUT_ && P * R == NN_, false, P * R == NN_>(s, t, act, tw, nio, nio, stf);
 
-#define NN_ 16
-#define E_ 4
-HQS_FFT_PAIR(16, 4, 4, FH(4, 1), FT(4, 4))
-#undef NN_
-#undef E_
 #define NN_ 32
 #define E_ 8
 HQS_FFT_PAIR(32, 8, 4, FH(8, 1), FT(8, 4))
@@ -556,21 +551,6 @@ HQS_FFT_PAIR(320, 40, 40, FH(8, 1), FT(8, 40))
 #define NN_ 384
 #define E_ 24
 HQS_FFT_PAIR(384, 24, 6, FH(8, 1) FH(8, 8), FT(8, 6) FT(8, 48))
-#undef NN_
-#undef E_
-#define NN_ 512
-#define E_ 16
-HQS_FFT_PAIR(512, 16, 8, FH(8, 1) FH(8, 8), FT(8, 8) FT(8, 64))
-#undef NN_
-#undef E_
-#define NN_ 640
-#define E_ 40
-HQS_FFT_PAIR(640, 40, 10, FH(8, 1) FH(8, 8), FT(8, 10) FT(8, 80))
-#undef NN_
-#undef E_
-#define NN_ 768
-#define E_ 24
-HQS_FFT_PAIR(768, 24, 12, FH(8, 1) FH(8, 8), FT(8, 12) FT(8, 96))
 #undef NN_
 #undef E_
 #undef FH

@@ -1108,7 +1108,7 @@ int run_half(const hqs_plan3d_s* p, int N, LD ld, ST st, int64_t nlines, int64_t
     return N == 128 ? go.template operator()<128>() : go.template operator()<256>();
 }
 // the last x pass with the coil sum on registers, for the coil counts that divide kLines
-template <bool ROT, class F> int with_coils(int L, F&& f) {
+template <class F> int with_coils(int L, F&& f) {
     switch (L) {
         case 1: return f.template operator()<1>();
         case 2: return f.template operator()<2>();
@@ -1771,7 +1771,7 @@ int adj3(hqs_plan3d_s* p, const float2* y, float2* x, cudaStream_t s) {
     // else per coil into bufC and a separate sum
     if (kLines % L == 0) {
         if (half3(Gx))
-            return with_coils<true>(L, [&]<int CO>() {
+            return with_coils(L, [&]<int CO>() {
                 return run_half<PASS_INV, true>(p, Gx, LdRaw{p->bufA, lx},
                                                 StCoilSumRow<CO>{x, p->smaps, nullptr, p->apod[0], p->apod[1], p->apod[2], nx,
                                                                  ny, p->scale, 0.f},
@@ -1823,7 +1823,7 @@ int toep3(hqs_plan3d_s* p, const float2* x, float2* out, float ca, float cb, con
     // x inverse with the conj(S_l) coil sum fused (whole rows per CTA), else per coil in bufC + sum
     if (kLines % L == 0) {
         if (half3(Tx))
-            return with_coils<false>(L, [&]<int CO>() {
+            return with_coils(L, [&]<int CO>() {
                 return run_half<PASS_INV, false>(
                     p, Tx, LdRaw{p->bufA, lx}, StCoilSumRow<CO>{out, p->smaps, z, nullptr, nullptr, nullptr, nx, ny, ca, cb},
                     nrow, L, s);

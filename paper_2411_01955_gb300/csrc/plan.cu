@@ -539,8 +539,7 @@ __global__ void k_replace_points(int64_t M, int64_t nlist, const int4* __restric
 }
 
 extern "C" int hqs_plan_retile(hqs_plan p, int tile, void* stream) {
-    if (!p || (tile != 8 && tile != 16 && tile != 32) || p->G % tile != 0 || 2 * tile < p->W)
-        return HQS_ERR_INVALID_ARG;
+    if (!p || (tile != 8 && tile != 16 && tile != 32) || p->G % tile != 0) return HQS_ERR_INVALID_ARG;
     if (tile == p->tile) return HQS_OK;
     cudaStream_t s = (cudaStream_t)stream;
     const int M = (int)p->M;
