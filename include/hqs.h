@@ -387,7 +387,8 @@ HQS_API int hqs_batch_toeplitz_normal(hqs_batch batch, const hqs_c64* const* x, 
  * zc z[i] (z NULL, or z[i] NULL: no axpy term), for every slice i.  The
  * slices whose grid is 2n (at any coil count from 128 points on, with full
  * 16-coil chunks below) run their row and column FFT passes together, one
- * launch per pass, grid size and lines per CTA; spreading, interpolation and the other slices' passes run per slice.  y[i]: (L_i, M_i),
+ * launch per pass, grid size and lines per CTA; spreading, interpolation and
+ * the other slices' passes run per slice.  y[i]: (L_i, M_i),
  * x[i], z[i]: (n_i, n_i), device complex64, caller-owned.  Enqueued on
  * `stream`; synchronises it first when the image pointers differ from the last
  * call.  Uses the plans' workspaces: calls on one batch (and on its plans) run
@@ -415,7 +416,9 @@ HQS_API const char* hqs_status_string(int status);
 
 /* Tuning knobs (no counterpart in the paper), set per plan by the autotuner:
  *   HQS_TUNE_FUSED_GRID  cap on the persistent solve's CTAs (0 = all resident)
- *   HQS_TUNE_PC_LINES    preconditioner rows/columns per work item (1..16)
+ *   HQS_TUNE_PC_LINES    preconditioner rows/columns per work item (1..16; at
+ *                        n = 256 a CTA transforms 8 lines at once, and more
+ *                        count as 8)
  *   HQS_TUNE_SPREAD_TILE edge of the point bins (8, 16 or 32): re-bins the
  *                        plan's points (hqs_plan_retile on the default stream)
  * and one test hook for the failure path of the persistent solve:

@@ -444,19 +444,19 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_hqs_batch(BatchArgs B) {
             });
             BB_BARRIER();
             FOR_ITEMS(BL_ROWS, {
-            STAGE_TW2(S.A);
-            item_rows_fwd(S, it_, S.p);
-        });
+                STAGE_TW2(S.A);
+                item_rows_fwd(S, it_, S.p);
+            });
             BB_BARRIER();
             FOR_ITEMS(BL_COLS, {
-            STAGE_TW2(S.A);
-            item_cols(S, it_);
-        });
+                STAGE_TW2(S.A);
+                item_cols(S, it_);
+            });
             BB_BARRIER();
             CLEAR_ACC();
             FOR_ITEMS(BL_ROWS, {
                 STAGE_TW2(S.A);
-            double v = item_rows_adj(S, it_, S.q, S.p, acoef, bcoef, 1);
+                double v = item_rows_adj(S, it_, S.q, S.p, acoef, bcoef, 1);
                 v = cta_sum(v, red);
                 if (threadIdx.x == 0) acc[0][si] += v;
             });
@@ -875,18 +875,18 @@ __global__ void __launch_bounds__(HQS_BATCH_BD, 2) k_aha_batch(AhaBatchArgs B) {
         }                                                                                  \
     }
     FOR_ITEMS(BL_ROWS, {
-            STAGE_TW2(S.A);
-            item_rows_fwd(S, it_, S.u);
-        });
+        STAGE_TW2(S.A);
+        item_rows_fwd(S, it_, S.u);
+    });
     AB_BARRIER();
     FOR_ITEMS(BL_COLS, {
-            STAGE_TW2(S.A);
-            item_cols(S, it_);
-        });
+        STAGE_TW2(S.A);
+        item_cols(S, it_);
+    });
     AB_BARRIER();
     FOR_ITEMS(BL_ROWS, {
         STAGE_TW2(S.A);
-            item_rows_adj(S, it_, S.q, nullptr, 1.f, 0.f, 0);
+        item_rows_adj(S, it_, S.q, nullptr, 1.f, 0.f, 0);
     });
     if (B.off[BL_EPI * (ns + 1) + ns] > 0) {   // several coil chunks: fixed-order chunk sum
         AB_BARRIER();

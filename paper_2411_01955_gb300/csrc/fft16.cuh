@@ -1,6 +1,7 @@
 // Two-stage transforms of 2n-point lines (N = 2n = 16 R) whose input half is zero or
-// whose output half is not wanted: the only transforms of the Toeplitz passes and of
-// the NUFFT's lower-half passes.
+// whose output half is not wanted: the transforms of the Toeplitz passes and of the
+// NUFFT's lower-half passes at 128 points and more (fft16_ok; shorter lines keep the
+// radix-8 stages of fft.cuh).
 //
 //   X[kk + 16 m] = sum_{i < R} w_R^(i m) w_N^(i kk) sum_{r < 8} w_16^(r kk) x[i + R r],   kk < 16, m < R
 //

@@ -407,9 +407,9 @@ __global__ void __launch_bounds__(256) k_interp(const float2* __restrict__ Gh, c
 // k-space values of 16 points at a time go to the warp's own shared memory with
 // cp.async while the 16 before are added: a warp needs no barrier.
 // A tile of at most HQS_SPREAD_LIGHT points belongs to one warp, eight such tiles to a
-// CTA; a heavier one to whole CTAs of up to 8 HQS_SPREAD_LIGHT points each, whose warps' tiles are summed through shared
-// memory, and, where there are several CTAs, through partial tiles in slot order by the
-// last to arrive.
+// CTA; a heavier one to whole CTAs of up to 8 HQS_SPREAD_LIGHT points each, whose warps'
+// tiles are summed through shared memory, and, where there are several CTAs, through
+// partial tiles in slot order by the last to arrive.
 // Bound: latency of a point's shared-memory reads and switch, and of the list, weight and
 // value reads per tile.  320^2 x 16 coils, 32,768 spiral points: a whole adjoint 85.5 ->
 // 62.1 us (384^2 x 13 coils, 56,064 radial points: 145 -> 94.8) against CTAs that scanned
@@ -941,16 +941,20 @@ int launch_half_group(int G, int n, int lines, int maxchunk, int maxcoils, int c
                 if (adjoint) {
                     constexpr int th = half_threads<GG, LN>();
                     constexpr size_t sm = half_smem<GG, LN>();
-                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_cols_h_b<GG, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows_h_b<GG, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_cols_h_b<GG, LN>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_adj_rows_h_b<GG, LN>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
                     HQS_CUDA_TRY(launch_pdl(k_adj_cols_h_b<GG, LN>, dim3(GG, maxchunk, count), th, sm, st, tab, zc));
                     HQS_CUDA_TRY(launch_pdl(k_adj_rows_h_b<GG, LN>, dim3(n, maxchunk, count), th, sm, st, tab, zc));
                 } else {
                     constexpr int LI = half_free_lines<GG, LN>(), th = half_threads<GG, LI>();
                     constexpr size_t sm = half_smem<GG, LI>();
                     const int nc = ceil_div(maxcoils, LI);
-                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h_b<GG, LI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h_b<GG, LI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_rows_h_b<GG, LI>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    HQS_CUDA_TRY(cudaFuncSetAttribute(k_fwd_cols_h_b<GG, LI>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
                     HQS_CUDA_TRY(launch_pdl(k_fwd_rows_h_b<GG, LI>, dim3(n, nc, count), th, sm, st, tab, zc));
                     HQS_CUDA_TRY(launch_pdl(k_fwd_cols_h_b<GG, LI>, dim3(GG, nc, count), th, sm, st, tab, zc));
                 }

@@ -23,6 +23,7 @@
 // the contiguous index, 16 lines per CTA, so loads and stores are coalesced
 // over b.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstddef>
 #include <vector>
@@ -438,7 +439,9 @@ constexpr int kBatch3 = 32;    // units staged at once (one per lane of the plan
 // bytes of one point's slot: the weights, CL values
 template <int W> constexpr int spread3_vals() { return 12 * taps3(W); }
 template <int W, int CPL> constexpr int spread3_slot() { return spread3_vals<W>() + 4 * CPL * (int)sizeof(float2); }
-template <int W, int CPL> constexpr size_t spread3_smem() { return (size_t)2 * kBatch3 * HQS3_UNIT * spread3_slot<W, CPL>(); }
+template <int W, int CPL> constexpr size_t spread3_smem() {
+    return (size_t)2 * kBatch3 * HQS3_UNIT * spread3_slot<W, CPL>();
+}
 // n points (slots from sp on): wxl the byte offset of the lane's x weight, or -32; wzl
 // that of the plane's z weight; vl that of the lane's values
 template <int W, int CPL, int OY>
@@ -474,9 +477,10 @@ HQS_DEV void spread_rows3(float2 (&acc)[HQS3_TILE][CPL], const char* sp, int n, 
 template <int W, int CPL>
 __global__ void __launch_bounds__(256, 2)
     k_spread3_tiles(const float2* __restrict__ ys, const float* __restrict__ kbw, const int2* __restrict__ list,
-                    const int64_t* __restrict__ tfirst, const int4* __restrict__ items, const int2* __restrict__ tinfo, unsigned* __restrict__ tickets,
-                    float2* __restrict__ partial, int nbx, int nby, int Gx, int Gy, int L, float2* __restrict__ grid) {
-    constexpr int T = HQS3_TILE, CL = 4 * CPL, U = HQS3_UNIT, SLOT = spread3_slot<W, CPL>(), VALS = spread3_vals<W>();
+                    const int64_t* __restrict__ tfirst, const int4* __restrict__ items, const int2* __restrict__ tinfo,
+                    unsigned* __restrict__ tickets, float2* __restrict__ partial, int nbx, int nby, int Gx, int Gy, int L, float2* __restrict__ grid) {
+    constexpr int T = HQS3_TILE, CL = 4 * CPL, U = HQS3_UNIT;
+    constexpr int SLOT = spread3_slot<W, CPL>(), VALS = spread3_vals<W>();
     static_assert(T == 8 && W <= 8 && U == 4, "one plane per warp; two points per 32 lanes of copies");
     extern __shared__ float4 smem4[];
     char* sbuf = reinterpret_cast<char*>(smem4);   // [2][kBatch3 U] point slots
@@ -899,9 +903,10 @@ __global__ void k_pass3(LD ld, ST st, MID mid, int64_t nlines, int64_t B, const 
 // by i^k (see nufft.cu).  They run on the two-stage transforms of fft16.cuh where those
 // cover the size (128 and 256 points here): one shared-memory round trip per transform.
 // Bound: instruction issue.
-// Their sizes fit 32 bits (at most 2^23 lines, strides of 2^23 elements): the line's
-// division and the element offsets are 32-bit operations, one wide multiply-add each (as
-// 64-bit ones they were a third of the passes' instructions).
+// Their sizes fit 32 bits (at most 384 x 384 x 64 coils = 9.4 million lines, and strides of as
+// many elements; run_half refuses more): the line's division and the element offsets are
+// 32-bit operations, one wide multiply-add each (as 64-bit ones they were a third of the
+// passes' instructions).
 struct LinesI {
     int64_t sA;
     int sP;
@@ -1095,7 +1100,7 @@ int run_half(const hqs_plan3d_s* p, int N, LD ld, ST st, int64_t nlines, int64_t
     const float2* tw = nullptr;
     for (int i = 0; i < 9; ++i)
         if (p->tw_sizes[i] == N) tw = p->tw + p->tw_offs[i] + N;
-    if (!tw || !half3(N)) return HQS_ERR_INVALID_ARG;
+    if (!tw || !half3(N) || nlines > INT_MAX - kLines) return HQS_ERR_INVALID_ARG;
     auto go = [&]<int NN>() -> int {
         auto kern = k_pass3h<NN, DIR, ROT, LD, ST, MID>;
         constexpr size_t sm = (size_t)(2 * NN * kLines + NN) * sizeof(float2);
@@ -1729,9 +1734,9 @@ int fwd3(hqs_plan3d_s* p, const float2* x, float2* y, cudaStream_t s) {
         TRY3((run_half<PASS_FWD, true>(p, Gx, LdImageRow{x, p->smaps, p->apod[0], p->apod[1], p->apod[2], nx, ny, L, p->scale},
                                        StRaw{p->bufA, Lines{(int64_t)Gx * L, L}}, (int64_t)nz * ny * L, L, s)));
     } else {
-    TRY3((run_pass<false, false, false>(
-        p, Gx, LdImageX{x, p->smaps, p->apod[0], p->apod[1], p->apod[2], nx, ny, Gx, L, p->scale},
-        StLine{p->bufA, {(int64_t)Gx * L, L}, Gx, 0, Gx}, (int64_t)nz * ny * L, L, s)));
+        TRY3((run_pass<false, false, false>(
+            p, Gx, LdImageX{x, p->smaps, p->apod[0], p->apod[1], p->apod[2], nx, ny, Gx, L, p->scale},
+            StLine{p->bufA, {(int64_t)Gx * L, L}, Gx, 0, Gx}, (int64_t)nz * ny * L, L, s)));
     }
     // y pass: [nz][Gy][Gx][L] in bufB
     const int64_t row = (int64_t)Gx * L, plane = (int64_t)Gy * row;
@@ -1812,7 +1817,8 @@ int toep3(hqs_plan3d_s* p, const float2* x, float2* out, float ca, float cb, con
     // z: FFT, Khat, IFFT, rows z < nz, in place in bufB
     const MidKhat mk{p->khat, (int64_t)Ty * Tx, L};
     if (half3(Tz))
-        TRY3((run_half<PASS_PAIR, false>(p, Tz, LdRaw{p->bufB, lz}, StRaw{p->bufB, lz}, plane, plane, s, MidKhatI{p->khat, Ty * Tx, L})));
+        TRY3((run_half<PASS_PAIR, false>(p, Tz, LdRaw{p->bufB, lz}, StRaw{p->bufB, lz}, plane, plane, s,
+                                         MidKhatI{p->khat, Ty * Tx, L})));
     else
         TRY3((run_pass<true, true, true>(p, Tz, LdLine{p->bufB, lz, nz}, StLine{p->bufB, lz, nz, 0, Tz}, plane, plane, s, mk)));
     // y inverse: [nz][ny][Tx][L] in bufA

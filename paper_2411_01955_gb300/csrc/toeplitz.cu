@@ -22,8 +22,9 @@ using namespace hqs;
 
 // --------------------------------------------------------- plain kernels
 template <int N2, int LINES>
-__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>()) k_toep_rows_fwd(ToepArgs A, const float2* __restrict__ src, float2* __restrict__ pvec,
-                                int fuse, const CgScalars* __restrict__ cg) {
+__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>())
+    k_toep_rows_fwd(ToepArgs A, const float2* __restrict__ src, float2* __restrict__ pvec, int fuse,
+                    const CgScalars* __restrict__ cg) {
     HQS_PDL_ENTRY();
     if (cg && cg->done) return;
     extern __shared__ __align__(16) float2 s[];
@@ -32,7 +33,8 @@ __global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<
 }
 
 template <int N2, int LINES>
-__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>()) k_toep_cols(ToepArgs A, const CgScalars* __restrict__ cg) {
+__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>())
+    k_toep_cols(ToepArgs A, const CgScalars* __restrict__ cg) {
     HQS_PDL_ENTRY();
     if (cg && cg->done) return;
     extern __shared__ __align__(16) float2 s[];
@@ -40,9 +42,9 @@ __global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<
 }
 
 template <int N2, int LINES>
-__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>()) k_toep_rows_adj(ToepArgs A, float2* __restrict__ out, const float2* __restrict__ pvec,
-                                float a, float b, int mode, double* __restrict__ part,
-                                const CgScalars* __restrict__ cg) {
+__global__ void __launch_bounds__(toep_threads<N2, LINES>(), 512 / toep_threads<N2, LINES>())
+    k_toep_rows_adj(ToepArgs A, float2* __restrict__ out, const float2* __restrict__ pvec, float a, float b, int mode,
+                    double* __restrict__ part, const CgScalars* __restrict__ cg) {
     HQS_PDL_ENTRY();
     if (cg && cg->done) return;
     extern __shared__ __align__(16) float2 s[];
