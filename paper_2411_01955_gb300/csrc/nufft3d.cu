@@ -299,8 +299,8 @@ __global__ void k_tile_fill3(const int4* __restrict__ pti, const int2* __restric
 // 8 x 1024 on the 128^3 grid has 6 points per distinct footprint) and the FMAs of the 4
 // points hide their latency.  CTAs take consecutive units, which share an L1-sized
 // neighbourhood.  Bound: L1 wavefronts (one per 128 bytes read) and the FMA pipe.
-// 64^3 x 16 coils, 524,288 points, W 6: 1556 -> 365 us against a half-warp per point (a
-// whole forward 1723 -> 521 us).
+// 64^3 x 16 coils, 524,288 points, W 6: 1556 -> 362 us against a half-warp per point (a
+// whole forward 1723 -> 497 us).
 template <int VEC> struct Vec3;
 template <> struct Vec3<2> {
     float2 a, b;
@@ -325,7 +325,10 @@ template <> struct Vec3<1> {
     HQS_DEV void fma(const Vec3& v, float2 w) { a = cfma2(v.a, w, a); }
     HQS_DEV void put(float2* y, int64_t, int) const { y[0] = a; }
 };
-constexpr int kInterpRounds = 4;   // most units of a lane group, one after the other
+// most units of a lane group, one after the other.  A whole forward with 1, 2, 4, 8, us:
+// 128^3 x 8 coils 2155, 2033, 2020, 2104; 64^3 x 16 505, 483, 499, 552; 64^3 x 4 156, 169, 198,
+// 199; 32^3 x 8 92, 92, 107, 106: 2 is as good or better at all of these but the largest
+constexpr int kInterpRounds = 4;
 template <int W, int VEC, int LPP>
 __global__ void __launch_bounds__(256, 2) k_interp3(const float2* __restrict__ Gh, const int4* __restrict__ pti,
                                                     const float* __restrict__ kbw, const int2* __restrict__ units,
@@ -410,9 +413,9 @@ __global__ void __launch_bounds__(256, 2) k_interp3(const float2* __restrict__ G
 // the rows selected by a switch on the unit's y offset (registers need static names).
 // A tile with several items sums their partial tiles in slot order when the last
 // arrives.  Bound: instruction issue, the FMA pipe (about 19 packed operations per point
-// and plane) and the batches' barriers.  64^3 x 16 coils, 524,288 points, W 6: 824 us
+// and plane) and the batches' barriers.  64^3 x 16 coils, 524,288 points, W 6: 798 us
 // against 2630 and a 41 us memset with patches of 4 coils added by atomics (a whole
-// adjoint 2824 -> 1013 us; units of one point and 256-point batches: 1297 us).
+// adjoint 2824 -> 964 us; units of one point and 256-point batches: 1297 us).
 #define HQS3_ITEM 256
 // k-space data to the sorted point order, coil-innermost: ys[inv[m]][l] = y[l][m].  A CTA
 // stages kSortPts caller-order points of every coil (coalesced rows of y) in shared

@@ -11,7 +11,11 @@
 #endif
 #define HQS_MAX_LC HQS_KLINES  // coils per chunk in the FFT passes
 #define HQS_MAX_BLOCKS 2048    // partial-sum slots per reduction (and >= 3 x 256 for the FCG dots)
-#define HQS_SPREAD_LIGHT 64    // points of a grid tile that one warp spreads; heavier tiles take whole CTAs
+// points of a grid tile that one warp spreads; heavier tiles take whole CTAs.  A whole adjoint
+// with 32, 64, 96, 128 points, us: 64^2 x 4 coils 13.7, 19.2, 22.6, 22.6; 128^2 x 8 20.3, 25.8,
+// 31.4, 37.9; 256^2 x 12 32.6, 40.0, 45.7, 51.2; 320^2 x 16 64.4, 61.8, 72.0, 74.6; 384^2 x 13
+// 103, 95.4, 96.2, 99.2: taken for the largest slices, 32 is the better one below them
+#define HQS_SPREAD_LIGHT 64
 #define HQS_TRACE_MAX 4096     // phase-trace stamps kept per persistent solve
 
 // CG scalars kept on the device so that the solve never needs the host
@@ -49,8 +53,11 @@ struct hqs_plan_s {
     int q_rows = 8;     // lines per CTA in the single-image FFT passes
     int fused_grid = 0; // cap on the persistent solver's CTAs (0: occupancy limit)
     bool nufft_only = false; // internal plans that only grid (no Toeplitz kernel, density symbol zero)
-    int pc_lines = 2;   // preconditioner lines per item in the persistent solver (1..16; one 320^2 slice,
-                        // 304 CTAs: 1, 2, 4 lines give a step of 5 iterations 781, 700, 717 us)
+    // preconditioner lines per item in the persistent solver (1..16).  5 iterations of one
+    // slice with 1, 2, 4, 8 lines, us: 64^2 x 4 coils 159, 159, 159, 165; 128^2 x 8 227, 229,
+    // 236, 253; 256^2 x 16 354, 354, 367, 394; 320^2 x 16 671, 591, 607, 657; 384^2 x 16 864,
+    // 774, 808, 879
+    int pc_lines = 2;
     int debug_barrier_skip = 0;  // test hook for the next persistent solve (HQS_TUNE_DEBUG_BARRIER_SKIP)
 
     // constant tables and plan data (device)
